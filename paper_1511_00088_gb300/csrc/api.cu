@@ -44,7 +44,7 @@ using namespace stag;
 
 namespace {
 
-size_t cplx_bytes(int P) { return P == P64 ? 16 : P == P32 ? 8 : 4; }
+size_t cplx_bytes(int P) { return (P == P64 || P == PFX) ? 16 : P == P32 ? 8 : 4; }
 
 struct DevBuf {
   void *p = nullptr;
@@ -212,6 +212,9 @@ struct stag_ctx {
   size_t l2_max_persist = 0, l2_max_window = 0;
   DevBuf links_canon;  // [4][V][3][3] FP64, kept for lazy reduced-precision copies
   DevBuf links64;
+  DevBuf links_fx;     // fixed-point copy (fixed.cuh) of a near-unitary field, else unused
+  bool fx_ok = false;  // the FP64 operator runs from links_fx
+  bool fx_mode = true; // STAG_FX=0: never (the FP64 pipe's operator, for A/B runs)
   DevBuf links_lo[4][2];
   bool lo_ok[4][2] = {{false, false}, {false, false}, {false, false}, {false, false}};
   DevBuf links_tile[4][2];  // tiled site-owned copies (bulk-copied by the CG kernels)
@@ -313,13 +316,23 @@ int vec_out(stag_ctx *c, const VecBuf &v, int k, double *dst) {
   return STAG_OK;
 }
 
+// FP64 operator form of the uploaded field: PFX (integer-pipe products of the
+// fixed-point links) on near-unitary fields, P64 on any other field
+int lp_for(const stag_ctx *c, int P) { return (P == P64 && c->fx_ok) ? PFX : P; }
+const void *links64_op(const stag_ctx *c) { return c->fx_ok ? c->links_fx.p : c->links64.p; }
+// launch_dslash with the FP64 form of this field
+cudaError_t launch_ds(const stag_ctx *c, int LP, int recon, int VP, int OP, int NS, int EPI, int lanes, int nblocks,
+                      cudaStream_t st, const DsArgs &a, const void **kptr = nullptr) {
+  return launch_dslash(lp_for(c, LP), recon, VP, OP, NS, EPI, lanes, nblocks, st, a, kptr);
+}
+
 int links_for(stag_ctx *c, int P, const void **out) {
   if (!c->have_links) {
     c->err = "no gauge field: call stag_links_upload first";
     return STAG_ERR_STATE;
   }
   if (P == P64) {
-    *out = c->links64.p;
+    *out = links64_op(c);
     return STAG_OK;
   }
   const int rc = (c->flags & STAG_RECON12) ? 1 : 0;
@@ -376,7 +389,8 @@ void set_l2_window(stag_ctx *c, int P, int tma, int on, DsArgs &a) {
   if (!c->l2persist || !on) return;
   const int rc = (P != P64 && (c->flags & STAG_RECON12)) ? 1 : 0;
   const DevBuf &b = (on == 2) ? c->w.vpool
-                              : (P == P64) ? c->links64 : (tma ? c->links_tile[P][rc] : c->links_lo[P][rc]);
+                              : (P == P64) ? (c->fx_ok ? c->links_fx : c->links64)
+                                           : (tma ? c->links_tile[P][rc] : c->links_lo[P][rc]);
   if (!b.p || b.n == 0) return;
   a.l2_base = b.p;
   a.l2_bytes = b.n < c->l2_max_window ? b.n : c->l2_max_window;
@@ -449,7 +463,7 @@ int cg_blocks(stag_ctx *c, int LP, int recon, int VP, int NS, int EPI, int lanes
   memset(&none, 0, sizeof none);
   none.tma = tma;
   const void *k = nullptr;
-  CK(launch_dslash(LP, recon, VP, VP, NS, EPI, lanes, 0, c->stream, none, &k));
+  CK(launch_ds(c, LP, recon, VP, VP, NS, EPI, lanes, 0, c->stream, none, &k));
   int per_sm = 0, nsm = 0;
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, DS_BT, tma == 1 ? tma_smem_bytes(LP, recon, lanes) : 0));
   CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
@@ -608,6 +622,12 @@ int tune_cg_pair(stag_ctx *c, int LP, int recon, int VP, int NS, int EPI1, DsArg
   }
   const bool fl = fl1 != 0;
   std::vector<CgForm> cand;
+  if (lp_for(c, LP) == PFX) {  // one thread mapping
+    CgForm f;
+    f.l1 = f.l2 = FX_LANES;
+    f.l2p = (l2modes & 0b100) ? 2 : (l2modes & 0b010) ? 1 : 0;
+    cand.push_back(f);
+  } else {
   for (int p = 0; p < 3; ++p)
     for (int t = 0; t < 3; ++t)
       for (int l1 = 1; l1 <= 2; ++l1)
@@ -620,12 +640,13 @@ int tune_cg_pair(stag_ctx *c, int LP, int recon, int VP, int NS, int EPI1, DsArg
             f.l2p = p;
             cand.push_back(f);
           }
+  }
   if (cand.size() == 1 && !ms_out) {
     *out = cand[0];
     return STAG_OK;
   }
   const int G = a1.ngroups;
-  const TuneKey key(LP, recon, VP, NS * 16 + EPI1 + 8, (G * 8 + modes) * 8 + l2modes, c->dims[0], c->dims[1],
+  const TuneKey key(lp_for(c, LP), recon, VP, NS * 16 + EPI1 + 8, (G * 8 + modes) * 8 + l2modes, c->dims[0], c->dims[1],
                     c->dims[2], c->dims[3]);
   if (!fl && !ms_out) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -661,8 +682,8 @@ int tune_cg_pair(stag_ctx *c, int LP, int recon, int VP, int NS, int EPI1, DsArg
     if (f.l2p) l2_setaside(c, true);
     for (int i = 0; i < tune_pairs(c) + 2; ++i) {
       if (i == 2) CK(cudaEventRecord(e0, c->stream));
-      CK(launch_dslash(LP, recon, VP, VP, NS, EPI1, f.l1, nb1[q], c->stream, a1));
-      CK(launch_dslash(LP, recon, VP, VP, NS, EPI_CG_K2, f.l2, nb2[q], c->stream, a2));
+      CK(launch_ds(c, LP, recon, VP, VP, NS, EPI1, f.l1, nb1[q], c->stream, a1));
+      CK(launch_ds(c, LP, recon, VP, VP, NS, EPI_CG_K2, f.l2, nb2[q], c->stream, a2));
     }
     CK(cudaEventRecord(e1, c->stream));
     CK(cudaEventSynchronize(e1));
@@ -694,12 +715,16 @@ int tune_cg_pair(stag_ctx *c, int LP, int recon, int VP, int NS, int EPI1, DsArg
 
 int tune_lanes(stag_ctx *c, int LP, int recon, int VP, int NS, int G, int nsys, const void *links, VecArg in,
                VecArg out, int *lanes_out) {
+  if (lp_for(c, LP) == PFX) {
+    *lanes_out = FX_LANES;
+    return STAG_OK;
+  }
   const char *force = getenv("STAG_LANES");
   if (force && (force[0] == '1' || force[0] == '2') && force[1] == 0) {
     *lanes_out = force[0] - '0';
     return STAG_OK;
   }
-  const TuneKey key(LP, recon, VP, NS, G, c->dims[0], c->dims[1], c->dims[2], c->dims[3]);
+  const TuneKey key(lp_for(c, LP), recon, VP, NS, G, c->dims[0], c->dims[1], c->dims[2], c->dims[3]);
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     tune_cache_load();
@@ -727,9 +752,9 @@ int tune_lanes(stag_ctx *c, int LP, int recon, int VP, int NS, int G, int nsys, 
   int best_l = 1;
   for (int l = 1; l <= 2; ++l) {
     const int nb = ds_blocks(c->Ve, l) * G;
-    for (int i = 0; i < 3; ++i) CK(launch_dslash(LP, recon, VP, VP, NS, EPI_PLAIN, l, nb, c->stream, a));
+    for (int i = 0; i < 3; ++i) CK(launch_ds(c, LP, recon, VP, VP, NS, EPI_PLAIN, l, nb, c->stream, a));
     CK(cudaEventRecord(e0, c->stream));
-    for (int i = 0; i < 10; ++i) CK(launch_dslash(LP, recon, VP, VP, NS, EPI_PLAIN, l, nb, c->stream, a));
+    for (int i = 0; i < 10; ++i) CK(launch_ds(c, LP, recon, VP, VP, NS, EPI_PLAIN, l, nb, c->stream, a));
     CK(cudaEventRecord(e1, c->stream));
     CK(cudaEventSynchronize(e1));
     float ms = 0.f;
@@ -776,7 +801,8 @@ int work_prepare(stag_ctx *c, int nsys, int precision, int ms = 0) {
   w.RP = RP;
   w.NS = 1;
   w.G = nsys;
-  w.NS64 = nsys >= 4 ? 4 : 1;
+  // the fixed-point operator holds one system's neighbour vectors a thread
+  w.NS64 = (nsys >= 4 && !c->fx_ok) ? 4 : 1;
   w.G64 = (nsys + w.NS64 - 1) / w.NS64;
   const int Ve = c->Ve;
   const int nbx_ds_max = (Ve + 31) / 32;  // most blocks per group of any CG kernel (32-site chunks)
@@ -846,12 +872,13 @@ int work_prepare(stag_ctx *c, int nsys, int precision, int ms = 0) {
     // Several systems: the candidates are timed (kernel pair, tune_cg_pair)
     // and the choice cached; STAG_NS = 1, 4 or 8 fixes it.
     std::vector<int> cands{1};
-    if (nsys >= 4) cands.push_back(4);
+    const bool fx = lp_for(c, prec) == PFX;  // one system a thread only
+    if (nsys >= 4 && !fx) cands.push_back(4);
     if (nsys >= 8 && prec != P64) cands.push_back(8);
     const char *fns = getenv("STAG_NS");
     if (fns && (fns[0] == '1' || fns[0] == '4' || fns[0] == '8') && fns[1] == 0) {
       const int f = fns[0] - '0';
-      if (f <= nsys && !(f == 8 && prec == P64)) cands.assign(1, f);
+      if (f <= nsys && !(f == 8 && prec == P64) && !(f > 1 && fx)) cands.assign(1, f);
     }
     // the shared-memory kernels (k_dslash_mrhs): FP32 links and vectors, 4 or 8
     // systems per block; encoded as 100 + nsw among the candidates
@@ -895,7 +922,7 @@ int work_prepare(stag_ctx *c, int nsys, int precision, int ms = 0) {
       }
     int best_ns = cands[0];
     if (cands.size() > 1) {
-      const TuneKey nkey(prec, recon, VP, 2000 + nsys, tma_ok ? 1 : 0, c->dims[0], c->dims[1], c->dims[2],
+      const TuneKey nkey(lp_for(c, prec), recon, VP, 2000 + nsys, tma_ok ? 1 : 0, c->dims[0], c->dims[1], c->dims[2],
                          c->dims[3]);
       bool cached = false;
       {
@@ -963,7 +990,7 @@ int work_prepare(stag_ctx *c, int nsys, int precision, int ms = 0) {
   }
   // the thread mapping of the plain inner and the FP64 half operators
   CKS(tune_lanes(c, prec, recon, VP, w.NS, w.G, nsys, lo, w.p.arg(), w.t.arg(), &w.lanes));
-  CKS(tune_lanes(c, P64, 0, P64, w.NS64, w.G64, nsys, c->links64.p, w.x64.arg(), w.t64.arg(), &w.lanes64));
+  CKS(tune_lanes(c, P64, 0, P64, w.NS64, w.G64, nsys, links64_op(c), w.x64.arg(), w.t64.arg(), &w.lanes64));
   return STAG_OK;
 }
 
@@ -1014,7 +1041,7 @@ cudaError_t launch_cg(stag_ctx *c, int kernel, int epi, cudaStream_t s, const Ds
     return launch_cg_nrhs(w.recon, w.nrhs_sl, epi, kernel == 0 ? w.nbx_k1 : w.nbx_k2, s, a);
   const int nb = (kernel == 0 ? w.nbx_k1 : w.nbx_k2) * w.G;
   if (w.mrhs) return launch_dslash_mrhs(w.prec, w.recon, w.mrhs, epi, nb, s, a);
-  return launch_dslash(w.prec, w.recon, w.VP, w.VP, w.NS, epi, kernel == 0 ? w.lanes_k1 : w.lanes_k2, nb, s, a);
+  return launch_ds(c, w.prec, w.recon, w.VP, w.VP, w.NS, epi, kernel == 0 ? w.lanes_k1 : w.lanes_k2, nb, s, a);
 }
 
 // The shifted-system update of a multi-shift solve (w.ms > 0), launched
@@ -1194,11 +1221,11 @@ int enqueue_update(stag_ctx *c, cudaStream_t s, const Ctl &ctl) {
     q.par_out = 1;
     q.in = w.p.arg();
     q.out = w.t.arg();
-    CK(launch_dslash(w.prec, w.recon, w.VP, w.VP, w.NS, EPI_PLAIN, w.lanes, ds_blocks(c->Ve, w.lanes) * w.G, s,
+    CK(launch_ds(c, w.prec, w.recon, w.VP, w.VP, w.NS, EPI_PLAIN, w.lanes, ds_blocks(c->Ve, w.lanes) * w.G, s,
                      q));
   }
   DsArgs a = ds_base(c);
-  a.links = c->links64.p;
+  a.links = links64_op(c);
   a.nsys = w.nsys;
   a.ngroups = w.G64;
   a.ctl = ctl;
@@ -1207,7 +1234,7 @@ int enqueue_update(stag_ctx *c, cudaStream_t s, const Ctl &ctl) {
   a.in = w.x64.arg();
   a.out = w.t64.arg();
   a.fin = FIN_NONE;
-  CK(launch_dslash(P64, 0, P64, P64, w.NS64, EPI_PLAIN, w.lanes64, ds_blocks(c->Ve, w.lanes64) * w.G64, s, a));
+  CK(launch_ds(c, P64, 0, P64, P64, w.NS64, EPI_PLAIN, w.lanes64, ds_blocks(c->Ve, w.lanes64) * w.G64, s, a));
   a.par_out = 0;
   a.in = w.t64.arg();
   a.center = w.x64.arg();
@@ -1215,7 +1242,7 @@ int enqueue_update(stag_ctx *c, cudaStream_t s, const Ctl &ctl) {
   a.out = w.r.arg();
   a.fin = FIN_RESID;
   if (w.VP == w.RP) a.dir = w.p.arg();  // Re<r_true, p> for the |p|^2 recurrence
-  CK(launch_dslash(P64, 0, P64, w.RP, w.NS64, EPI_RESID, w.lanes64, ds_blocks(c->Ve, w.lanes64) * w.G64, s, a));
+  CK(launch_ds(c, P64, 0, P64, w.RP, w.NS64, EPI_RESID, w.lanes64, ds_blocks(c->Ve, w.lanes64) * w.G64, s, a));
   CK(launch_finalize(ctl, FIN_RESID, ds_blocks(c->Ve, w.lanes64), 2, w.nsys, s));
   return STAG_OK;
 }
@@ -1499,9 +1526,9 @@ VecArg vec_slot(const VecBuf &v, int k) {
 
 int apply_m64(stag_ctx *c, int par_out, double m4, double scale, VecArg in, VecArg center, VecArg out) {
   int lanes = 1;
-  CKS(tune_lanes(c, P64, 0, P64, 1, 1, 1, c->links64.p, in, out, &lanes));
+  CKS(tune_lanes(c, P64, 0, P64, 1, 1, 1, links64_op(c), in, out, &lanes));
   DsArgs a = ds_base(c);
-  a.links = c->links64.p;
+  a.links = links64_op(c);
   a.nsys = 1;
   a.ngroups = 1;
   a.ctl = no_ctl();
@@ -1513,7 +1540,7 @@ int apply_m64(stag_ctx *c, int par_out, double m4, double scale, VecArg in, VecA
   a.in = in;
   a.center = center;
   a.out = out;
-  CK(launch_dslash(P64, 0, P64, P64, 1, EPI_MDAGM, lanes, ds_blocks(c->Ve, lanes), c->stream, a));
+  CK(launch_ds(c, P64, 0, P64, P64, 1, EPI_MDAGM, lanes, ds_blocks(c->Ve, lanes), c->stream, a));
   return STAG_OK;
 }
 
@@ -1591,6 +1618,43 @@ int op_impl(stag_ctx *c, int which, int precision, double mass, const double *in
   const int Ve = c->Ve;
   const double2 *d = nullptr;
   CKS(vec_in(c, in, c->stage_in, 0, &d));
+  if (lp_for(c, P) == PFX) {
+    // the fixed-point kernel reads and writes the caller's layout itself; a
+    // result that overlaps the input is staged
+    const size_t bytes = sizeof(double) * 6ull * Ve;
+    const bool overlap = (const char *)out < (const char *)in + bytes && (const char *)in < (const char *)out + bytes;
+    const bool direct = is_device_ptr(out) && !overlap;
+    if (!direct) CK(c->stage_out.ensure(bytes));
+    double2 *o = direct ? reinterpret_cast<double2 *>(out) : reinterpret_cast<double2 *>(c->stage_out.p);
+    DsArgs a = ds_base(c);
+    a.links = links;
+    a.nsys = 1;
+    a.ngroups = 1;
+    a.ctl = no_ctl();
+    a.gate = GATE_NONE;
+    a.fin = FIN_NONE;
+    a.m4_single = 4.0 * mass * mass;
+    a.in.v = const_cast<double2 *>(d);
+    a.abi_in = 1;
+    const int nb = ds_blocks(Ve, FX_LANES);
+    if (which == 2) {
+      CK(c->api_c.ensure(P64, 1, Ve));
+      a.par_out = 1;
+      a.out = c->api_c.arg();
+      CK(launch_ds(c, P64, 0, P64, P64, 1, EPI_PLAIN, FX_LANES, nb, c->stream, a));
+      a.in = c->api_c.arg();
+      a.abi_in = 0;
+      a.center.v = const_cast<double2 *>(d);
+      a.abi_center = 1;
+    }
+    a.par_out = which == 0 ? 1 : 0;
+    a.out.v = o;
+    a.abi_out = 1;
+    CK(launch_ds(c, P64, 0, P64, P64, 1, which == 2 ? EPI_MDAGM : EPI_PLAIN, FX_LANES, nb, c->stream, a));
+    if (!direct) CK(cudaMemcpyAsync(out, o, bytes, cudaMemcpyDefault, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    return STAG_OK;
+  }
   CK(c->api_a.ensure(VP, 1, Ve));
   CK(c->api_b.ensure(VP, 1, Ve));
   CK(c->api_c.ensure(VP, 1, Ve));
@@ -1617,18 +1681,18 @@ int op_impl(stag_ctx *c, int which, int precision, double mass, const double *in
     a.par_out = which == 0 ? 1 : 0;
     a.in = c->api_a.arg();
     a.out = c->api_b.arg();
-    CK(launch_dslash(P, recon, VP, VP, 1, EPI_PLAIN, lanes, nb, c->stream, a));
+    CK(launch_ds(c, P, recon, VP, VP, 1, EPI_PLAIN, lanes, nb, c->stream, a));
   } else {  // M^dag M
     a.par_out = 1;
     a.in = c->api_a.arg();
     a.out = c->api_c.arg();
     CK(c->api_c.ensure(VP, 1, Ve));
-    CK(launch_dslash(P, recon, VP, VP, 1, EPI_PLAIN, lanes, nb, c->stream, a));
+    CK(launch_ds(c, P, recon, VP, VP, 1, EPI_PLAIN, lanes, nb, c->stream, a));
     a.par_out = 0;
     a.in = c->api_c.arg();
     a.center = c->api_a.arg();
     a.out = c->api_b.arg();
-    CK(launch_dslash(P, recon, VP, VP, 1, EPI_MDAGM, lanes, nb, c->stream, a));
+    CK(launch_ds(c, P, recon, VP, VP, 1, EPI_MDAGM, lanes, nb, c->stream, a));
   }
   CKS(vec_out(c, c->api_b, 0, out));
   CK(cudaStreamSynchronize(c->stream));
@@ -1724,9 +1788,9 @@ int ms_impl(stag_ctx *c, const double *const src[], int nrhs, const double masse
 // out = D in (FP64) on the sites of parity par_out, one system
 int apply_m64_plain(stag_ctx *c, int par_out, VecArg in, VecArg out) {
   int lanes = 1;
-  CKS(tune_lanes(c, P64, 0, P64, 1, 1, 1, c->links64.p, in, out, &lanes));
+  CKS(tune_lanes(c, P64, 0, P64, 1, 1, 1, links64_op(c), in, out, &lanes));
   DsArgs a = ds_base(c);
-  a.links = c->links64.p;
+  a.links = links64_op(c);
   a.nsys = 1;
   a.ngroups = 1;
   a.ctl = no_ctl();
@@ -1735,7 +1799,7 @@ int apply_m64_plain(stag_ctx *c, int par_out, VecArg in, VecArg out) {
   a.par_out = par_out;
   a.in = in;
   a.out = out;
-  CK(launch_dslash(P64, 0, P64, P64, 1, EPI_PLAIN, lanes, ds_blocks(c->Ve, lanes), c->stream, a));
+  CK(launch_ds(c, P64, 0, P64, P64, 1, EPI_PLAIN, lanes, ds_blocks(c->Ve, lanes), c->stream, a));
   return STAG_OK;
 }
 
@@ -1980,6 +2044,8 @@ int stag_create(const int dims[4], int flags, void *cuda_stream, stag_ctx **out)
   }
   const char *eager = getenv("STAG_EAGER");
   c->use_graph = !(eager && eager[0] == '1');
+  const char *fx = getenv("STAG_FX");
+  c->fx_mode = !(fx && fx[0] == '0');
   const char *pdl = getenv("STAG_PDL");
   c->pdl = !(pdl && pdl[0] == '0');
   const char *fold = getenv("STAG_FOLD");
@@ -2060,12 +2126,28 @@ int stag_links_upload(stag_ctx *c, const double *links) {
     }
   }
   CK(c->links64.ensure(cplx_bytes(P64) * 9ull * 8ull * c->Ve));
-  CK(launch_pack_links(P64, 0, reinterpret_cast<const double2 *>(c->links_canon.p), c->links64.p, c->g,
-                       c->stream));
+  // The FP64 copy, and with room for it the fixed-point copy; a field that is
+  // not near unitary keeps the FP64 operator.
+  const bool fx_was = c->fx_ok;
+  int fx_bad = 1;
+  c->fx_ok = false;
+  if (c->fx_mode && c->links_fx.ensure(cplx_bytes(PFX) * 9ull * 8ull * c->Ve) == cudaSuccess) {
+    CK(c->defect.ensure(sizeof(unsigned long long)));
+    CK(cudaMemsetAsync(c->defect.p, 0, sizeof(unsigned long long), c->stream));
+    CK(launch_pack_links_fx(reinterpret_cast<const double2 *>(c->links_canon.p), (double2 *)c->links64.p,
+                            (int4 *)c->links_fx.p, c->g, (int *)c->defect.p, c->stream));
+    CK(cudaMemcpyAsync(&fx_bad, c->defect.p, sizeof fx_bad, cudaMemcpyDeviceToHost, c->stream));
+  } else {
+    cudaGetLastError();
+    CK(launch_pack_links(P64, 0, reinterpret_cast<const double2 *>(c->links_canon.p), c->links64.p, c->g,
+                         c->stream));
+  }
   for (int p = 0; p < 4; ++p) c->lo_ok[p][0] = c->lo_ok[p][1] = c->tile_ok[p][0] = c->tile_ok[p][1] = false;
   c->have_links = true;
   c->w.drop_graph();  // the graph holds link pointers of the reduced-precision copies
   CK(cudaStreamSynchronize(c->stream));
+  c->fx_ok = fx_bad == 0;
+  if (c->fx_ok != fx_was) c->w.nsys = 0;  // the FP64 launch forms were chosen for the other operator
   return STAG_OK;
 }
 

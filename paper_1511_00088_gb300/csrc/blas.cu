@@ -8,6 +8,7 @@ cudaError_t launch_dslash(int LP, int recon, int VP, int OP, int NS, int EPI, in
                           cudaStream_t st, const DsArgs &a, const void **kptr) {
   switch (LP) {
     case P64: return launch_dslash_p64(recon, VP, OP, NS, EPI, lanes, nblocks, st, a, kptr);
+    case PFX: return launch_dslash_fx(recon, VP, OP, NS, EPI, lanes, nblocks, st, a, kptr);
     case P32: return launch_dslash_p32(recon, VP, OP, NS, EPI, lanes, nblocks, st, a, kptr);
     case P16: return launch_dslash_p16(recon, VP, OP, NS, EPI, lanes, nblocks, st, a, kptr);
     case PBF: return launch_dslash_pbf(recon, VP, OP, NS, EPI, lanes, nblocks, st, a, kptr);
@@ -248,6 +249,45 @@ cudaError_t launch_pack_links(int LP, int recon, const double2 *src, void *dst, 
   STAG_PL(PBF, 0) STAG_PL(PBF, 1)
 #undef STAG_PL
   return cudaErrorNotSupported;
+}
+
+// One thread per link: bound by memory (144 B read, 288 B written); the
+// fixed-point split works on the FP64 bit patterns, as its conversions would
+// otherwise hold the FP64 pipe for longer than the copy takes.
+__global__ void __launch_bounds__(256) k_pack_links_fx(const double2 *__restrict__ src, double2 *__restrict__ dst64,
+                                                       int4 *__restrict__ dstfx, Geom g, int *bad) {
+  const long long V = 2ll * g.Ve;
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= 4 * V) return;
+  const int mu = (int)(i / V);
+  const long long lex = i % V;
+  const int s = (int)(lex >> 1);
+  const unsigned q1 = fast_div((unsigned)s, g.dLxh), q2 = fast_div(q1, g.dL1), q3 = fast_div(q2, g.dL2);
+  const int par = (int)((lex & 1) + (q1 - q2 * g.L1) + (q2 - q3 * g.L2) + q3) & 1;
+  const long long o = (long long)((par * 4 + mu) * 9) * g.Ve + s;
+  float row[3] = {0.f, 0.f, 0.f}, col[3] = {0.f, 0.f, 0.f};
+  bool ok = true;
+#pragma unroll
+  for (int e = 0; e < 9; ++e) {
+    const double2 w = src[i * 9 + e];
+    dst64[o + (long long)e * g.Ve] = w;
+    const int hx = __double2hiint(w.x), hy = __double2hiint(w.y);
+    ok = ok && (hx & 0x7fffffff) < 0x40000000 && (hy & 0x7fffffff) < 0x40000000;  // |.| < 2 (false for NaN)
+    const Fx a = fx_link(hx, __double2loint(w.x)), b = fx_link(hy, __double2loint(w.y));
+    const int4 f = make_int4(a.h, a.l, b.h, b.l);
+    dstfx[o + (long long)e * g.Ve] = f;
+    const float x = (float)a.h * 0x1p-29f, y = (float)b.h * 0x1p-29f, n = x * x + y * y;
+    row[e / 3] += n;
+    col[e % 3] += n;
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) ok = ok && fabsf(row[k] - 1.f) <= 1e-3f && fabsf(col[k] - 1.f) <= 1e-3f;
+  if (!ok) *bad = 1;
+}
+
+cudaError_t launch_pack_links_fx(const double2 *src, double2 *dst64, int4 *dstfx, Geom g, int *bad, cudaStream_t st) {
+  k_pack_links_fx<<<nblk(8ll * g.Ve, 256), 256, 0, st>>>(src, dst64, dstfx, g, bad);
+  return cudaGetLastError();
 }
 
 // max over links of max(|U U^dag - 1|_max, |det U - 1|), FP64

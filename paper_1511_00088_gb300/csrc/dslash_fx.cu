@@ -1,0 +1,326 @@
+// dslash_fx.cu -- the FP64 half operator from fixed-point links (PFX): the
+// FP64 CG, the reliable updates and the operator calls on near-unitary gauge
+// fields.  The products run on the integer pipe (fixed.cuh).
+//
+// A block owns chunks of 32 output sites; warp mu holds direction mu of all of
+// them, one lane a site, and each thread takes the forward and the backward
+// hop: 6 vector and 18 link loads of 16 bytes, all of a warp's 32 lanes on
+// consecutive sites, issued before any arithmetic (one memory round trip; with
+// whole sites to a thread or two the links came in a second, register-bound
+// one: 103 us at 20^3 x 64 where the bytes take 48).  Each thread scales its two
+// neighbour vectors by their own largest exponent; its six sums meet the other
+// directions' in shared memory as 64-bit integers, where 96 threads, one a
+// (site, colour), bring them to a common exponent, add, round once to FP64 and
+// run the epilogue: FP64 instructions are spent once a component, not once a
+// lane, as they are the scarce ones (a warp's takes 16 clocks of an SM).
+// Measured (M^dag M call on device buffers, 20^3 x 64; its two passes over the
+// links take 96 us at the copy rate): 364 us on FP64 FMAs with packed copies of
+// the vectors, 178 us in this form, 149 us with the caller's layout read and
+// written directly (abi_in, abi_center, abi_out); FP64 CG iteration on 16^3 x 32:
+// 115 us before, 50 us.
+// A thread whose neighbours hold an infinity, a NaN or only numbers near the
+// ends of the exponent range sums its hops on FP64 FMAs instead.
+#include "launch.h"
+
+namespace stag {
+
+namespace {
+
+constexpr int FXB = 128;        // threads: 4 directions x 32 sites
+constexpr int FX_FP64 = -1;     // exponent mark of a partial sum held as FP64
+constexpr int FX_E0 = 64;       // smallest exponent field of the integer form (and that of a zero sum)
+constexpr int FX_E1 = 2030;     // the largest
+
+__device__ __forceinline__ double fx_value(int h, int l) {
+  return __fma_rn((double)h, 0x1p-29, (double)l * 0x1p-58);
+}
+
+// the two hops of one direction on FP64 FMAs
+__device__ __noinline__ void hops_fp64(const int4 *uf, const int4 *ub, const double2 *vf, const double2 *vb, int Ve,
+                                       long long cs, unsigned flipf, unsigned flipb, double *out) {
+  double acc[6] = {0, 0, 0, 0, 0, 0};
+#pragma unroll 1
+  for (int q = 0; q < 2; ++q) {
+    const int4 *L = q ? ub : uf;
+    const double2 *in = q ? vb : vf;
+    const double sg = (q ? flipb : flipf) ? -1.0 : 1.0;
+    for (int b = 0; b < 3; ++b) {
+      const double2 v = __ldg(in + b * cs);
+      for (int a = 0; a < 3; ++a) {
+        const int4 w = __ldg(L + (long long)(q ? 3 * b + a : 3 * a + b) * Ve);
+        const double ur = sg * fx_value(w.x, w.y), ui = (q ? -sg : sg) * fx_value(w.z, w.w);
+        acc[2 * a] += ur * v.x - ui * v.y;
+        acc[2 * a + 1] += ur * v.y + ui * v.x;
+      }
+    }
+  }
+  for (int i = 0; i < 6; ++i) out[i] = acc[i];
+}
+
+// Blocks an SM: 4 (128 registers) for the plain operator, 3 (168) for the CG
+// kernels and the residual, whose epilogue operands would spill (20^3 x 64: M^dag
+// M call 149 us at 4, 163 at 3; FP64 CG on 16^3 x 32, 713 iterations: 42 and 35.5 ms).
+template <int EPI, int OP>
+__global__ void __launch_bounds__(FXB, (EPI == EPI_PLAIN || EPI == EPI_MDAGM) ? 4 : 3) k_dslash_fx(const DsArgs a) {
+  typedef typename Tr<OP>::S2 OS2;
+  typedef typename Tr<OP>::R OR;
+  constexpr int NV = (EPI == EPI_CG_K2 || EPI == EPI_RESID) ? 2 : 1;
+  constexpr bool REDUCES = EPI == EPI_CG_K1R || EPI == EPI_CG_K2 || EPI == EPI_RESID;
+  __shared__ long long part_t[2][4][6][32];
+  __shared__ int part_e[2][4][32];
+  const Geom g = a.g;
+  const int Ve = g.Ve, P = a.par_out, G = a.ngroups;
+  const int grp = blockIdx.x % G, bx0 = blockIdx.x / G, nbx = (int)gridDim.x / G;
+  const int nchunk = (Ve + 31) / 32;
+  const int lane = threadIdx.x & 31, mu = threadIdx.x >> 5;
+  grid_dep_trigger();
+  grid_dep_wait();
+  __shared__ SysState sst[1];
+  const SysState *S = (a.ctl.st != nullptr) ? a.ctl.st + grp : nullptr;
+  if (a.fold != FIN_NONE) {
+    fold_state<1, FXB>(a, grp, bx0, sst);
+    S = sst;
+  }
+  const bool act = a.gate == GATE_NONE || S == nullptr || state_gate(*S, a.gate);
+  const double m4 = S != nullptr ? S->m4 : a.m4_single;
+  const double beta = S != nullptr ? S->beta : 0.0;
+  const double alpha = S != nullptr ? S->alpha : 0.0;
+  double part[1][NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) part[0][v] = 0.0;
+  if (act) {
+    const int4 *links = reinterpret_cast<const int4 *>(a.links);
+    const long long sys = (long long)grp * a.in.sstr;
+    const double2 *in = reinterpret_cast<const double2 *>(a.in.v) + sys;
+    // strides of a vector's sites and colours, the ABI's or the device layout's
+    const long long is = a.abi_in ? 3 : 1, ic = a.abi_in ? 1 : Ve;
+    const int Lmu = mu == 0 ? g.L0 : mu == 1 ? g.L1 : mu == 2 ? g.L2 : g.L3;
+    int buf = 0;
+    for (int bx = bx0; bx < nchunk; bx += nbx, buf ^= 1) {
+      const int s = bx * 32 + lane;
+      // the epilogue's operands of (site lane, colour mu), in flight with the hops
+      const bool epi = mu < 3 && s < Ve;
+      const long long o = sys + (long long)mu * Ve + s, oa = 3ll * s + mu;
+      double2 c0, c1, c2;
+      if (epi) {
+        if (EPI == EPI_CG_K2) {
+          c0 = reinterpret_cast<const double2 *>(a.center.v)[o];
+          c1 = reinterpret_cast<const double2 *>(a.aux.v)[o];
+          c2 = reinterpret_cast<const double2 *>(a.xlo.v)[o];
+        } else if (EPI == EPI_CG_K1R) {
+          c0 = reinterpret_cast<const double2 *>(a.out.v)[o];
+        } else if (EPI == EPI_MDAGM) {
+          c0 = __ldg(reinterpret_cast<const double2 *>(a.center.v) + (a.abi_center ? oa : o));
+        } else if (EPI == EPI_RESID) {
+          c0 = __ldg(reinterpret_cast<const double2 *>(a.center.v) + o);
+          c1 = __ldg(reinterpret_cast<const double2 *>(a.aux.v) + o);
+          c2 = make_double2(0.0, 0.0);
+          if (a.dir.v != nullptr) {
+            const auto w = to_r2(ldg2(reinterpret_cast<const OS2 *>(a.dir.v) + o));
+            c2 = make_double2((double)w.x, (double)w.y);
+          }
+        }
+      }
+      if (s < Ve) {
+        int x[4];
+        site_coords(g, P, s, x);
+        int eb = 0;  // x_0 + ... + x_{mu-1}
+        if (mu > 0) eb += x[0];
+        if (mu > 1) eb += x[1];
+        if (mu > 2) eb += x[2];
+        const int xm = mu == 0 ? x[0] : mu == 1 ? x[1] : mu == 2 ? x[2] : x[3];
+        const int xp = (xm + 1 == Lmu) ? 0 : xm + 1, xn = (xm == 0) ? Lmu - 1 : xm - 1;
+        const int sf = cb_of(g, mu == 0 ? xp : x[0], mu == 1 ? xp : x[1], mu == 2 ? xp : x[2], mu == 3 ? xp : x[3]);
+        const int sb = cb_of(g, mu == 0 ? xn : x[0], mu == 1 ? xn : x[1], mu == 2 ? xn : x[2], mu == 3 ? xn : x[3]);
+        unsigned ff = (eb & 1) ? 0x80000000u : 0u, fb = ff ^ 0x80000000u;  // backward hops enter with a minus
+        if (mu == 3 && g.ap) {
+          if (xm == g.L3 - 1) ff ^= 0x80000000u;
+          if (xm == 0) fb ^= 0x80000000u;
+        }
+        const int4 *uf = links + (long long)((P * 4 + mu) * 9) * Ve + s;
+        const int4 *ub = links + (long long)(((1 - P) * 4 + mu) * 9) * Ve + sb;
+        double2 wf[3], wb[3];
+        int4 lf[9], lb[9];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          wf[c] = __ldg(in + c * ic + sf * is);
+          wb[c] = __ldg(in + c * ic + sb * is);
+        }
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+          lf[e] = __ldg(uf + (long long)e * Ve);
+          lb[e] = __ldg(ub + (long long)e * Ve);
+        }
+        int top = 0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          top = max(top, max(__double2hiint(wf[c].x) & 0x7fffffff, __double2hiint(wf[c].y) & 0x7fffffff));
+          top = max(top, max(__double2hiint(wb[c].x) & 0x7fffffff, __double2hiint(wb[c].y) & 0x7fffffff));
+        }
+        int E = top >> 20;
+        long long T[6];
+        bool zero = false;
+        if (E < FX_E0 && top == 0) {
+          int any = 0;
+#pragma unroll
+          for (int c = 0; c < 3; ++c)
+            any |= __double2loint(wf[c].x) | __double2loint(wf[c].y) | __double2loint(wb[c].x) | __double2loint(wb[c].y);
+          zero = any == 0;
+        }
+        if (zero) {
+          E = FX_E0;
+#pragma unroll
+          for (int i = 0; i < 6; ++i) T[i] = 0;
+        } else if (E < FX_E0 || E > FX_E1) {
+          E = FX_FP64;
+          double d[6];
+          hops_fp64(uf, ub, in + sf * is, in + sb * is, Ve, ic, ff, fb, d);
+#pragma unroll
+          for (int i = 0; i < 6; ++i) T[i] = __double_as_longlong(d[i]);
+        } else {
+          FxAcc sum[6];
+#pragma unroll
+          for (int i = 0; i < 6; ++i) sum[i].hh = sum[i].cr = 0;
+#pragma unroll
+          for (int b = 0; b < 3; ++b) {  // (ur + i ui)(r + i m)
+            const Fx r = fx_vec(__double2hiint(wf[b].x) ^ (int)ff, __double2loint(wf[b].x), E);
+            const Fx m = fx_vec(__double2hiint(wf[b].y) ^ (int)ff, __double2loint(wf[b].y), E);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+              const int4 u = lf[3 * k + b];
+              fx_mac(sum[2 * k], u.x, u.y, r.h, r.l);
+              fx_mac(sum[2 * k], u.z, u.w, -m.h, -m.l);
+              fx_mac(sum[2 * k + 1], u.x, u.y, m.h, m.l);
+              fx_mac(sum[2 * k + 1], u.z, u.w, r.h, r.l);
+            }
+          }
+#pragma unroll
+          for (int b = 0; b < 3; ++b) {  // (ur - i ui)(r + i m)
+            const Fx r = fx_vec(__double2hiint(wb[b].x) ^ (int)fb, __double2loint(wb[b].x), E);
+            const Fx m = fx_vec(__double2hiint(wb[b].y) ^ (int)fb, __double2loint(wb[b].y), E);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+              const int4 u = lb[3 * b + k];
+              fx_mac(sum[2 * k], u.x, u.y, r.h, r.l);
+              fx_mac(sum[2 * k], u.z, u.w, m.h, m.l);
+              fx_mac(sum[2 * k + 1], u.x, u.y, m.h, m.l);
+              fx_mac(sum[2 * k + 1], u.z, u.w, -r.h, -r.l);
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < 6; ++i) T[i] = fx_sum(sum[i]);
+        }
+        part_e[buf][mu][lane] = E;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) part_t[buf][mu][i][lane] = T[i];
+      }
+      // one barrier a chunk: the next chunk writes the other buffer, and its
+      // barrier follows every read of this one
+      __syncthreads();
+      if (epi) {
+        int E = FX_E0;
+        bool f64 = false;
+#pragma unroll
+        for (int d = 0; d < 4; ++d) {
+          const int e = part_e[buf][d][lane];
+          f64 |= e == FX_FP64;
+          E = max(E, e);
+        }
+        double2 v;
+        if (!f64) {
+          long long re = 0, im = 0;
+#pragma unroll
+          for (int d = 0; d < 4; ++d) {
+            const int sh = min(E - part_e[buf][d][lane], 63);
+            re += part_t[buf][d][2 * mu][lane] >> sh;
+            im += part_t[buf][d][2 * mu + 1][lane] >> sh;
+          }
+          // unit 2^(E - 1022 - 57): its exponent field stays in 1 .. 2046
+          const double unit = __hiloint2double((E - 1022 - FX_VBITS + 1023) << 20, 0);
+          v = make_double2((double)re * unit, (double)im * unit);
+        } else {
+          v = make_double2(0.0, 0.0);
+#pragma unroll 1
+          for (int d = 0; d < 4; ++d) {
+            const int e = part_e[buf][d][lane];
+            const long long re = part_t[buf][d][2 * mu][lane], im = part_t[buf][d][2 * mu + 1][lane];
+            if (e == FX_FP64) {
+              v.x += __longlong_as_double(re);
+              v.y += __longlong_as_double(im);
+            } else {
+              const double unit = __hiloint2double((e - 1022 - FX_VBITS + 1023) << 20, 0);
+              v.x += (double)re * unit;
+              v.y += (double)im * unit;
+            }
+          }
+        }
+        if (EPI == EPI_CG_K2) {
+          // p = r + beta p_old; Ap = 4 m^2 p - D_eo t; r -= alpha Ap; x += alpha p
+          c0.x = __fma_rn(beta, c0.x, c1.x);
+          c0.y = __fma_rn(beta, c0.y, c1.y);
+          c1.x = __fma_rn(-alpha, __fma_rn(m4, c0.x, -v.x), c1.x);
+          c1.y = __fma_rn(-alpha, __fma_rn(m4, c0.y, -v.y), c1.y);
+          c2.x = __fma_rn(alpha, c0.x, c2.x);
+          c2.y = __fma_rn(alpha, c0.y, c2.y);
+          reinterpret_cast<double2 *>(a.center.v)[o] = c0;
+          reinterpret_cast<double2 *>(a.aux.v)[o] = c1;
+          reinterpret_cast<double2 *>(a.xlo.v)[o] = c2;
+          part[0][0] = __fma_rn(c1.x, c1.x, __fma_rn(c1.y, c1.y, part[0][0]));
+          part[0][NV - 1] = __fma_rn(c1.x, c0.x, __fma_rn(c1.y, c0.y, part[0][NV - 1]));
+        } else if (EPI == EPI_CG_K1R) {
+          // t = D_oe r + beta t_old
+          v.x = __fma_rn(beta, c0.x, v.x);
+          v.y = __fma_rn(beta, c0.y, v.y);
+          reinterpret_cast<double2 *>(a.out.v)[o] = v;
+          part[0][0] = __fma_rn(v.x, v.x, __fma_rn(v.y, v.y, part[0][0]));
+        } else if (EPI == EPI_RESID) {
+          // r = b - (4 m^2 x - D in), stored at OP; |r|^2, and Re<r, p> of the stored r
+          v.x = c1.x - __fma_rn(m4, c0.x, -v.x);
+          v.y = c1.y - __fma_rn(m4, c0.y, -v.y);
+          const OR rx = (OR)v.x, ry = (OR)v.y;
+          reinterpret_cast<OS2 *>(a.out.v)[o] = from_r<OP>(rx, ry);
+          part[0][0] = __fma_rn(v.x, v.x, __fma_rn(v.y, v.y, part[0][0]));
+          part[0][NV - 1] = __fma_rn((double)rx, c2.x, __fma_rn((double)ry, c2.y, part[0][NV - 1]));
+        } else {
+          if (EPI == EPI_MDAGM) {
+            v.x = __fma_rn(m4, c0.x, -v.x);
+            v.y = __fma_rn(m4, c0.y, -v.y);
+            if (a.out_scale != 0.0) {
+              v.x *= a.out_scale;
+              v.y *= a.out_scale;
+            }
+          }
+          reinterpret_cast<double2 *>(a.out.v)[a.abi_out ? oa : o] = v;
+        }
+      }
+    }
+  }
+  if (REDUCES) {
+    if (a.ctl.st != nullptr) block_partials<1, NV>(a.ctl, part, grp, a.nsys, bx0);
+  }
+}
+
+template <int EPI, int OP>
+cudaError_t fx_one(int nblocks, cudaStream_t st, const DsArgs &a, const void **kptr) {
+  auto k = k_dslash_fx<EPI, OP>;
+  if (kptr) {
+    *kptr = (const void *)k;
+    return cudaSuccess;
+  }
+  return launch_ex_full(k, nblocks, FXB, 0u, st, a.pdl != 0, a.l2_base, a.l2_bytes, a.l2_hit, a);
+}
+
+}  // namespace
+
+cudaError_t launch_dslash_fx(int recon, int VP, int OP, int NS, int EPI, int lanes, int nblocks, cudaStream_t st,
+                             const DsArgs &a, const void **kptr) {
+  if (recon != 0 || VP != P64 || NS != 1 || lanes != FX_LANES) return cudaErrorNotSupported;
+#define STAG_FX_CASE(EPI_, OP_) \
+  if (EPI == EPI_ && OP == OP_) return fx_one<EPI_, OP_>(nblocks, st, a, kptr);
+  STAG_FX_CASE(EPI_PLAIN, P64) STAG_FX_CASE(EPI_MDAGM, P64) STAG_FX_CASE(EPI_CG_K1R, P64)
+  STAG_FX_CASE(EPI_CG_K2, P64) STAG_FX_CASE(EPI_RESID, P64) STAG_FX_CASE(EPI_RESID, P32)
+#undef STAG_FX_CASE
+  return cudaErrorNotSupported;
+}
+
+}  // namespace stag

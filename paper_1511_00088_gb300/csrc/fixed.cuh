@@ -1,0 +1,86 @@
+// fixed.cuh -- FP64-grade products on the integer pipe.
+//
+// GB300 issues FP64 FMAs at 2 lanes a clock and SM, 32 x 32 + 64 bit integer
+// multiply-adds (IMAD.WIDE) at 64 (both measured: 4.08 ms and 0.18 ms for the
+// same 2.5e9 of them).  SU(3) links are bounded by 1 and a site's neighbour
+// vectors can be scaled by one power of two, so their products need no
+// floating point: a link element u becomes U = u 2^58, a vector element v of
+// |v| <= 1 (after scaling) V = v 2^57, each split as
+//   h 2^29 + l,  -2^28 <= l < 2^28,
+// and a product is three multiply-adds into two 64-bit sums,
+//   hh += h h'  (unit 2^-57),   cr += h l' + l h'  (unit 2^-86);
+// l l' is dropped (below 2^-59 a product, either sign).  The sums are exact; the
+// result hh + cr / 2^29 has an absolute error near 2^-57 of the largest factor,
+// a tenth of an FP64 FMA chain's, and becomes FP64 with one rounding.
+// Range, for a row of u of 2-norm^2 <= 2 (the fields allowed are within 1e-3 of 1) on 6 components
+// |v| <= 1, eight hops: by Cauchy-Schwarz |hh| <= 8 sqrt(12) 2^57 < 2^61.8 and
+// |cr| <= 8 (sqrt(12) 2^57 + 6 2^56) < 2^62.7.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace stag {
+
+#define FX_HD __host__ __device__ __forceinline__
+
+constexpr int FX_LO = 29;    // bits of the low limb
+constexpr int FX_VBITS = 57; // fraction bits of a vector element
+
+struct Fx {
+  int h, l;
+};
+
+// V as its two limbs
+FX_HD Fx fx_split(long long V) {
+  const long long t = V + (1ll << (FX_LO - 1));
+  Fx f;
+  f.h = (int)(t >> FX_LO);
+  f.l = (int)((unsigned)t & ((1u << FX_LO) - 1u)) - (1 << (FX_LO - 1));
+  return f;
+}
+
+// the FP64 number (hi, lo) as (mantissa << UP) >> (E - its exponent field),
+// E >= that field; the bits shifted out are dropped, and zeros and denormals
+// become 0 where E >= 64
+template <int UP>
+FX_HD Fx fx_from(int hi, int lo, int E) {
+  int sh = E - ((hi >> 20) & 0x7ff);
+  sh = sh < 63 ? sh : 63;
+  unsigned long long m = ((unsigned long long)(unsigned)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)lo;
+  m = (m << UP) >> sh;
+  const Fx a = fx_split((long long)m);
+  const int s = (hi >> 31) | 1;
+  Fx f;
+  f.h = a.h * s;
+  f.l = a.l * s;
+  return f;
+}
+// a link element, |u| < 2: u 2^58
+FX_HD Fx fx_link(int hi, int lo) { return fx_from<6>(hi, lo, 1023); }
+// a vector element scaled by 2^(1022 - E), E >= the exponent fields of its site: v 2^57
+FX_HD Fx fx_vec(int hi, int lo, int E) { return fx_from<4>(hi, lo, E); }
+
+// sums of products
+struct FxAcc {
+  long long hh, cr;
+};
+// s += a b, one IMAD.WIDE (written as PTX: from s + (long long)a * b the
+// compiler may make a multiply and a two-instruction add)
+FX_HD void fx_wide(long long &s, int a, int b) {
+#ifdef __CUDA_ARCH__
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(s) : "r"(a), "r"(b));
+#else
+  s += (long long)a * b;
+#endif
+}
+FX_HD void fx_mac(FxAcc &s, int ah, int al, int bh, int bl) {
+  fx_wide(s.hh, ah, bh);
+  fx_wide(s.cr, ah, bl);
+  fx_wide(s.cr, al, bh);
+}
+// the sum at the unit of hh
+FX_HD long long fx_sum(const FxAcc &s) {
+  return s.hh + ((s.cr + (1ll << (FX_LO - 1))) >> FX_LO);
+}
+
+}  // namespace stag

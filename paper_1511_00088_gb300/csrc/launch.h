@@ -77,6 +77,10 @@ cudaError_t launch_dslash(int LP, int recon, int VP, int OP, int NS, int EPI, in
                           cudaStream_t st, const DsArgs &a, const void **kptr = nullptr);
 cudaError_t launch_dslash_p64(int recon, int VP, int OP, int NS, int EPI, int lanes, int nblocks,
                               cudaStream_t st, const DsArgs &a, const void **kptr);
+// k_dslash_fx (dslash_fx.cu): FX_LANES threads per site, blocks of DS_BT threads
+constexpr int FX_LANES = 4;
+cudaError_t launch_dslash_fx(int recon, int VP, int OP, int NS, int EPI, int lanes, int nblocks,
+                             cudaStream_t st, const DsArgs &a, const void **kptr);
 cudaError_t launch_dslash_p32(int recon, int VP, int OP, int NS, int EPI, int lanes, int nblocks,
                               cudaStream_t st, const DsArgs &a, const void **kptr);
 cudaError_t launch_dslash_p16(int recon, int VP, int OP, int NS, int EPI, int lanes, int nblocks,
@@ -121,6 +125,9 @@ cudaError_t launch_convert_vec(int PIN, int POUT, VecArg src, VecArg dst, int ns
                                cudaStream_t st);
 cudaError_t launch_pack_links(int LP, int recon, const double2 *src, void *dst, Geom g,
                               cudaStream_t st);
+// the FP64 (dst64) and fixed-point (dstfx) copies; *bad (device) set to 1 when
+// the field is not near unitary
+cudaError_t launch_pack_links_fx(const double2 *src, double2 *dst64, int4 *dstfx, Geom g, int *bad, cudaStream_t st);
 // the tiled site-owned copy (LP = P32, P16 or PBF); dst already zeroed
 cudaError_t launch_pack_links_tiled(int LP, int recon, const double2 *src, void *dst, Geom g, int ntile,
                                     cudaStream_t st);

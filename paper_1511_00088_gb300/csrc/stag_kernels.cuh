@@ -19,6 +19,8 @@
 //          mu = U_mu(x), slot 4 + mu = U_mu(x - mu) (the backward link, stored
 //          again at the site that uses it), so the 8 links of a chunk of sites
 //          are one contiguous block, moved into shared memory by one bulk copy.
+//   fixed-point links (PFX): as links, each complex element an int4 (the two
+//          limbs of its real, then of its imaginary part).
 // One thread owns one output site and NS systems; the 8 links of the site are
 // loaded once into registers and applied to all NS systems.
 #pragma once
@@ -28,9 +30,13 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "fixed.cuh"
+
 namespace stag {
 
-enum { P64 = 0, P32 = 1, P16 = 2, PBF = 3 };
+// PFX: FP64 links held as fixed-point limbs (fixed.cuh), their products with
+// FP64 vectors formed on the integer pipe (k_dslash_fx)
+enum { P64 = 0, P32 = 1, P16 = 2, PBF = 3, PFX = 4 };
 
 template <int P> struct Tr;
 template <> struct Tr<P64> { typedef double R; typedef double2 S2; static constexpr bool scaled = false; };
@@ -122,6 +128,9 @@ enum { FIN_NONE = 0, FIN_ALPHA = 1, FIN_NORM = 2, FIN_RESID = 3, FIN_INIT = 4, F
 struct DsArgs {
   Geom g;
   int par_out;           // parity of the output sites
+  // k_dslash_fx, one system: in / center / out are FP64 ABI vectors [Ve][3]
+  // (a caller's buffer) instead of [3][Ve]
+  int abi_in, abi_center, abi_out;
   const void *links;     // [2][4][NE][Ve] of the link storage type
   VecArg in;             // input on the other parity (EPI_CG_K1: p_old)
   VecArg center;         // EPI_MDAGM: the vector the mass term multiplies; EPI_RESID: x;
@@ -1587,6 +1596,13 @@ __global__ void k_pack_links(const double2 *__restrict__ src, void *dst, Geom g)
     d[(long long)e * g.Ve] = from_r<LP>(re, im);
   }
 }
+
+// the FP64 and the fixed-point copies of a gauge field in one pass over it;
+// *bad is set where a link is not near unitary (a row or column whose 2-norm^2
+// is off 1 by over 1e-3, a non-finite element): such a field's fixed-point
+// copy is not used
+__global__ void k_pack_links_fx(const double2 *__restrict__ src, double2 *__restrict__ dst64,
+                                int4 *__restrict__ dstfx, Geom g, int *bad);
 
 // tiled site-owned copy of the links (see the layout notes at the top): one
 // thread per (parity, site, slot); dst zeroed beforehand (the tail of the last
