@@ -2223,7 +2223,7 @@ int stag_npr_contract(stag_ctx *c, const int spin_taste[4], const double *chibar
   double2 *out = (O_hyp && is_device_ptr(O_hyp)) ? reinterpret_cast<double2 *>(O_hyp) : (double2 *)c->npr_o.p;
   double2 *sum = (double2 *)c->npr_o.p + nh;
   CK(launch_npr(c->dims, reinterpret_cast<const double2 *>(c->links_canon.p), spin_taste, d[0], d[1], d[2], d[3],
-                out, O_sum ? sum : nullptr, c->stream));
+                out, O_sum ? sum : nullptr, c->fx_ok, c->stream));
   if (O_hyp && out == (double2 *)c->npr_o.p)
     CK(cudaMemcpyAsync(O_hyp, out, sizeof(double2) * (size_t)nh, cudaMemcpyDeviceToHost, c->stream));
   if (O_sum) CK(cudaMemcpyAsync(O_sum, sum, sizeof(double2), cudaMemcpyDefault, c->stream));

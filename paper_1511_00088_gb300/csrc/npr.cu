@@ -23,6 +23,7 @@
 #include <cuda_runtime.h>
 
 #include "launch.h"
+#include "su3_fixed.cuh"
 
 namespace stag {
 
@@ -198,6 +199,192 @@ __global__ void __launch_bounds__(NPR_BT) k_npr(const NprArgs a) {
   }
 }
 
+// ---------------------------------------------------------------------------
+// the same contraction on the integer pipe (near-unitary fields)
+// ---------------------------------------------------------------------------
+// k_npr keeps the FP64 pipe 95 % busy (12 000 complex multiply-adds a
+// hypercube; 3.90 ms at 20^3 x 64, 1.24 ms here: issue slots 48 % and shared
+// memory 50 % busy, the levels' barriers between).  Here they are fixed-point sums (fixed.cuh): links and path
+// averages at 2^58, the fields at 2^57 under one exponent a field and
+// hypercube.  Ranges, rows and columns of a link being of norm 1 to 1e-3: an
+// element of a path product of up to 4 links is below 3 even for a field that
+// is not unitary (rank 1), so h < 2^31, and the sums of a level (4 steps of 3
+// products) stay below 2^62.3, as do those of the contraction.  FP64 is left for
+// the product of the two bilinears and the sum of the 256 terms.  A hypercube
+// whose fields hold numbers far from 1, infinities or NaNs contracts its path
+// averages in FP64 as k_npr does.
+// v / n, n = 2, 3, 4
+__device__ __forceinline__ long long fx_over(long long v, int n) {
+  return n == 2 ? v >> 1 : n == 4 ? v >> 2 : fx_third(v);
+}
+
+constexpr int NPR_E0 = 600, NPR_E1 = 1400;  // exponent fields of the integer form
+
+__global__ void __launch_bounds__(NPR_BT, 4) k_npr_fx(const NprArgs a) {
+  __shared__ int4 W[256][9];      // as k_npr, fixed-point
+  __shared__ int4 fld[4][16][3];  // the fields at the corners, fixed-point
+  __shared__ double2 term[NPR_BT];
+  __shared__ int top[4];  // largest exponent bits of a field
+  __shared__ unsigned char pa[120], pd[120];
+  const long long h = blockIdx.x;
+  int zc[4];
+  {
+    long long r = h;
+    zc[0] = (int)(r % a.H[0]);
+    r /= a.H[0];
+    zc[1] = (int)(r % a.H[1]);
+    r /= a.H[1];
+    zc[2] = (int)(r % a.H[2]);
+    zc[3] = (int)(r / a.H[2]);
+  }
+  auto site = [&](int A) -> long long {
+    const int x0 = 2 * zc[0] + (A & 1), x1 = 2 * zc[1] + ((A >> 1) & 1), x2 = 2 * zc[2] + ((A >> 2) & 1),
+              x3 = 2 * zc[3] + ((A >> 3) & 1);
+    return x0 + (long long)a.L[0] * (x1 + (long long)a.L[1] * (x2 + (long long)a.L[2] * x3));
+  };
+  const int t = threadIdx.x;
+  const int ff = t / 48, fa = (t / 3) % 16, fc = t % 3;  // this thread's field, corner and colour (t < 192)
+  const double2 *fsrc = ff == 0 ? a.cb1 : ff == 1 ? a.c2 : ff == 2 ? a.cb3 : a.c4;
+  double2 fv = make_double2(0.0, 0.0);
+  if (t < 192) fv = fsrc[site(fa) * 3 + fc];
+  if (t < 4) top[t] = 0;
+  for (int k = t; k < 32 * 9; k += NPR_BT) {
+    const int l = k / 9, e = k % 9, mu = l / 8, y = l % 8;
+    const int A = ((y >> mu) << (mu + 1)) | (y & ((1 << mu) - 1)), D = A | (1 << mu);
+    const double2 u = a.U[((long long)mu * a.V + site(A)) * 9 + e];
+    const Fx re = fx_link(__double2hiint(u.x), __double2loint(u.x));
+    const Fx im = fx_link(__double2hiint(u.y), __double2loint(u.y));
+    const int4 w = make_int4(re.h, re.l, im.h, im.l);
+    W[A * 16 + D][e] = w;
+    W[D * 16 + A][(e % 3) * 3 + e / 3] = fx_conj(w);
+  }
+  for (int k = t; k < 16 * 9; k += NPR_BT) {
+    const int Y = k / 9, e = k % 9;
+    W[Y * 17][e] = make_int4((e % 4 == 0) ? 1 << FX_LO : 0, 0, 0, 0);
+  }
+  if (t < 120) {
+    pa[t] = c_pairs.a[t];
+    pd[t] = c_pairs.d[t];
+  }
+  __syncthreads();
+  if (t < 192) atomicMax(&top[ff], max(__double2hiint(fv.x) & 0x7fffffff, __double2hiint(fv.y) & 0x7fffffff));
+  // levels n = 2, 3: one thread a row of W(A, D) (each W(A, P) row serves three
+  // elements); level 4, with only 8 pairs: one thread an element
+#pragma unroll
+  for (int n = 2; n <= 4; ++n) {
+    const int p0 = c_pairs.off[n - 1], np = c_pairs.off[n] - p0;
+    constexpr int COLS = 3;
+    const int per = n < 4 ? 3 : 9;
+    for (int item = t; item < np * per; item += NPR_BT) {
+      const int pr = p0 + item / per, e = item % per;
+      const int A = pa[pr], D = pd[pr];
+      const int i = n < 4 ? e : e / 3, j0 = n < 4 ? 0 : e % 3;
+      CAcc c[COLS];
+#pragma unroll
+      for (int j = 0; j < COLS; ++j) c[j] = cacc_zero();
+      for (int mu = 0; mu < 4; ++mu) {
+        if (!(((A ^ D) >> mu) & 1)) continue;
+        const int Pm = D ^ (1 << mu);
+        const int4 *wa = W[A * 16 + Pm], *wb = W[Pm * 16 + D];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const int4 x = wa[i * 3 + k];
+          if (n < 4) {
+#pragma unroll
+            for (int j = 0; j < COLS; ++j) fx_cmac(c[j], x, wb[k * 3 + j]);
+          } else {
+            fx_cmac(c[0], x, wb[k * 3 + j0]);
+          }
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < COLS; ++j) {
+        if (n == 4 && j > 0) break;
+        const int4 w = fx_pair(fx_over(fx_sum(c[j].re), n), fx_over(fx_sum(c[j].im), n));
+        W[A * 16 + D][i * 3 + j0 + j] = w;
+        W[D * 16 + A][(j0 + j) * 3 + i] = fx_conj(w);
+      }
+    }
+    __syncthreads();
+  }
+  int E[4];
+  bool wide = false;  // uniform over the block
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+    E[f] = top[f] >> 20;
+    wide |= E[f] < NPR_E0 || E[f] > NPR_E1;
+  }
+  const int A = t >> 4, C = t & 15;
+  const int B = A ^ a.S1 ^ a.F1, Dd = C ^ a.S2 ^ a.F2;
+  const double s = spin_taste(a.S1, a.F1, A, B) * spin_taste(a.S2, a.F2, C, Dd);
+  if (!wide) {
+    if (t < 192) {
+      const int Ef = top[ff] >> 20;
+      const Fx re = fx_vec(__double2hiint(fv.x), __double2loint(fv.x), Ef);
+      const Fx im = fx_vec(__double2hiint(fv.y), __double2loint(fv.y), Ef);
+      fld[ff][fa][fc] = make_int4(re.h, re.l, im.h, im.l);
+    }
+    __syncthreads();
+    // one bilinear: x^T W y with x, y at 2^57, W at 2^58: W y at 2^57, the sum at 2^56
+    auto bilinear = [&](const int4 *x, const int4 *w, const int4 *y, long long &re, long long &im) {
+      CAcc sum = cacc_zero();
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        CAcc v = cacc_zero();
+#pragma unroll
+        for (int j = 0; j < 3; ++j) fx_cmac(v, w[i * 3 + j], y[j]);
+        fx_cmac(sum, x[i], fx_cval(v));
+      }
+      re = fx_sum(sum.re);
+      im = fx_sum(sum.im);
+    };
+    long long r1, i1, r2, i2;
+    bilinear(fld[0][A], W[A * 16 + Dd], fld[3][Dd], r1, i1);
+    bilinear(fld[2][C], W[C * 16 + B], fld[1][B], r2, i2);
+    // units 2^(E - 1022) of each field and 2^-56
+    const double u1 = s * __hiloint2double((E[0] + E[3] - 2 * 1022 - 56 + 1023) << 20, 0);
+    const double u2 = __hiloint2double((E[1] + E[2] - 2 * 1022 - 56 + 1023) << 20, 0);
+    term[t] = zm(make_double2((double)r1 * u1, (double)i1 * u1), make_double2((double)r2 * u2, (double)i2 * u2));
+  } else {
+    // the path averages to FP64 in place, the fields as they are
+    double2 *Wd = reinterpret_cast<double2 *>(&W[0][0]);
+    for (int k = t; k < 256 * 9; k += NPR_BT) {
+      const int4 w = (&W[0][0])[k];
+      Wd[k] = make_double2(__fma_rn((double)w.x, 0x1p-29, (double)w.y * 0x1p-58),
+                           __fma_rn((double)w.z, 0x1p-29, (double)w.w * 0x1p-58));
+    }
+    double2 *fd = reinterpret_cast<double2 *>(&fld[0][0][0]);
+    if (t < 192) fd[t] = fv;
+    __syncthreads();
+    double2 t1 = make_double2(0.0, 0.0), t2 = make_double2(0.0, 0.0);
+#pragma unroll 1
+    for (int i = 0; i < 3; ++i) {
+      double2 v1 = make_double2(0.0, 0.0), v2 = make_double2(0.0, 0.0);
+      for (int j = 0; j < 3; ++j) {
+        v1 = zfma(Wd[(A * 16 + Dd) * 9 + i * 3 + j], fd[(3 * 16 + Dd) * 3 + j], v1);
+        v2 = zfma(Wd[(C * 16 + B) * 9 + i * 3 + j], fd[(16 + B) * 3 + j], v2);
+      }
+      t1 = zfma(fd[A * 3 + i], v1, t1);
+      t2 = zfma(fd[(2 * 16 + C) * 3 + i], v2, t2);
+    }
+    const double2 z = zm(t1, t2);
+    term[t] = make_double2(s * z.x, s * z.y);
+  }
+  __syncthreads();
+  // fixed-order sum of the 256 terms by one warp
+  if (t < 32) {
+    double2 o = term[t];
+#pragma unroll
+    for (int k = 1; k < NPR_BT / 32; ++k) o = za(o, term[t + 32 * k]);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      o.x += __shfl_xor_sync(0xffffffffu, o.x, d);
+      o.y += __shfl_xor_sync(0xffffffffu, o.y, d);
+    }
+    if (t == 0) a.out[h] = o;
+  }
+}
+
 // out[0] = sum of the n values of in, fixed order (one block)
 __global__ void __launch_bounds__(NPR_BT) k_npr_sum(const double2 *in, long long n, double2 *out) {
   __shared__ double2 red[NPR_BT / 32];
@@ -220,7 +407,7 @@ __global__ void __launch_bounds__(NPR_BT) k_npr_sum(const double2 *in, long long
 }  // namespace
 
 cudaError_t launch_npr(const int dims[4], const double2 *U, const int st[4], const double2 *cb1, const double2 *c2,
-                       const double2 *cb3, const double2 *c4, double2 *out, double2 *sum, cudaStream_t s) {
+                       const double2 *cb3, const double2 *c4, double2 *out, double2 *sum, bool fx, cudaStream_t s) {
   NprArgs a;
   long long nh = 1;
   for (int k = 0; k < 4; ++k) {
@@ -239,7 +426,8 @@ cudaError_t launch_npr(const int dims[4], const double2 *U, const int st[4], con
   a.S2 = st[2];
   a.F2 = st[3];
   a.out = out;
-  k_npr<<<(unsigned)nh, NPR_BT, 0, s>>>(a);
+  if (fx) k_npr_fx<<<(unsigned)nh, NPR_BT, 0, s>>>(a);
+  else k_npr<<<(unsigned)nh, NPR_BT, 0, s>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || !sum) return e;
   k_npr_sum<<<1, NPR_BT, 0, s>>>(out, nh, sum);
