@@ -17,11 +17,14 @@
 // g = |det Y|^(-1/3); Higham, "Computing the polar decomposition", 1986),
 // which reaches the same unique factor in fewer steps than the plain one, and
 // the determinant's phase from Newton's iteration for a complex cube root.
+// Near-unitary fields run on the integer pipe instead (k_hyp*_fx below).
 // One thread per (decorated link, site); links in the ABI layout
 // [direction][site][3][3] complex (decorated: [12 (mu, decoration) slots][site][3][3]).
+#include <cmath>
 #include <cuda_runtime.h>
 
 #include "launch.h"
+#include "su3_fixed.cuh"
 
 namespace stag {
 
@@ -222,8 +225,11 @@ __device__ __forceinline__ void smear_store(const double2 *u, double a, double w
   for (int k = 0; k < 9; ++k) out[k] = W.a[k];
 }
 
+// The FP64 levels.  run != nullptr: only where *run is set (a field that the
+// fixed-point levels left alone).
 // level 1: thread over (mu, e != mu, site); Vb stored [dslot(mu, e)][V]
-__global__ void k_hyp1(Lat g, const double2 *U, double a3, double2 *Vb) {
+__global__ void k_hyp1(Lat g, const int *run, const double2 *U, double a3, double2 *Vb) {
+  if (run != nullptr && *run == 0) return;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 12 * g.V) return;
   const long long i = t % g.V;
@@ -239,7 +245,8 @@ __global__ void k_hyp1(Lat g, const double2 *U, double a3, double2 *Vb) {
 }
 
 // level 2: thread over (mu, nu != mu, site); Vt stored [dslot(mu, nu)][V]
-__global__ void k_hyp2(Lat g, const double2 *U, const double2 *Vb, double a2, double2 *Vt) {
+__global__ void k_hyp2(Lat g, const int *run, const double2 *U, const double2 *Vb, double a2, double2 *Vt) {
+  if (run != nullptr && *run == 0) return;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 12 * g.V) return;
   const long long i = t % g.V;
@@ -259,7 +266,8 @@ __global__ void k_hyp2(Lat g, const double2 *U, const double2 *Vb, double a2, do
 }
 
 // level 3: thread over (mu, site); out may alias U (each thread reads only its own thin link)
-__global__ void k_hyp3(Lat g, const double2 *U, const double2 *Vt, double a1, double2 *out) {
+__global__ void k_hyp3(Lat g, const int *run, const double2 *U, const double2 *Vt, double a1, double2 *out) {
+  if (run != nullptr && *run == 0) return;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 4 * g.V) return;
   const long long i = t % g.V;
@@ -295,21 +303,303 @@ __global__ void k_hyp3(Lat g, const double2 *U, const double2 *Vt, double a1, do
   smear_store(u, a1, a1 / 6.0, acc, out + ((long long)mu * g.V + i) * 9);
 }
 
+// ---------------------------------------------------------------------------
+// the same three levels on the integer pipe (near-unitary fields)
+// ---------------------------------------------------------------------------
+// The FP64 levels keep the FP64 pipe 95 % busy: per site 20 700 FMAs of staples
+// and 33 600 of projections (44.8 ms at 20^3 x 64).  Here the staples are
+// fixed-point products (fixed.cuh; decorated links are SU(3), the thin ones within
+// 1e-3 of unitary, so products stay below 2) and the projection is
+// project_su3_fx.  The sum to project is formed as c U + (staples) 2^-q with
+// c = 2^-q (1 - a) / w and 2^q >= (1 - a) / w + number of staples: P ignores a
+// positive scale.  Fields lie as [slot][element][site] int4, so that a warp's
+// 32 sites are 512 contiguous bytes a load.  A thread whose projection does not
+// converge (a sum near singular) projects in FP64; where that has no result
+// either, levels 1 and 2 set *bad, as the conversion does on a field that is not
+// near unitary, and the FP64 levels run.
+struct FLat {
+  Lat g;
+  FastDiv d0, d1, d2;
+};
+
+__device__ __forceinline__ void coords_fx(const FLat &f, unsigned i, int (&x)[4]) {
+  const unsigned q1 = fast_div(i, f.d0), q2 = fast_div(q1, f.d1), q3 = fast_div(q2, f.d2);
+  x[0] = (int)(i - q1 * f.g.L[0]);
+  x[1] = (int)(q1 - q2 * f.g.L[1]);
+  x[2] = (int)(q2 - q3 * f.g.L[2]);
+  x[3] = (int)q3;
+}
+
+// the site one step s = +-1 from site i (coordinate xd) in direction d
+__device__ __forceinline__ unsigned step_fx(const FLat &f, unsigned i, int xd, int d, int s) {
+  const unsigned str = d == 0 ? 1u : d == 1 ? (unsigned)f.g.L[0]
+                                 : d == 2 ? (unsigned)(f.g.L[0] * f.g.L[1])
+                                          : (unsigned)(f.g.L[0] * f.g.L[1] * f.g.L[2]);
+  const int L = f.g.L[d];
+  const int k = s > 0 ? (xd + 1 == L ? 1 - L : 1) : (xd == 0 ? L - 1 : -1);
+  return i + (unsigned)(k * (int)str);
+}
+
+constexpr int HFX_BT = 128;
+
+// two 64-bit integers in the four words of an int4
+__device__ __forceinline__ long long lo64(const int4 &v) { return ((long long)v.y << 32) | (unsigned)v.x; }
+__device__ __forceinline__ long long hi64(const int4 &v) { return ((long long)v.w << 32) | (unsigned)v.z; }
+__device__ __forceinline__ int4 pack64(long long a, long long b) {
+  return make_int4((int)a, (int)(a >> 32), (int)b, (int)(b >> 32));
+}
+
+// X (unit 2^-58, pairs of 64-bit sums, one column of shared memory a thread: element k at X[k HFX_BT])
+// += a b c^dag (neg = 0) or a^dag b c (neg = 1); each factor at p + element V.
+// One body serves both: the daggers are strides and signs.
+__device__ __forceinline__ void staple_fx(const int4 *pa, const int4 *pb, const int4 *pc, int V, int neg, int4 *X) {
+  int4 b[9], c[9], a[3], an[3];
+  const int ra = neg ? V : 3 * V, ca = neg ? 3 * V : V;  // row i of (a or a^dag): i ra + k ca
+  const int rc = neg ? 3 * V : V, cc = neg ? V : 3 * V;  // element (k, j) of (c^dag or c): k rc + j cc
+  const int sa = neg ? -1 : 1, sc = -sa;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) a[k] = __ldg(pa + k * ca);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) b[k] = __ldg(pb + k * V);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    c[k] = __ldg(pc + (k / 3) * rc + (k % 3) * cc);
+    c[k].z *= sc;
+    c[k].w *= sc;
+  }
+#pragma unroll 1
+  for (int i = 0; i < 3; ++i) {
+    const int nx = i < 2 ? (i + 1) * ra : 0;  // the next row, in flight while this one is computed
+#pragma unroll
+    for (int k = 0; k < 3; ++k) an[k] = __ldg(pa + nx + k * ca);
+    int4 t[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      a[k].z *= sa;
+      a[k].w *= sa;
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      CAcc s = cacc_zero();
+#pragma unroll
+      for (int k = 0; k < 3; ++k) fx_cmac(s, a[k], b[3 * k + j]);
+      t[j] = fx_cval(s);
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      CAcc s = cacc_zero();
+#pragma unroll
+      for (int k = 0; k < 3; ++k) fx_cmac(s, t[k], c[3 * k + j]);
+      const int4 x = X[(3 * i + j) * HFX_BT];
+      X[(3 * i + j) * HFX_BT] = pack64(lo64(x) + fx_sum(s.re), hi64(x) + fx_sum(s.im));
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) a[k] = an[k];
+  }
+}
+
+// P(X) in FP64 where the fixed-point projection gave up; false: no finite result
+__device__ __noinline__ bool project_fallback(const int4 *X, int4 *W) {
+  M3 x;
+  for (int k = 0; k < 9; ++k) {
+    const int4 v = X[k * HFX_BT];
+    x.a[k] = make_double2((double)fx_join(v.x, v.y) * 0x1p-58, (double)fx_join(v.z, v.w) * 0x1p-58);
+  }
+  const M3 w = project_su3(x);
+  bool ok = true;
+  for (int k = 0; k < 9; ++k) {
+    ok = ok && fabs(w.a[k].x) < 1.5 && fabs(w.a[k].y) < 1.5;
+    W[k * HFX_BT] = fx_pair(__double2ll_rn(w.a[k].x * 0x1p58), __double2ll_rn(w.a[k].y * 0x1p58));
+  }
+  return ok;
+}
+
+struct HfxShared {
+  int4 X[9][HFX_BT];   // the staple sums (64-bit), then the matrix to project
+  int4 Q[9][HFX_BT];   // its projection
+  float f[27][HFX_BT];
+};
+
+// the link's mix of c U and the staples in X, and its projection into Q; c = (h, l) limbs
+__device__ __forceinline__ bool smear_fx(const int4 *pu, long long V, Fx c, int q, int4 *X, int4 *Q, float *f) {
+  const long long half = q > 0 ? 1ll << (q - 1) : 0ll;
+#pragma unroll 3
+  for (int k = 0; k < 9; ++k) {
+    const int4 u = __ldg(pu + k * V);
+    FxAcc re, im;
+    re.hh = re.cr = im.hh = im.cr = 0;
+    fx_mac(re, u.x, u.y, c.h, c.l);
+    fx_mac(im, u.z, u.w, c.h, c.l);
+    const int4 s = X[k * HFX_BT];
+    X[k * HFX_BT] = fx_pair(fx_sum(re) + ((lo64(s) + half) >> q), fx_sum(im) + ((hi64(s) + half) >> q));
+  }
+  if (project_su3_fx<HFX_BT>(X, Q, f)) return true;
+  return project_fallback(X, Q);
+}
+
+// canonical FP64 links -> [mu][9][V] fixed-point; *bad where not near unitary
+__global__ void __launch_bounds__(256) k_hyp_fix(long long V, const double2 *__restrict__ U, int4 *F, int *bad) {
+  const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
+  if (t >= 4 * V) return;
+  const long long mu = t / V, i = t - mu * V;
+  float row[3] = {0.f, 0.f, 0.f}, col[3] = {0.f, 0.f, 0.f};
+  bool ok = true;
+#pragma unroll
+  for (int e = 0; e < 9; ++e) {
+    const double2 w = U[t * 9 + e];
+    const int hx = __double2hiint(w.x), hy = __double2hiint(w.y);
+    ok = ok && (hx & 0x7fffffff) < 0x40000000 && (hy & 0x7fffffff) < 0x40000000;
+    const Fx a = fx_link(hx, __double2loint(w.x)), b = fx_link(hy, __double2loint(w.y));
+    F[(mu * 9 + e) * V + i] = make_int4(a.h, a.l, b.h, b.l);
+    const float x = (float)a.h * 0x1p-29f, y = (float)b.h * 0x1p-29f, n = x * x + y * y;
+    row[e / 3] += n;
+    col[e % 3] += n;
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) ok = ok && fabsf(row[k] - 1.f) <= 1e-3f && fabsf(col[k] - 1.f) <= 1e-3f;
+  if (!ok) *bad = 1;
+}
+
+struct HypFx {
+  FLat f;
+  long long V;
+  const int4 *U;  // [4][9][V]
+  int *bad;
+  Fx c;
+  int q;
+};
+
+// level 1 (LEVEL = 1: Vb from U) and level 2 (Vt from Vb); blockIdx.y = slot
+template <int LEVEL>
+__global__ void __launch_bounds__(HFX_BT, 3) k_hyp12_fx(const HypFx h, const int4 *__restrict__ src, int4 *dst) {
+  if (*(volatile int *)h.bad != 0) return;
+  // threads past the last site repeat it (whole warps project together) and store nothing
+  const unsigned i0 = blockIdx.x * HFX_BT + threadIdx.x, i = i0 < h.V ? i0 : (unsigned)h.V - 1;
+  const int pr = blockIdx.y, mu = pr / 3, e = (pr % 3 >= mu) ? pr % 3 + 1 : pr % 3;
+  const long long V = h.V;
+  int x[4];
+  coords_fx(h.f, i, x);
+  const int xmu = mu == 0 ? x[0] : mu == 1 ? x[1] : mu == 2 ? x[2] : x[3];
+  const unsigned imu = step_fx(h.f, i, xmu, mu, 1);
+  extern __shared__ HfxShared hsh[];
+  int4 *X = &hsh->X[0][threadIdx.x], *Q = &hsh->Q[0][threadIdx.x];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) X[k * HFX_BT] = make_int4(0, 0, 0, 0);
+#pragma unroll 1
+  for (int d = 0; d < 4; ++d) {
+    if (LEVEL == 1 ? d != e : (d == mu || d == e)) continue;
+    const int s = 6 - mu - e - d;  // level 2: the direction outside {mu, nu, d}
+    const int4 *A = src + (LEVEL == 1 ? d : dslot(d, s)) * 9 * V;
+    const int4 *B = src + (LEVEL == 1 ? mu : dslot(mu, s)) * 9 * V;
+    const int xd = d == 0 ? x[0] : d == 1 ? x[1] : d == 2 ? x[2] : x[3];
+    const unsigned up = step_fx(h.f, i, xd, d, 1), dn = step_fx(h.f, i, xd, d, -1), dnmu = step_fx(h.f, imu, xd, d, -1);
+#pragma unroll 1
+    for (int neg = 0; neg < 2; ++neg)
+      staple_fx(A + (neg ? dn : i), B + (neg ? dn : up), A + (neg ? dnmu : imu), (int)V, neg, X);
+  }
+  if (!smear_fx(h.U + (long long)mu * 9 * V + i, V, h.c, h.q, X, Q, &hsh->f[0][threadIdx.x])) *h.bad = 1;
+  if (i0 >= h.V) return;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) dst[((long long)pr * 9 + k) * V + i] = Q[k * HFX_BT];
+}
+
+// level 3 (the smeared links, FP64 ABI layout; may be the buffer U came from); blockIdx.y = mu
+__global__ void __launch_bounds__(HFX_BT, 3) k_hyp3_fx(const HypFx h, const int4 *__restrict__ Vt, double2 *out) {
+  if (*(volatile int *)h.bad != 0) return;
+  const unsigned i0 = blockIdx.x * HFX_BT + threadIdx.x, i = i0 < h.V ? i0 : (unsigned)h.V - 1;
+  const int mu = blockIdx.y;
+  const long long V = h.V;
+  int x[4];
+  coords_fx(h.f, i, x);
+  const int xmu = mu == 0 ? x[0] : mu == 1 ? x[1] : mu == 2 ? x[2] : x[3];
+  const unsigned imu = step_fx(h.f, i, xmu, mu, 1);
+  extern __shared__ HfxShared hsh[];
+  int4 *X = &hsh->X[0][threadIdx.x], *Q = &hsh->Q[0][threadIdx.x];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) X[k * HFX_BT] = make_int4(0, 0, 0, 0);
+#pragma unroll 1
+  for (int nu = 0; nu < 4; ++nu) {
+    if (nu == mu) continue;
+    const int4 *A = Vt + dslot(nu, mu) * 9 * V, *B = Vt + dslot(mu, nu) * 9 * V;
+    const int xn = nu == 0 ? x[0] : nu == 1 ? x[1] : nu == 2 ? x[2] : x[3];
+    const unsigned up = step_fx(h.f, i, xn, nu, 1), dn = step_fx(h.f, i, xn, nu, -1), dnmu = step_fx(h.f, imu, xn, nu, -1);
+#pragma unroll 1
+    for (int neg = 0; neg < 2; ++neg)
+      staple_fx(A + (neg ? dn : i), B + (neg ? dn : up), A + (neg ? dnmu : imu), (int)V, neg, X);
+  }
+  const bool ok = smear_fx(h.U + (long long)mu * 9 * V + i, V, h.c, h.q, X, Q, &hsh->f[0][threadIdx.x]);
+  if (i0 >= h.V) return;
+  const double one = ok ? 0x1p-58 : __longlong_as_double(0x7ff8000000000000ll);
+  double2 *o = out + ((long long)mu * V + i) * 9;
+#pragma unroll 3
+  for (int k = 0; k < 9; ++k) {
+    const int4 w = Q[k * HFX_BT];
+    o[k] = make_double2((double)fx_join(w.x, w.y) * one, (double)fx_join(w.z, w.w) * one);
+  }
+}
+
+// coefficient and shift of a level; false where the fixed-point mix does not hold it
+bool mix_of(double a, double w, int staples, Fx *c, int *q) {
+  if (!(a > 0.0) || !(a <= 1.0)) return false;
+  const double r = (1.0 - a) / w;
+  if (!(r <= 60.0)) return false;
+  *q = 0;
+  while ((double)(1 << *q) < r + staples) ++*q;
+  const long long C = llrint(ldexp(r, 58 - *q));
+  *c = fx_split(C);
+  return true;
+}
+
 }  // namespace
 
 cudaError_t launch_hyp(const int dims[4], const double2 *U, const double alpha[3], double2 *Vb, double2 *Vt,
-                       double2 *out, cudaStream_t st) {
+                       double2 *out, void *fixU, int *bad, cudaStream_t st) {
   Lat g;
   for (int k = 0; k < 4; ++k) g.L[k] = dims[k];
   g.V = (long long)dims[0] * dims[1] * dims[2] * dims[3];
   const int bt = 128;
-  k_hyp1<<<(unsigned)((12 * g.V + bt - 1) / bt), bt, 0, st>>>(g, U, alpha[2], Vb);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_hyp2<<<(unsigned)((12 * g.V + bt - 1) / bt), bt, 0, st>>>(g, U, Vb, alpha[1], Vt);
+  Fx c[3];
+  int q[3];
+  cudaError_t e = cudaSuccess;
+  const int *run = nullptr;
+  if (fixU != nullptr && g.V < (1ll << 27) && mix_of(alpha[2], alpha[2] / 2.0, 2, &c[0], &q[0]) &&
+      mix_of(alpha[1], alpha[1] / 4.0, 4, &c[1], &q[1]) && mix_of(alpha[0], alpha[0] / 6.0, 6, &c[2], &q[2])) {
+    for (const void *k : {(const void *)k_hyp12_fx<1>, (const void *)k_hyp12_fx<2>, (const void *)k_hyp3_fx}) {
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(HfxShared));
+      if (e != cudaSuccess) return e;
+    }
+    e = cudaMemsetAsync(bad, 0, sizeof(int), st);
+    if (e != cudaSuccess) return e;
+    run = bad;
+    HypFx h;
+    h.f.g = g;
+    h.f.d0 = make_fastdiv((unsigned)dims[0]);
+    h.f.d1 = make_fastdiv((unsigned)dims[1]);
+    h.f.d2 = make_fastdiv((unsigned)dims[2]);
+    h.V = g.V;
+    h.U = reinterpret_cast<const int4 *>(fixU);
+    h.bad = bad;
+    k_hyp_fix<<<(unsigned)((4 * g.V + 255) / 256), 256, 0, st>>>(g.V, U, reinterpret_cast<int4 *>(fixU), bad);
+    const unsigned nb = (unsigned)((g.V + HFX_BT - 1) / HFX_BT);
+    h.c = c[0];
+    h.q = q[0];
+    k_hyp12_fx<1><<<dim3(nb, 12), HFX_BT, sizeof(HfxShared), st>>>(h, h.U, reinterpret_cast<int4 *>(Vb));
+    h.c = c[1];
+    h.q = q[1];
+    k_hyp12_fx<2><<<dim3(nb, 12), HFX_BT, sizeof(HfxShared), st>>>(h, reinterpret_cast<const int4 *>(Vb), reinterpret_cast<int4 *>(Vt));
+    h.c = c[2];
+    h.q = q[2];
+    k_hyp3_fx<<<dim3(nb, 4), HFX_BT, sizeof(HfxShared), st>>>(h, reinterpret_cast<const int4 *>(Vt), out);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  k_hyp1<<<(unsigned)((12 * g.V + bt - 1) / bt), bt, 0, st>>>(g, run, U, alpha[2], Vb);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_hyp3<<<(unsigned)((4 * g.V + bt - 1) / bt), bt, 0, st>>>(g, U, Vt, alpha[0], out);
+  k_hyp2<<<(unsigned)((12 * g.V + bt - 1) / bt), bt, 0, st>>>(g, run, U, Vb, alpha[1], Vt);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_hyp3<<<(unsigned)((4 * g.V + bt - 1) / bt), bt, 0, st>>>(g, run, U, Vt, alpha[0], out);
   return cudaGetLastError();
 }
 
