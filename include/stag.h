@@ -150,8 +150,9 @@ int stag_mdagm(stag_ctx *ctx, int precision, double mass, const double *in_even,
  * Returns STAG_OK when every system converged, STAG_NOT_CONVERGED when some
  * system hit maxiter (its x is the last iterate), STAG_ERR_BREAKDOWN on a
  * non-positive <p, A p> or a non-finite residual, STAG_ERR_TIMEOUT when a
- * kernel's bounded wait for its staged links gave up (only with the
- * shared-memory link path, STAG_TMA=1), STAG_ERR_ARG / _STATE / _CUDA.
+ * kernel's bounded wait gave up (for its staged links, with the shared-memory
+ * link path, STAG_TMA=1; for the other blocks of its grid, in the persistent
+ * form), STAG_ERR_ARG / _STATE / _CUDA.
  */
 int stag_cg_solve(stag_ctx *ctx, const double *const src[], int nrhs, const double masses[],
                   int nmass, double tol, int maxiter, int precision, double *const x[],
@@ -259,7 +260,9 @@ int stag_solve_full(stag_ctx *ctx, const double *const src[], int nrhs, const do
  * (the default), an event between two launches would stop the overlap of a
  * kernel's launch with its predecessor's tail that the solve has, so the
  * pairs are also timed with events only around the whole sequence and each
- * kernel is given its share, from the separated timings, of that pair time:
+ * kernel is given its share, from the separated timings, of that pair time
+ * (where solves run in the persistent form, stag_solve_form out[7] = 4, the two
+ * kernels are timed in their one-lane form, which those solves do not launch):
  *   kernel 0: t = D_oe r + beta t_old (FP32/FP64 Krylov vectors) or
  *             t = D_oe (r + beta p_old) (STAG_HALF_VECTORS), with |t|^2;
  *   kernel 1: p = r + beta p_old, r -= alpha (4 m^2 p - D_eo t),
@@ -316,7 +319,8 @@ int stag_solve_stats(const stag_ctx *ctx, int sys, int *iters, int *reliable_upd
  * executions of the FP64 reliable-update step (Sec. 3; each recomputes the
  * residual of every system with an update due).  From them the kernels
  * launched follow: 2 U + 1 per pass and 5 per update step (4 with
- * STAG_HALF_VECTORS).  Either pointer may be NULL.  STAG_ERR_ARG before the
+ * STAG_HALF_VECTORS); with the persistent kernel (stag_solve_form out[7] = 4) a
+ * pass is 2 launches and runs every system up to its next update.  Either pointer may be NULL.  STAG_ERR_ARG before the
  * first solve.
  */
 int stag_solve_counters(const stag_ctx *ctx, int *loop_passes, int *update_steps);
@@ -333,7 +337,9 @@ int stag_solve_counters(const stag_ctx *ctx, int *loop_passes, int *update_steps
  * block (one warp per system), 2 when every block runs every system on
  * links staged once per tile in shared memory (out[0] = the systems,
  * out[2] = out[3] = threads per site), 3 the same with the first kernel
- * taking two systems per pass through each thread.  Implementation detail of this
+ * taking two systems per pass through each thread, 4 when one persistent
+ * cooperative kernel runs all iterations up to the next reliable update
+ * (then out[2] = out[3] = its lanes per site, and out[6] does not apply).  Implementation detail of this
  * library (the paper has no counterpart), for reports.  STAG_ERR_ARG before
  * the first solve.
  */

@@ -25,8 +25,13 @@
 // the pass's finalize / K6's finalize sets ("any system still running"); the
 // update kernels sit in an IF node set by the pass's finalize.  One graph
 // launch runs the whole solve.
+// Where the persistent form is the better one (choose_persist: lattices whose
+// links stay in L2, a few systems), the two kernels of all iterations up to the
+// next reliable update are one cooperative kernel (k_cg_persist), so a pass is
+// that kernel and the updates.
 // Without conditional-node support the same kernel sequence runs eagerly, with
 // the host polling a device flag every few loop passes.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -150,6 +155,9 @@ struct Work {
                                    // the links staged once per tile): threads per site, + 10 with
                                    // one link stage
   const void *links_tile = nullptr;
+  int ps_form = 0;                 // > 0: the iterations run in k_cg_persist, this form
+  int ps_blocks = 0;               // its blocks, all systems together
+  DevBuf ps_sync;                  // its exchange words and arrival counts
   int nbx_bl = 0, pstride = 0;
   VecBuf b64, x64, t64, r, x, p, t;
   DevBuf vpool;  // r, x, p, t (and their scales) in one range: one L2 window can cover them
@@ -196,12 +204,16 @@ struct stag_ctx {
   std::string err;
   bool have_links = false;
   bool use_graph = true;
+  bool coop = false;   // the device runs cooperative launches
+  int nsm = 0;
+  int ps_mode = -1;    // k_cg_persist: -1 by rule, 0 never, else this form (STAG_PS)
   bool pdl = true;  // CG kernels launched as programmatic dependents of their predecessors
   bool fold = true;     // each CG kernel finishes its predecessor's reduction itself
   bool persist = true;  // CG kernels launched as one wave of resident blocks
   int tma_modes = 0b101;  // link paths (bit t: DsArgs::tma = t) the tuner may choose for one system
-  // STAG_TEST_WAIT_GIVEUP=1: in the solve loop, the bounded waits of the
-  // shared-memory link path give up at once (tests of the failure path)
+  // STAG_TEST_WAIT_GIVEUP=1: in the solve loop, the bounded waits (of the
+  // shared-memory link path, of the persistent kernel's blocks for one another)
+  // give up at once (tests of the failure path)
   int wait_giveup = 0;
   // L2 residency of the inner-precision links during a solve: the CG kernels
   // mark them as an access-policy window whose lines persist in L2 (the rest
@@ -593,26 +605,31 @@ struct CgForm {
   int tma = 0, l1 = 1, l2 = 1, l2p = 0;  // link path, lanes of the two kernels, L2-persisting links
 };
 
+// What may persist in L2 during a solve (bit 0 nothing, 1 the links, 2 the
+// Krylov vectors): by rule, not by timing -- short timings favoured persisting
+// links where whole solves ran slower.  The links for one system whose links
+// fit the persisting set-aside to within 25 % (20^3 x 64 reconstruct-12 FP32:
+// 98 MB against 84.7 MB, 10 % faster solves); nothing where they do not fit
+// (full FP32 links, 147 MB: 6 % slower) and for several systems, whose vectors
+// need the rest of L2 (16 sources: 27 % slower).
+int l2_modes_for(const stag_ctx *c, int LP, int recon, int nsys) {
+  if (!c->l2persist) return 1;
+  if (c->l2_modes != 0b11) return c->l2_modes;
+  const int rc = (LP != P64 && recon) ? 1 : 0;
+  const double lb = (double)cplx_bytes(LP) * (rc ? 6 : 9) * 8.0 * c->Ve;
+  return (nsys == 1 && lb <= 1.25 * (double)c->l2_max_persist) ? 0b10 : 0b01;
+}
+// the same as one choice: 0 nothing, 1 the links, 2 the Krylov vectors
+int persisting_links(const stag_ctx *c, int LP, int recon, int nsys) {
+  const int m = l2_modes_for(c, LP, recon, nsys);
+  return (m & 0b100) ? 2 : (m & 0b010) ? 1 : 0;
+}
+
 int tune_cg_pair(stag_ctx *c, int LP, int recon, int VP, int NS, int EPI1, DsArgs a1, DsArgs a2, bool tma_ok,
                  CgForm *out, float *ms_out = nullptr) {
   if (ms_out) *ms_out = -1.f;
   const int modes = tma_ok ? c->tma_modes : 1;  // bit t: link path t allowed
-  // persisting links (bit p of l2modes: p allowed): by rule, not by timing --
-  // short timings favoured them where whole solves ran slower.  On for one
-  // system whose links fit the persisting set-aside to within 25 % (20^3 x 64
-  // reconstruct-12 FP32: 98 MB against 84.7 MB, 10 % faster solves); off where
-  // they do not fit (full FP32 links, 147 MB: 6 % slower) and for several
-  // systems, whose vectors need the rest of L2 (16 sources: 27 % slower).
-  int l2modes = 1;
-  if (c->l2persist) {
-    if (c->l2_modes != 0b11) {
-      l2modes = c->l2_modes;
-    } else {
-      const int rc = (LP != P64 && recon) ? 1 : 0;
-      const double lb = (double)cplx_bytes(LP) * (rc ? 6 : 9) * 8.0 * c->Ve;
-      l2modes = (a1.nsys == 1 && lb <= 1.25 * (double)c->l2_max_persist) ? 0b10 : 0b01;
-    }
-  }
+  const int l2modes = l2_modes_for(c, LP, recon, a1.nsys);
   // STAG_LANES = 1 or 2 fixes the lanes of both kernels; two digits (12, 21
   // ...) those of the first and the second
   const char *force = getenv("STAG_LANES");
@@ -626,7 +643,7 @@ int tune_cg_pair(stag_ctx *c, int LP, int recon, int VP, int NS, int EPI1, DsArg
   if (lp_for(c, LP) == PFX) {  // one thread mapping
     CgForm f;
     f.l1 = f.l2 = FX_LANES;
-    f.l2p = (l2modes & 0b100) ? 2 : (l2modes & 0b010) ? 1 : 0;
+    f.l2p = persisting_links(c, LP, recon, a1.nsys);
     cand.push_back(f);
   } else {
   for (int p = 0; p < 3; ++p)
@@ -783,6 +800,41 @@ int tune_lanes(stag_ctx *c, int LP, int recon, int VP, int NS, int G, int nsys, 
 Ctl work_ctl(stag_ctx *c, bool graph);
 DsArgs ds_base(stag_ctx *c);
 
+// exchange words and arrival counts of k_cg_persist for nsys systems
+size_t ps_sync_bytes(int nsys) {
+  return (sizeof(unsigned long long) * 2 * PS_MAXB + sizeof(unsigned) * (PS_ASTRIDE + 2)) * (size_t)nsys + 2 * sizeof(int);
+}
+
+// The persistent form (k_cg_persist) of a workspace: lanes a site and blocks, or form 0 where the two-kernel forms are the better ones.  Measured on 152
+// SMs, us per iteration of a whole solve (persistent / two kernels):
+//   lanes: 4 while a group's warps hold all sites at once (17 280 sites a parity: 4 lanes
+//   7.3, 2 lanes 8.2 / 17.8; 24 576: 9.0, 8.3 / 16.3); 2 while two rounds do (49 152: 2 lanes 11.7,
+//   1 lane 12.6 / 23.3; 98 304: 18.6, 17.1 / 28.0); else 1;
+//   one system: while its links stay in L2 -- reconstruct-12 up to 1.25 of the persisting
+//   set-aside (20^3 x 64, 98 MB: 39.3 / 49.2; 32^3 x 64, 402 MB: 218 / 198), full links up to the
+//   set-aside (20^3 x 32, 74 MB: 25.1 / 31.0; 20^3 x 44, 101 MB: 46.2 / 43.9);
+//   several: by all systems' sites an SM, 2600 with reconstruct-12 (16^3 x 32 x 6: 50.3 / 68.2,
+//   12^3 x 24 x 12: 41.6 / 42.8; 20^3 x 64 x 2: 81.5 / 78.5), 1300 with full links (16^3 x 32 x 3:
+//   30.1 / 34.1; x 6: 58.0 / 51.2).
+void choose_persist(const stag_ctx *c, int LP, int VP, int nsys, int ms, int *form, int *blocks) {
+  *form = *blocks = 0;
+  if (!c->coop || c->ps_mode == 0 || LP != P32 || VP != P32 || ms != 0) return;
+  int nb = c->nsm / nsys;
+  if (nb > PS_MAXB) nb = PS_MAXB;
+  if (nb < 1) return;
+  const int Ve = c->Ve, rc = (c->flags & STAG_RECON12) ? 1 : 0;
+  int f = c->ps_mode;
+  if (f < 0) {
+    const double lb = 8.0 * (rc ? 6 : 9) * 8.0 * Ve, set_aside = c->l2_max_persist ? (double)c->l2_max_persist : 80e6;
+    if (nsys == 1 ? lb > (rc ? 1.25 : 1.0) * set_aside : (double)nsys * Ve > (rc ? 2600.0 : 1300.0) * c->nsm) return;
+    f = Ve <= nb * cg_persist_sites(4) ? 4 : Ve <= 2 * nb * cg_persist_sites(2) ? 2 : 1;
+  }
+  const int per = cg_persist_sites(f);
+  const int full = (Ve + per - 1) / per;
+  *form = f;
+  *blocks = (long long)nsys * full < c->nsm ? nsys * full : c->nsm;
+}
+
 int work_prepare(stag_ctx *c, int nsys, int precision, int ms = 0) {
   Work &w = c->w;
   int prec, VP, RP;
@@ -792,8 +844,13 @@ int work_prepare(stag_ctx *c, int nsys, int precision, int ms = 0) {
     w.drop_graph();
     w.ms = ms;
   }
-  if (w.nsys == nsys && w.prec == prec && w.VP == VP && w.recon == recon) return STAG_OK;
+  int psf = 0, psn = 0;
+  choose_persist(c, prec, VP, nsys, ms, &psf, &psn);
+  if (w.nsys == nsys && w.prec == prec && w.VP == VP && w.recon == recon && w.ps_form == psf) return STAG_OK;
   w.drop_graph();
+  w.ps_form = psf;
+  w.ps_blocks = psn;
+  if (psf) CK(w.ps_sync.ensure(ps_sync_bytes(nsys)));
   c->last_nsys = 0;
   w.nsys = nsys;
   w.prec = prec;
@@ -852,7 +909,7 @@ int work_prepare(stag_ctx *c, int nsys, int precision, int ms = 0) {
     a.fin = FIN_NONE;
     a.aux = w.r.arg();
     a.xlo = w.x.arg();
-    const bool tma_ok = (w.NS == 1 && prec != P64 && c->tma_modes != 1);
+    const bool tma_ok = (w.NS == 1 && prec != P64 && c->tma_modes != 1 && !w.ps_form);
     w.links_tile = nullptr;
     if (tma_ok) CKS(links_tile_for(c, prec, &w.links_tile));
     a.links_tile = w.links_tile;
@@ -866,131 +923,140 @@ int work_prepare(stag_ctx *c, int nsys, int precision, int ms = 0) {
     a2.par_out = 0;
     a2.in = w.t.arg();
     a2.center = w.p.arg();
-    // Systems per thread of the CG kernels.  NS = 1 gives every system its own
-    // blocks; the blocks of one chunk (consecutive in the grid) run together and
-    // share its links through L2.  NS = 4 or 8 holds the links in registers
-    // for all the thread's systems, at the price of registers (occupancy).
-    // Several systems: the candidates are timed (kernel pair, tune_cg_pair)
-    // and the choice cached; STAG_NS = 1, 4 or 8 fixes it.
-    std::vector<int> cands{1};
-    const bool fx = lp_for(c, prec) == PFX;  // one system a thread only
-    if (nsys >= 4 && !fx) cands.push_back(4);
-    if (nsys >= 8 && prec != P64) cands.push_back(8);
-    const char *fns = getenv("STAG_NS");
-    if (fns && (fns[0] == '1' || fns[0] == '4' || fns[0] == '8') && fns[1] == 0) {
-      const int f = fns[0] - '0';
-      if (f <= nsys && !(f == 8 && prec == P64) && !(f > 1 && fx)) cands.assign(1, f);
-    }
-    // the shared-memory kernels (k_dslash_mrhs): FP32 links and vectors, 4 or 8
-    // systems per block; encoded as 100 + nsw among the candidates
-    if (prec == P32 && VP == P32 && !(fns && fns[0] != 0)) {
-      if (nsys >= 4) cands.push_back(104);
-      if (nsys >= 8) cands.push_back(108);
-    }
-    const char *fmr = getenv("STAG_MRHS");
-    if (fmr && (fmr[0] == '4' || fmr[0] == '8') && fmr[1] == 0 && prec == P32 && VP == P32 && nsys >= 2)
-      cands.assign(1, 100 + (fmr[0] - '0'));
-    // k_cg_nrhs (every system in every block, the links staged once per tile in
-    // shared memory): FP32 links and vectors, 2..64 systems; encoded 200 + sl
-    const bool nrhs_ok = prec == P32 && VP == P32 && nsys >= 2 && nsys <= CG_NRHS_MAX;
-    if (nrhs_ok && !(fns && fns[0] != 0) && !(fmr && fmr[0] != 0)) {
-      cands.push_back(202);
-      cands.push_back(204);
-      if (recon) cands.push_back(224);
-    }
-    // STAG_NRHS = 2 or 4: this form with that many threads per site (two link
-    // stages), 14: 4 threads per site with one stage (3 blocks per SM; measured
-    // slower: 48-system 20^3 x 64 solve 3.34 s vs 2.36 s, so not a default
-    // candidate), 24: kernel 1 with two systems per pass through the thread
-    // (reconstruct-12 links; kernel 2 as form 4); 0: never this form
-    const char *fnr = getenv("STAG_NRHS");
-    if (fnr && nrhs_ok) {
-      const int f = atoi(fnr);
-      if (f == 2 || f == 4 || f == 14 || (f == 24 && recon)) cands.assign(1, 200 + f);
-    }
-    if (fnr && fnr[0] == '0' && fnr[1] == 0) {
-      std::vector<int> keep;
-      for (int v : cands)
-        if (v < 200) keep.push_back(v);
-      cands = keep;
-    }
-    const void *tiled = nullptr;
-    for (int v : cands)
-      if (v > 200) {
-        CKS(links_tile_for(c, prec, &tiled));
-        a.links_tile = a2.links_tile = tiled;
-        break;
-      }
-    int best_ns = cands[0];
-    if (cands.size() > 1) {
-      const TuneKey nkey(lp_for(c, prec), recon, VP, 2000 + nsys, tma_ok ? 1 : 0, c->dims[0], c->dims[1], c->dims[2],
-                         c->dims[3]);
-      bool cached = false;
-      {
-        std::lock_guard<std::mutex> lk(g_tune_mu);
-        tune_cache_load();
-        auto it = g_tune.find(nkey);
-        if (it != g_tune.end()) {
-          best_ns = it->second;
-          cached = true;
-        }
-      }
-      if (!cached) {
-        float best_ms = 1e30f;
-        for (int ns : cands) {
-          float ms = -1.f;
-          if (ns > 200) {
-            CKS(time_nrhs_pair(c, recon, ns - 200, a, a2, &ms));
-          } else if (ns > 100) {
-            CKS(time_mrhs_pair(c, recon, ns - 100, a, a2, &ms));
-          } else {
-            a.ngroups = a2.ngroups = (nsys + ns - 1) / ns;
-            CgForm f;
-            CKS(tune_cg_pair(c, prec, recon, VP, ns, epi1, a, a2, tma_ok && ns == 1, &f, &ms));
-          }
-          if (ms >= 0.f && ms < best_ms) {
-            best_ms = ms;
-            best_ns = ns;
-          }
-        }
-        std::lock_guard<std::mutex> lk(g_tune_mu);
-        g_tune[nkey] = best_ns;
-        tune_cache_store(nkey, best_ns);
-      }
-    }
-    w.nrhs_sl = best_ns > 200 ? best_ns - 200 : 0;
-    w.mrhs = (best_ns > 100 && best_ns < 200) ? best_ns - 100 : 0;
-    w.NS = w.mrhs ? w.mrhs : (w.nrhs_sl ? 1 : best_ns);
-    w.G = (nsys + w.NS - 1) / w.NS;
-    a.ngroups = a2.ngroups = w.G;
-    if (w.nrhs_sl) {
-      // the BLAS and update kernels keep one system per group; the CG kernels
-      // are one grid of nbx_k1 / nbx_k2 blocks, each a partial per system
-      CKS(links_tile_for(c, prec, &w.links_tile));
-      w.tma = 1;
-      w.lanes_k1 = w.lanes_k2 = w.nrhs_sl % 10;
-      w.l2p = 0;
-      CKS(nrhs_blocks(c, recon, w.nrhs_sl, EPI_CG_K1R, &w.nbx_k1));
-      CKS(nrhs_blocks(c, recon, w.nrhs_sl, EPI_CG_K2, &w.nbx_k2));
-    } else if (w.mrhs) {
-      w.tma = 0;
-      w.lanes_k1 = w.lanes_k2 = 1;
-      w.l2p = 0;
-      CKS(mrhs_blocks(c, recon, w.mrhs, EPI_CG_K1R, w.G, &w.nbx_k1));
-      CKS(mrhs_blocks(c, recon, w.mrhs, EPI_CG_K2, w.G, &w.nbx_k2));
+    if (w.ps_form) {
+      // k_cg_persist iterates; the two CG kernels are only timed (stag_time_cg_kernel)
+      w.nrhs_sl = w.mrhs = w.tma = 0;
+      w.lanes_k1 = w.lanes_k2 = w.lanes = 1;
+      w.l2p = persisting_links(c, prec, recon, nsys);
+      CKS(cg_blocks(c, prec, recon, VP, 1, epi1, 1, w.G, 0, &w.nbx_k1));
+      CKS(cg_blocks(c, prec, recon, VP, 1, EPI_CG_K2, 1, w.G, 0, &w.nbx_k2));
     } else {
-      CgForm form;
-      CKS(tune_cg_pair(c, prec, recon, VP, w.NS, epi1, a, a2, tma_ok && w.NS == 1, &form));
-      w.tma = form.tma;
-      w.lanes_k1 = form.l1;
-      w.lanes_k2 = form.l2;
-      w.l2p = form.l2p;
-      CKS(cg_blocks(c, prec, recon, VP, w.NS, epi1, w.lanes_k1, w.G, w.tma, &w.nbx_k1));
-      CKS(cg_blocks(c, prec, recon, VP, w.NS, EPI_CG_K2, w.lanes_k2, w.G, w.tma, &w.nbx_k2));
+      // Systems per thread of the CG kernels.  NS = 1 gives every system its own
+      // blocks; the blocks of one chunk (consecutive in the grid) run together and
+      // share its links through L2.  NS = 4 or 8 holds the links in registers
+      // for all the thread's systems, at the price of registers (occupancy).
+      // Several systems: the candidates are timed (kernel pair, tune_cg_pair)
+      // and the choice cached; STAG_NS = 1, 4 or 8 fixes it.
+      std::vector<int> cands{1};
+      const bool fx = lp_for(c, prec) == PFX;  // one system a thread only
+      if (nsys >= 4 && !fx) cands.push_back(4);
+      if (nsys >= 8 && prec != P64) cands.push_back(8);
+      const char *fns = getenv("STAG_NS");
+      if (fns && (fns[0] == '1' || fns[0] == '4' || fns[0] == '8') && fns[1] == 0) {
+        const int f = fns[0] - '0';
+        if (f <= nsys && !(f == 8 && prec == P64) && !(f > 1 && fx)) cands.assign(1, f);
+      }
+      // the shared-memory kernels (k_dslash_mrhs): FP32 links and vectors, 4 or 8
+      // systems per block; encoded as 100 + nsw among the candidates
+      if (prec == P32 && VP == P32 && !(fns && fns[0] != 0)) {
+        if (nsys >= 4) cands.push_back(104);
+        if (nsys >= 8) cands.push_back(108);
+      }
+      const char *fmr = getenv("STAG_MRHS");
+      if (fmr && (fmr[0] == '4' || fmr[0] == '8') && fmr[1] == 0 && prec == P32 && VP == P32 && nsys >= 2)
+        cands.assign(1, 100 + (fmr[0] - '0'));
+      // k_cg_nrhs (every system in every block, the links staged once per tile in
+      // shared memory): FP32 links and vectors, 2..64 systems; encoded 200 + sl
+      const bool nrhs_ok = prec == P32 && VP == P32 && nsys >= 2 && nsys <= CG_NRHS_MAX;
+      if (nrhs_ok && !(fns && fns[0] != 0) && !(fmr && fmr[0] != 0)) {
+        cands.push_back(202);
+        cands.push_back(204);
+        if (recon) cands.push_back(224);
+      }
+      // STAG_NRHS = 2 or 4: this form with that many threads per site (two link
+      // stages), 14: 4 threads per site with one stage (3 blocks per SM; measured
+      // slower: 48-system 20^3 x 64 solve 3.34 s vs 2.36 s, so not a default
+      // candidate), 24: kernel 1 with two systems per pass through the thread
+      // (reconstruct-12 links; kernel 2 as form 4); 0: never this form
+      const char *fnr = getenv("STAG_NRHS");
+      if (fnr && nrhs_ok) {
+        const int f = atoi(fnr);
+        if (f == 2 || f == 4 || f == 14 || (f == 24 && recon)) cands.assign(1, 200 + f);
+      }
+      if (fnr && fnr[0] == '0' && fnr[1] == 0) {
+        std::vector<int> keep;
+        for (int v : cands)
+          if (v < 200) keep.push_back(v);
+        cands = keep;
+      }
+      const void *tiled = nullptr;
+      for (int v : cands)
+        if (v > 200) {
+          CKS(links_tile_for(c, prec, &tiled));
+          a.links_tile = a2.links_tile = tiled;
+          break;
+        }
+      int best_ns = cands[0];
+      if (cands.size() > 1) {
+        const TuneKey nkey(lp_for(c, prec), recon, VP, 2000 + nsys, tma_ok ? 1 : 0, c->dims[0], c->dims[1], c->dims[2],
+                           c->dims[3]);
+        bool cached = false;
+        {
+          std::lock_guard<std::mutex> lk(g_tune_mu);
+          tune_cache_load();
+          auto it = g_tune.find(nkey);
+          if (it != g_tune.end()) {
+            best_ns = it->second;
+            cached = true;
+          }
+        }
+        if (!cached) {
+          float best_ms = 1e30f;
+          for (int ns : cands) {
+            float ms = -1.f;
+            if (ns > 200) {
+              CKS(time_nrhs_pair(c, recon, ns - 200, a, a2, &ms));
+            } else if (ns > 100) {
+              CKS(time_mrhs_pair(c, recon, ns - 100, a, a2, &ms));
+            } else {
+              a.ngroups = a2.ngroups = (nsys + ns - 1) / ns;
+              CgForm f;
+              CKS(tune_cg_pair(c, prec, recon, VP, ns, epi1, a, a2, tma_ok && ns == 1, &f, &ms));
+            }
+            if (ms >= 0.f && ms < best_ms) {
+              best_ms = ms;
+              best_ns = ns;
+            }
+          }
+          std::lock_guard<std::mutex> lk(g_tune_mu);
+          g_tune[nkey] = best_ns;
+          tune_cache_store(nkey, best_ns);
+        }
+      }
+      w.nrhs_sl = best_ns > 200 ? best_ns - 200 : 0;
+      w.mrhs = (best_ns > 100 && best_ns < 200) ? best_ns - 100 : 0;
+      w.NS = w.mrhs ? w.mrhs : (w.nrhs_sl ? 1 : best_ns);
+      w.G = (nsys + w.NS - 1) / w.NS;
+      a.ngroups = a2.ngroups = w.G;
+      if (w.nrhs_sl) {
+        // the BLAS and update kernels keep one system per group; the CG kernels
+        // are one grid of nbx_k1 / nbx_k2 blocks, each a partial per system
+        CKS(links_tile_for(c, prec, &w.links_tile));
+        w.tma = 1;
+        w.lanes_k1 = w.lanes_k2 = w.nrhs_sl % 10;
+        w.l2p = 0;
+        CKS(nrhs_blocks(c, recon, w.nrhs_sl, EPI_CG_K1R, &w.nbx_k1));
+        CKS(nrhs_blocks(c, recon, w.nrhs_sl, EPI_CG_K2, &w.nbx_k2));
+      } else if (w.mrhs) {
+        w.tma = 0;
+        w.lanes_k1 = w.lanes_k2 = 1;
+        w.l2p = 0;
+        CKS(mrhs_blocks(c, recon, w.mrhs, EPI_CG_K1R, w.G, &w.nbx_k1));
+        CKS(mrhs_blocks(c, recon, w.mrhs, EPI_CG_K2, w.G, &w.nbx_k2));
+      } else {
+        CgForm form;
+        CKS(tune_cg_pair(c, prec, recon, VP, w.NS, epi1, a, a2, tma_ok && w.NS == 1, &form));
+        w.tma = form.tma;
+        w.lanes_k1 = form.l1;
+        w.lanes_k2 = form.l2;
+        w.l2p = form.l2p;
+        CKS(cg_blocks(c, prec, recon, VP, w.NS, epi1, w.lanes_k1, w.G, w.tma, &w.nbx_k1));
+        CKS(cg_blocks(c, prec, recon, VP, w.NS, EPI_CG_K2, w.lanes_k2, w.G, w.tma, &w.nbx_k2));
+      }
     }
   }
   // the thread mapping of the plain inner and the FP64 half operators
-  CKS(tune_lanes(c, prec, recon, VP, w.NS, w.G, nsys, lo, w.p.arg(), w.t.arg(), &w.lanes));
+  if (!w.ps_form) CKS(tune_lanes(c, prec, recon, VP, w.NS, w.G, nsys, lo, w.p.arg(), w.t.arg(), &w.lanes));
   CKS(tune_lanes(c, P64, 0, P64, w.NS64, w.G64, nsys, links64_op(c), w.x64.arg(), w.t64.arg(), &w.lanes64));
   return STAG_OK;
 }
@@ -1135,6 +1201,31 @@ int enqueue_main(stag_ctx *c, cudaStream_t s, const Ctl &ctl) {
 // the states in w.st.
 int enqueue_pass(stag_ctx *c, cudaStream_t s, const Ctl &ctl, int unroll) {
   Work &w = c->w;
+  if (w.ps_form) {
+    // every running system up to its next reliable update, in one launch
+    PsArgs p;
+    memset(&p, 0, sizeof p);
+    p.g = c->g;
+    CKS(links_for(c, w.prec, &p.links));
+    p.r = w.r.arg();
+    p.p = w.p.arg();
+    p.t = w.t.arg();
+    p.x = w.x.arg();
+    p.ctl = ctl;
+    p.slots = (unsigned long long *)w.ps_sync.p;
+    p.arrived = (unsigned *)(p.slots + 2ll * PS_MAXB * w.nsys);
+    p.counted = p.arrived + (long long)PS_ASTRIDE * w.nsys;
+    p.map = (int *)(p.counted + w.nsys);
+    p.nsys = w.nsys;
+    p.giveup = c->wait_giveup;
+    DsArgs win = ds_base(c);
+    set_l2_window(c, w.prec, 0, w.l2p, win);
+    p.l2_base = win.l2_base;
+    p.l2_bytes = win.l2_bytes;
+    p.l2_hit = win.l2_hit;
+    CK(launch_cg_persist(w.recon, w.ps_form, w.ps_blocks, s, p));
+    return STAG_OK;
+  }
   // k_cg_nrhs does not fold its predecessor's sums (each block holds every
   // system): a finalize kernel follows each CG kernel
   if (!c->fold || w.nrhs_sl) {
@@ -1401,6 +1492,7 @@ int solve_start(stag_ctx *c, const double masses[], int nmass, double tol, int m
     for (int i = 4; i < 8; ++i) hf[i] = 0;  // [4]: a bulk-copy wait in a CG kernel gave up
     CK(cudaMemcpyAsync(w.flags.p, hf, sizeof(int) * 8, cudaMemcpyHostToDevice, c->stream));
   }
+  if (w.ps_form) CK(cudaMemsetAsync(w.ps_sync.p, 0, ps_sync_bytes(nsys), c->stream));
   {
     const Ctl ctl0 = work_ctl(c, false);
     BlasArgs b = blas_base(c, ctl0);
@@ -1424,7 +1516,10 @@ int solve_eager(stag_ctx *c, int maxiter) {
   int *hf = (int *)w.h_flags.p;
   const int passes_per_poll = 4;  // the same sequence as the graph body, polled every 4 passes
   const int unroll = solve_unroll();
-  for (long long it = 0; it <= (long long)maxiter + 2 * unroll * passes_per_poll; it += unroll * passes_per_poll) {
+  // (a pass of the persistent kernel ends at the first update due, so their
+  // number is bounded by the pass counter alone)
+  for (long long it = 0; w.ps_form || it <= (long long)maxiter + 2 * unroll * passes_per_poll;
+       it += unroll * passes_per_poll) {
     for (int i = 0; i < passes_per_poll; ++i) {
       CKS(enqueue_pass(c, c->stream, ctl, unroll));
       CKS(enqueue_update(c, c->stream, ctl));
@@ -1465,7 +1560,7 @@ int solve_status(stag_ctx *c, int iters[], double true_res[]) {
   }
   cudaGetLastError();
   if (hf[4] != 0) {
-    c->err = "a CG kernel gave up waiting for its bulk-copied links; the solution is void";
+    c->err = "a CG kernel gave up waiting (for its bulk-copied links, or for the other blocks); the solution is void";
     return STAG_ERR_TIMEOUT;
   }
   int status = STAG_OK;
@@ -1926,8 +2021,26 @@ int ragged_impl(const stag_solve_desc *d, int n, double tol, int maxiter, int pr
       stag_ctx *c = c0;
       CK(cudaGraphCreate(&rg.graph, 0));
       int st = STAG_OK;
-      for (int i = 0; i < n && st == STAG_OK; ++i) {
-        st = add_solve_loop(d[i].ctx, rg.graph, nullptr, 0, nullptr);
+      // Every lattice's loop is a branch of its own, but persistent kernels, whose
+      // blocks wait for one another, run together only as far as the GPU holds
+      // all their blocks: in waves, from the smallest, each after the last.
+      std::vector<int> order(n);
+      for (int i = 0; i < n; ++i) order[i] = i;
+      std::stable_sort(order.begin(), order.end(),
+                       [&](int p, int q) { return d[p].ctx->w.ps_blocks < d[q].ctx->w.ps_blocks; });
+      std::vector<cudaGraphNode_t> before, wave;
+      int held = 0;
+      for (int q = 0; q < n && st == STAG_OK; ++q) {
+        const int i = order[q], nb = d[i].ctx->w.ps_form ? d[i].ctx->w.ps_blocks : 0;
+        if (nb > 0 && held > 0 && held + nb > c0->nsm) {
+          before.swap(wave);
+          wave.clear();
+          held = 0;
+        }
+        held += nb;
+        cudaGraphNode_t node = nullptr;
+        st = add_solve_loop(d[i].ctx, rg.graph, nb > 0 ? before.data() : nullptr, nb > 0 ? before.size() : 0, &node);
+        if (nb > 0) wave.push_back(node);
         if (st != STAG_OK) {
           cudaStreamCaptureStatus cs;
           cudaGraph_t tmp = nullptr;
@@ -2045,6 +2158,11 @@ int stag_create(const int dims[4], int flags, void *cuda_stream, stag_ctx **out)
   }
   const char *eager = getenv("STAG_EAGER");
   c->use_graph = !(eager && eager[0] == '1');
+  const char *ps = getenv("STAG_PS");
+  if (ps && ps[0] != 0) c->ps_mode = atoi(ps);
+  // a form forced for the two-kernel iteration
+  for (const char *v : {"STAG_TMA", "STAG_LANES", "STAG_NS", "STAG_MRHS", "STAG_NRHS", "STAG_FOLD", "STAG_PERSIST", "STAG_PDL"})
+    if (getenv(v)) c->ps_mode = 0;
   const char *fx = getenv("STAG_FX");
   c->fx_mode = !(fx && fx[0] == '0');
   const char *pdl = getenv("STAG_PDL");
@@ -2067,6 +2185,13 @@ int stag_create(const int dims[4], int flags, void *cuda_stream, stag_ctx **out)
     cudaGetLastError();
     delete c;
     return STAG_ERR_CUDA;
+  }
+  {
+    int v = 0;
+    c->coop = cudaDeviceGetAttribute(&v, cudaDevAttrCooperativeLaunch, c->device) == cudaSuccess && v != 0;
+    if (cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess || c->nsm < 1)
+      c->coop = false;
+    cudaGetLastError();
   }
   {
     // STAG_L2PERSIST = 0 off, 1 the links persist, 2 the Krylov vectors persist
@@ -2129,10 +2254,12 @@ int stag_links_upload(stag_ctx *c, const double *links) {
   CK(c->links64.ensure(cplx_bytes(P64) * 9ull * 8ull * c->Ve));
   // The FP64 copy, and with room for it the fixed-point copy; a field that is
   // not near unitary keeps the FP64 operator.
+  // (Below 128 sites a parity the FP64 form stays: a few warps' work, where the
+  // pipe does not matter.)
   const bool fx_was = c->fx_ok;
   int fx_bad = 1;
   c->fx_ok = false;
-  if (c->fx_mode && c->links_fx.ensure(cplx_bytes(PFX) * 9ull * 8ull * c->Ve) == cudaSuccess) {
+  if (c->fx_mode && c->Ve >= 128 && c->links_fx.ensure(cplx_bytes(PFX) * 9ull * 8ull * c->Ve) == cudaSuccess) {
     CK(c->defect.ensure(sizeof(unsigned long long)));
     CK(cudaMemsetAsync(c->defect.p, 0, sizeof(unsigned long long), c->stream));
     CK(launch_pack_links_fx(reinterpret_cast<const double2 *>(c->links_canon.p), (double2 *)c->links64.p,
@@ -2413,12 +2540,12 @@ int stag_solve_form(const stag_ctx *c, int out[8]) {
   const Work &w = c->w;
   out[0] = w.NS;
   out[1] = w.G;
-  out[2] = w.lanes_k1;
-  out[3] = w.lanes_k2;
+  out[2] = w.ps_form ? w.ps_form : w.lanes_k1;
+  out[3] = w.ps_form ? w.ps_form : w.lanes_k2;
   out[4] = w.tma;
   out[5] = w.l2p;
   out[6] = solve_unroll();
-  out[7] = w.mrhs ? 1 : (w.nrhs_sl == 24 ? 3 : (w.nrhs_sl ? 2 : 0));
+  out[7] = w.ps_form ? 4 : w.mrhs ? 1 : (w.nrhs_sl == 24 ? 3 : (w.nrhs_sl ? 2 : 0));
   if (w.nrhs_sl) {
     out[0] = w.nsys;  // every system in every block
     out[1] = 1;

@@ -103,6 +103,33 @@ unsigned cg_nrhs_smem(int recon, int form);
 int nrhs_kernel_form(int form, int EPI);
 constexpr int CG_NRHS_MAX = 64;
 
+// k_cg_persist (cg_persist.cu): the iterations of every running system up to its
+// next reliable update, in one cooperative launch of nblocks >= nsys blocks, a
+// group for each system; lanes = lanes a site (1, 2, 4).
+constexpr int PS_MAXB = 160;  // blocks of a group
+constexpr int PS_PER = PS_MAXB / 32;
+constexpr int PS_ASTRIDE = 32;  // words between two systems' arrival counters (a cache line)
+struct PsArgs {
+  Geom g;
+  const void *links;  // FP32 [2][4][NE][Ve]
+  VecArg r, p, t, x;
+  Ctl ctl;
+  unsigned long long *slots;  // [nsys][2][PS_MAXB] the blocks' sums of a half iteration, two FP32 a word
+  unsigned *arrived;          // [nsys][PS_ASTRIDE] arrivals counted (its first word), zero before a
+                              // solve's first launch
+  unsigned *counted;          // [nsys] arrivals at the end of the last launch, likewise
+  int *map;                   // [2 + nsys] running systems, blocks of each, which ones (k_ps_map)
+  int nsys;
+  int giveup;                 // 1: every wait gives up at once (the failure path run on purpose)
+  int nres;                   // set by the launcher: chunks whose links stay in shared memory
+  const void *l2_base;        // L2 access-policy window (host side), as DsArgs
+  size_t l2_bytes;
+  float l2_hit;
+};
+cudaError_t launch_cg_persist(int recon, int lanes, int nblocks, cudaStream_t st, PsArgs a,
+                              const void **kptr = nullptr);
+int cg_persist_sites(int lanes);  // sites of a block's warps at a time
+
 cudaError_t launch_accum_x(int RP, int NS, int nblocks, cudaStream_t st, const BlasArgs &a);
 // multi-shift CG (multishift.cu): the shifted-system update between the two CG
 // kernels (a.nbx blocks per base system), and the pending-update mark of a

@@ -521,8 +521,8 @@ class Context:
         return {"systems_per_thread": f[0], "groups": f[1], "lanes_k1": f[2], "lanes_k2": f[3],
                 "link_path": ("planes", "tiled_smem", "tiled")[f[4]], "l2_persisting_links": f[5] == 1,
                 "l2_persisting": ("none", "links", "vectors")[f[5]],
-                "iterations_per_pass": f[6], "shared_memory_links": bool(f[7]),
-                "kernels": ("k_dslash", "k_dslash_mrhs", "k_cg_nrhs", "k_cg_nrhs")[f[7]],
+                "iterations_per_pass": f[6], "shared_memory_links": f[7] in (1, 2, 3),
+                "kernels": ("k_dslash", "k_dslash_mrhs", "k_cg_nrhs", "k_cg_nrhs", "k_cg_persist")[f[7]],
                 "k1_systems_per_pass": 2 if f[7] == 3 else 1}
 
     def time_cg_kernel(self, kernel, precision=STAG_FP32, nlaunch=50):

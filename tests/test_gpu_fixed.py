@@ -114,3 +114,43 @@ def test_fields_that_are_not_unitary(how):
             if how != "large":
                 xs, _, _, _ = ctx.cg_solve([b] * 5, [0.3], tol=1e-10, precision=stag.STAG_FP64)
                 assert all(oracle.true_residual(L, field, 0.3, b, x) <= 1e-10 for x in xs)
+
+
+@pytest.mark.parametrize("case", ["far", "mixed_sites", "zero", "inf"])
+def test_npr_fields_off_the_integer_range(case):
+    """Hypercubes whose fields leave the integer form's exponent range contract in FP64 (1e-13 of the largest |O|,
+    both sides FP64); a non-finite field value stays in its hypercube."""
+    L = (4, 2, 6, 4)
+    V = synth.volume(L)
+    U = synth.random_links(L, 0.4, 741)
+    fs = [synth.gaussian_vector(V, 742 + k) for k in range(4)]
+    if case == "far":
+        fs = [f * s for f, s in zip(fs, (1e160, 1e-160, 1e140, 1e-150))]
+    elif case == "mixed_sites":  # neighbouring corners 10^30 apart
+        fs = [f * 10.0 ** np.random.default_rng(750 + k).uniform(-15, 15, (V, 1)) for k, f in enumerate(fs)]
+    elif case == "zero":
+        fs[2] = np.zeros_like(fs[2])
+    ref = oracle.npr_contract(L, U, 1, 2, 4, 7, *fs)
+    if case == "inf":
+        fs[1] = fs[1].copy()
+        fs[1][5, 2] = np.inf
+    with stag.Context(L) as ctx:
+        ctx.links_upload(U)
+        O, _ = ctx.npr_contract((1, 2, 4, 7), *fs)
+    if case == "inf":
+        bad = ~np.isfinite(O)
+        assert bad.sum() == 1 and np.abs(O - ref)[~bad].max() <= 1e-13 * np.abs(ref).max()
+    else:
+        assert np.abs(O - ref).max() <= 1e-13 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("alpha", [(0.9, 0.9, 0.9), (0.05, 0.6, 0.3), (0.75, 0.6, 0.0), (-0.2, 1.3, 0.3)])
+def test_hyp_parameters_on_both_forms(alpha):
+    """Mixes the fixed-point form holds, and those it leaves to FP64 (a weight near or below zero, or above one);
+    links within 1e-13 of the oracle's."""
+    L = (4, 2, 6, 8)
+    U = synth.random_links(L, 0.3, 761)
+    ref = oracle.hyp(L, U, alpha)
+    with stag.Context(L) as ctx:
+        H = ctx.hyp_smear(torch.from_numpy(U).cuda(), alpha).cpu().numpy()
+    assert np.abs(H - ref).max() <= 1e-13
