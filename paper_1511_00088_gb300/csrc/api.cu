@@ -805,8 +805,8 @@ size_t ps_sync_bytes(int nsys) {
   return (sizeof(unsigned long long) * 2 * PS_MAXB + sizeof(unsigned) * (PS_ASTRIDE + 2)) * (size_t)nsys + 2 * sizeof(int);
 }
 
-// The persistent form (k_cg_persist) of a workspace: lanes a site and blocks, or form 0 where the two-kernel forms are the better ones.  Measured on 152
-// SMs, us per iteration of a whole solve (persistent / two kernels):
+// The persistent form (k_cg_persist) of a workspace: lanes a site and blocks, or
+// form 0 where the two-kernel forms are the better ones.  Measured on 152 SMs, us per iteration of a whole solve (persistent / two kernels):
 //   lanes: 4 while a group's warps hold all sites at once (17 280 sites a parity: 4 lanes
 //   7.3, 2 lanes 8.2 / 17.8; 24 576: 9.0, 8.3 / 16.3); 2 while two rounds do (49 152: 2 lanes 11.7,
 //   1 lane 12.6 / 23.3; 98 304: 18.6, 17.1 / 28.0); else 1;
