@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(256) k_pack_links_fx(const double2 *__restrict
   const unsigned q1 = fast_div((unsigned)s, g.dLxh), q2 = fast_div(q1, g.dL1), q3 = fast_div(q2, g.dL2);
   const int par = (int)((lex & 1) + (q1 - q2 * g.L1) + (q2 - q3 * g.L2) + q3) & 1;
   const long long o = (long long)((par * 4 + mu) * 9) * g.Ve + s;
-  float row[3] = {0.f, 0.f, 0.f}, col[3] = {0.f, 0.f, 0.f};
+  float2 u[9];
   bool ok = true;
 #pragma unroll
   for (int e = 0; e < 9; ++e) {
@@ -276,13 +276,9 @@ __global__ void __launch_bounds__(256) k_pack_links_fx(const double2 *__restrict
     const Fx a = fx_link(hx, __double2loint(w.x)), b = fx_link(hy, __double2loint(w.y));
     const int4 f = make_int4(a.h, a.l, b.h, b.l);
     dstfx[o + (long long)e * g.Ve] = f;
-    const float x = (float)a.h * 0x1p-29f, y = (float)b.h * 0x1p-29f, n = x * x + y * y;
-    row[e / 3] += n;
-    col[e % 3] += n;
+    u[e] = make_float2((float)a.h * 0x1p-29f, (float)b.h * 0x1p-29f);
   }
-#pragma unroll
-  for (int k = 0; k < 3; ++k) ok = ok && fabsf(row[k] - 1.f) <= 1e-3f && fabsf(col[k] - 1.f) <= 1e-3f;
-  if (!ok) *bad = 1;
+  if (!ok || !near_unitary(u)) *bad = 1;
 }
 
 cudaError_t launch_pack_links_fx(const double2 *src, double2 *dst64, int4 *dstfx, Geom g, int *bad, cudaStream_t st) {

@@ -12,7 +12,7 @@
 // l l' is dropped (below 2^-59 a product, either sign).  The sums are exact; the
 // result hh + cr / 2^29 has an absolute error near 2^-57 of the largest factor,
 // a tenth of an FP64 FMA chain's, and becomes FP64 with one rounding.
-// Range, for a row of u of 2-norm^2 <= 2 (the fields allowed are within 1e-3 of 1) on 6 components
+// Range, for a row of u of 2-norm^2 <= 2 (near_unitary: within 1e-3 of 1) on 6 components
 // |v| <= 1, eight hops: by Cauchy-Schwarz |hh| <= 8 sqrt(12) 2^57 < 2^61.8 and
 // |cr| <= 8 (sqrt(12) 2^57 + 6 2^56) < 2^62.7.
 #pragma once
@@ -81,6 +81,29 @@ FX_HD void fx_mac(FxAcc &s, int ah, int al, int bh, int bl) {
 // the sum at the unit of hh
 FX_HD long long fx_sum(const FxAcc &s) {
   return s.hh + ((s.cr + (1ll << (FX_LO - 1))) >> FX_LO);
+}
+
+// Whether the rows of a 3 x 3 matrix are orthonormal to 1e-3, element by element
+// of u u^dag (false for NaN): then |u v| <= 1.0015 |v| for any v, and so for
+// products of such matrices.  Norms alone would not do: a matrix with all
+// elements 3^-1/2 has rows and columns of norm 1 and stretches by sqrt(3), which
+// took the limbs of the NPR contraction out of their 32 bits.
+FX_HD bool near_unitary(const float2 (&u)[9]) {
+  bool ok = true;
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = i; j < 3; ++j) {
+      float re = i == j ? -1.f : 0.f, im = 0.f;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const float2 a = u[3 * i + k], b = u[3 * j + k];
+        re += a.x * b.x + a.y * b.y;
+        im += a.y * b.x - a.x * b.y;
+      }
+      ok = ok && fabsf(re) <= 1e-3f && fabsf(im) <= 1e-3f;
+    }
+  return ok;
 }
 
 }  // namespace stag

@@ -442,7 +442,7 @@ __global__ void __launch_bounds__(256) k_hyp_fix(long long V, const double2 *__r
   const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
   if (t >= 4 * V) return;
   const long long mu = t / V, i = t - mu * V;
-  float row[3] = {0.f, 0.f, 0.f}, col[3] = {0.f, 0.f, 0.f};
+  float2 u[9];
   bool ok = true;
 #pragma unroll
   for (int e = 0; e < 9; ++e) {
@@ -451,13 +451,9 @@ __global__ void __launch_bounds__(256) k_hyp_fix(long long V, const double2 *__r
     ok = ok && (hx & 0x7fffffff) < 0x40000000 && (hy & 0x7fffffff) < 0x40000000;
     const Fx a = fx_link(hx, __double2loint(w.x)), b = fx_link(hy, __double2loint(w.y));
     F[(mu * 9 + e) * V + i] = make_int4(a.h, a.l, b.h, b.l);
-    const float x = (float)a.h * 0x1p-29f, y = (float)b.h * 0x1p-29f, n = x * x + y * y;
-    row[e / 3] += n;
-    col[e % 3] += n;
+    u[e] = make_float2((float)a.h * 0x1p-29f, (float)b.h * 0x1p-29f);
   }
-#pragma unroll
-  for (int k = 0; k < 3; ++k) ok = ok && fabsf(row[k] - 1.f) <= 1e-3f && fabsf(col[k] - 1.f) <= 1e-3f;
-  if (!ok) *bad = 1;
+  if (!ok || !near_unitary(u)) *bad = 1;
 }
 
 struct HypFx {

@@ -206,10 +206,12 @@ __global__ void __launch_bounds__(NPR_BT) k_npr(const NprArgs a) {
 // hypercube; 3.90 ms at 20^3 x 64, 1.24 ms here: issue slots 48 % and shared
 // memory 50 % busy, the levels' barriers between).  Here they are fixed-point sums (fixed.cuh): links and path
 // averages at 2^58, the fields at 2^57 under one exponent a field and
-// hypercube.  Ranges, rows and columns of a link being of norm 1 to 1e-3: an
-// element of a path product of up to 4 links is below 3 even for a field that
-// is not unitary (rank 1), so h < 2^31, and the sums of a level (4 steps of 3
-// products) stay below 2^62.3, as do those of the contraction.  FP64 is left for
+// hypercube.  Ranges, every link stretching a vector by at most 1.0015
+// (near_unitary): a path average W of up to 4 links by 1.006, so its elements
+// have |h| < 2^29.1, W y of a y with components |.| <= 1 has components below
+// 1.006 sqrt(6) 2^57, |h| < 2^29.4, and x . (W y) is below 6.1 2^56.  A sum of up
+// to 4 x 3 complex products has |hh| <= 4 x 1.006 2^58 and, its limbs at most
+// 2^29.4 and 2^28, |cr| <= 48 2^57.4 < 2^63.  FP64 is left for
 // the product of the two bilinears and the sum of the 256 terms.  A hypercube
 // whose fields hold numbers far from 1, infinities or NaNs contracts its path
 // averages in FP64 as k_npr does.

@@ -1598,9 +1598,8 @@ __global__ void k_pack_links(const double2 *__restrict__ src, void *dst, Geom g)
 }
 
 // the FP64 and the fixed-point copies of a gauge field in one pass over it;
-// *bad is set where a link is not near unitary (a row or column whose 2-norm^2
-// is off 1 by over 1e-3, a non-finite element): such a field's fixed-point
-// copy is not used
+// *bad is set where a link is not near unitary (near_unitary, |element| < 2):
+// such a field's fixed-point copy is not used
 __global__ void k_pack_links_fx(const double2 *__restrict__ src, double2 *__restrict__ dst64,
                                 int4 *__restrict__ dstfx, Geom g, int *bad);
 
