@@ -224,7 +224,7 @@ struct stag_ctx {
   size_t l2_max_persist = 0, l2_max_window = 0;
   DevBuf links_canon;  // [4][V][3][3] FP64, kept for lazy reduced-precision copies
   DevBuf links64;
-  DevBuf links_fx;     // fixed-point copy (fixed.cuh) of a near-unitary field, else unused
+  DevBuf links_fx;     // fixed-point copy (fixed.cuh) of a field it holds (fx_field), else unused
   bool fx_ok = false;  // the FP64 operator runs from links_fx
   bool fx_mode = true; // STAG_FX=0: never (the FP64 pipe's operator, for A/B runs)
   DevBuf links_lo[4][2];
@@ -330,7 +330,7 @@ int vec_out(stag_ctx *c, const VecBuf &v, int k, double *dst) {
 }
 
 // FP64 operator form of the uploaded field: PFX (integer-pipe products of the
-// fixed-point links) on near-unitary fields, P64 on any other field
+// fixed-point links) on near-unitary fields that mix (fx_field), P64 on any other
 int lp_for(const stag_ctx *c, int P) { return (P == P64 && c->fx_ok) ? PFX : P; }
 const void *links64_op(const stag_ctx *c) { return c->fx_ok ? c->links_fx.p : c->links64.p; }
 // launch_dslash with the FP64 form of this field
@@ -1080,6 +1080,7 @@ DsArgs ds_base(stag_ctx *c) {
   DsArgs a;
   memset(&a, 0, sizeof a);
   a.g = c->g;
+  a.canon = (const double2 *)c->links_canon.p;
   return a;
 }
 
@@ -2252,19 +2253,19 @@ int stag_links_upload(stag_ctx *c, const double *links) {
     }
   }
   CK(c->links64.ensure(cplx_bytes(P64) * 9ull * 8ull * c->Ve));
-  // The FP64 copy, and with room for it the fixed-point copy; a field that is
-  // not near unitary keeps the FP64 operator.
+  // The FP64 copy, and with room for it the fixed-point copy; a field that does
+  // not pass fx_field keeps the FP64 operator.
   // (Below 128 sites a parity the FP64 form stays: a few warps' work, where the
   // pipe does not matter.)
   const bool fx_was = c->fx_ok;
-  int fx_bad = 1;
+  FieldCheck check = {0, 1};
   c->fx_ok = false;
   if (c->fx_mode && c->Ve >= 128 && c->links_fx.ensure(cplx_bytes(PFX) * 9ull * 8ull * c->Ve) == cudaSuccess) {
-    CK(c->defect.ensure(sizeof(unsigned long long)));
-    CK(cudaMemsetAsync(c->defect.p, 0, sizeof(unsigned long long), c->stream));
+    CK(c->defect.ensure(sizeof(FieldCheck)));
+    CK(cudaMemsetAsync(c->defect.p, 0, sizeof(FieldCheck), c->stream));
     CK(launch_pack_links_fx(reinterpret_cast<const double2 *>(c->links_canon.p), (double2 *)c->links64.p,
-                            (int4 *)c->links_fx.p, c->g, (int *)c->defect.p, c->stream));
-    CK(cudaMemcpyAsync(&fx_bad, c->defect.p, sizeof fx_bad, cudaMemcpyDeviceToHost, c->stream));
+                            (int4 *)c->links_fx.p, c->g, (FieldCheck *)c->defect.p, c->stream));
+    CK(cudaMemcpyAsync(&check, c->defect.p, sizeof check, cudaMemcpyDeviceToHost, c->stream));
   } else {
     cudaGetLastError();
     CK(launch_pack_links(P64, 0, reinterpret_cast<const double2 *>(c->links_canon.p), c->links64.p, c->g,
@@ -2274,7 +2275,7 @@ int stag_links_upload(stag_ctx *c, const double *links) {
   c->have_links = true;
   c->w.drop_graph();  // the graph holds link pointers of the reduced-precision copies
   CK(cudaStreamSynchronize(c->stream));
-  c->fx_ok = fx_bad == 0;
+  c->fx_ok = fx_field(check, 4 * c->V);
   if (c->fx_ok != fx_was) c->w.nsys = 0;  // the FP64 launch forms were chosen for the other operator
   return STAG_OK;
 }

@@ -255,34 +255,38 @@ cudaError_t launch_pack_links(int LP, int recon, const double2 *src, void *dst, 
 // fixed-point split works on the FP64 bit patterns, as its conversions would
 // otherwise hold the FP64 pipe for longer than the copy takes.
 __global__ void __launch_bounds__(256) k_pack_links_fx(const double2 *__restrict__ src, double2 *__restrict__ dst64,
-                                                       int4 *__restrict__ dstfx, Geom g, int *bad) {
+                                                       int4 *__restrict__ dstfx, Geom g, FieldCheck *check) {
   const long long V = 2ll * g.Ve;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 4 * V) return;
-  const int mu = (int)(i / V);
-  const long long lex = i % V;
-  const int s = (int)(lex >> 1);
-  const unsigned q1 = fast_div((unsigned)s, g.dLxh), q2 = fast_div(q1, g.dL1), q3 = fast_div(q2, g.dL2);
-  const int par = (int)((lex & 1) + (q1 - q2 * g.L1) + (q2 - q3 * g.L2) + q3) & 1;
-  const long long o = (long long)((par * 4 + mu) * 9) * g.Ve + s;
-  float2 u[9];
   bool ok = true;
+  int nsmall = 0;
+  if (i < 4 * V) {
+    const int mu = (int)(i / V);
+    const long long lex = i % V;
+    const int s = (int)(lex >> 1);
+    const unsigned q1 = fast_div((unsigned)s, g.dLxh), q2 = fast_div(q1, g.dL1), q3 = fast_div(q2, g.dL2);
+    const int par = (int)((lex & 1) + (q1 - q2 * g.L1) + (q2 - q3 * g.L2) + q3) & 1;
+    const long long o = (long long)((par * 4 + mu) * 9) * g.Ve + s;
+    float2 u[9];
 #pragma unroll
-  for (int e = 0; e < 9; ++e) {
-    const double2 w = src[i * 9 + e];
-    dst64[o + (long long)e * g.Ve] = w;
-    const int hx = __double2hiint(w.x), hy = __double2hiint(w.y);
-    ok = ok && (hx & 0x7fffffff) < 0x40000000 && (hy & 0x7fffffff) < 0x40000000;  // |.| < 2 (false for NaN)
-    const Fx a = fx_link(hx, __double2loint(w.x)), b = fx_link(hy, __double2loint(w.y));
-    const int4 f = make_int4(a.h, a.l, b.h, b.l);
-    dstfx[o + (long long)e * g.Ve] = f;
-    u[e] = make_float2((float)a.h * 0x1p-29f, (float)b.h * 0x1p-29f);
+    for (int e = 0; e < 9; ++e) {
+      const double2 w = src[i * 9 + e];
+      dst64[o + (long long)e * g.Ve] = w;
+      const int hx = __double2hiint(w.x), hy = __double2hiint(w.y);
+      ok = ok && (hx & 0x7fffffff) < 0x40000000 && (hy & 0x7fffffff) < 0x40000000;  // |.| < 2 (false for NaN)
+      const Fx a = fx_link(hx, __double2loint(w.x)), b = fx_link(hy, __double2loint(w.y));
+      dstfx[o + (long long)e * g.Ve] = make_int4(a.h, a.l, b.h, b.l);
+      u[e] = make_float2((float)a.h * 0x1p-29f, (float)b.h * 0x1p-29f);
+    }
+    ok = ok && near_unitary(u);
+    nsmall = small_parts(u);
   }
-  if (!ok || !near_unitary(u)) *bad = 1;
+  check_link(check, ok, nsmall);
 }
 
-cudaError_t launch_pack_links_fx(const double2 *src, double2 *dst64, int4 *dstfx, Geom g, int *bad, cudaStream_t st) {
-  k_pack_links_fx<<<nblk(8ll * g.Ve, 256), 256, 0, st>>>(src, dst64, dstfx, g, bad);
+cudaError_t launch_pack_links_fx(const double2 *src, double2 *dst64, int4 *dstfx, Geom g, FieldCheck *check,
+                                 cudaStream_t st) {
+  k_pack_links_fx<<<nblk(8ll * g.Ve, 256), 256, 0, st>>>(src, dst64, dstfx, g, check);
   return cudaGetLastError();
 }
 

@@ -18,8 +18,20 @@
 // the vectors, 178 us in this form, 149 us with the caller's layout read and
 // written directly (abi_in, abi_center, abi_out); FP64 CG iteration on 16^3 x 32:
 // 115 us before, 50 us.
-// A thread whose neighbours hold an infinity, a NaN or only numbers near the
-// ends of the exponent range sums its hops on FP64 FMAs instead.
+// The error of such a sum is absolute: up to 11.4 units of 2^-57 of a direction's
+// scale 2^E, the power of two above its largest neighbour component (neighbours truncated
+// 4.9, links rounded 3, l l' dropped 3, rounding 1/2), so up to 50 of the site's with the
+// alignment.  A component made of products far below the scale alone (colours of
+// very different sizes that these links do not mix) would lose bits that FP64
+// keeps.  So one of its four direction sums or their forward halves, each a lower
+// bound of m, the sum of its 48 products' magnitudes, has to reach 2^-5 of the scale:
+// then it errs by at most 99 x 2^-53 m, where 48 FMAs may err by 48 x 2^-53 m (typically
+// by five times as much as this).  Else the thread sums the component on FP64 FMAs
+// from the FP64 links, as it does next to an infinity, a NaN or numbers near the
+// ends of the exponent range.  That branch costs its block some 5 us.  On links exp(i c H),
+// c = 0.1 ... 0.4, and Gaussian vectors less than 1e-6 of the components take it (a line
+// at 2^-4: 5e-6; the direction sums alone, at 2^-5: 4e-5, which made the FP64 CG on
+// 16^3 x 32 a quarter slower).
 #include "launch.h"
 
 namespace stag {
@@ -27,34 +39,56 @@ namespace stag {
 namespace {
 
 constexpr int FXB = 128;        // threads: 4 directions x 32 sites
-constexpr int FX_FP64 = -1;     // exponent mark of a partial sum held as FP64
-constexpr int FX_E0 = 64;       // smallest exponent field of the integer form (and that of a zero sum)
-constexpr int FX_E1 = 2030;     // the largest
+constexpr int FX_ZERO = 0;        // exponent mark of a direction whose neighbours are zero
+constexpr int FX_FP64 = 1 << 16;  // and of one that the integer form does not hold
+constexpr int FX_E0 = 64;         // smallest exponent field of the integer form
+constexpr int FX_E1 = 2030;       // the largest
+constexpr int FX_LINE = 1 << 20;  // 2^-5 of the scale, in the high word of a sum
 
-__device__ __forceinline__ double fx_value(int h, int l) {
-  return __fma_rn((double)h, 0x1p-29, (double)l * 0x1p-58);
-}
-
-// the two hops of one direction on FP64 FMAs
-__device__ __noinline__ void hops_fp64(const int4 *uf, const int4 *ub, const double2 *vf, const double2 *vb, int Ve,
-                                       long long cs, unsigned flipf, unsigned flipb, double *out) {
-  double acc[6] = {0, 0, 0, 0, 0, 0};
+// row `col` of D in at site s of parity P on FP64 FMAs, `in` with strides is, ic
+__device__ __noinline__ double2 row_fp64(const Geom &g, const double2 *canon, const double2 *in, long long is,
+                                         long long ic, int P, int s, int col) {
+  int x[4];
+  site_coords(g, P, s, x);
+  const long long V = 2ll * g.Ve;
+  const long long lex = x[0] + (long long)g.L0 * (x[1] + (long long)g.L1 * (x[2] + (long long)g.L2 * x[3]));
+  double2 acc = make_double2(0.0, 0.0);
+  int eb = 0;
+  long long str = 1;
 #pragma unroll 1
-  for (int q = 0; q < 2; ++q) {
-    const int4 *L = q ? ub : uf;
-    const double2 *in = q ? vb : vf;
-    const double sg = (q ? flipb : flipf) ? -1.0 : 1.0;
-    for (int b = 0; b < 3; ++b) {
-      const double2 v = __ldg(in + b * cs);
-      for (int a = 0; a < 3; ++a) {
-        const int4 w = __ldg(L + (long long)(q ? 3 * b + a : 3 * a + b) * Ve);
-        const double ur = sg * fx_value(w.x, w.y), ui = (q ? -sg : sg) * fx_value(w.z, w.w);
-        acc[2 * a] += ur * v.x - ui * v.y;
-        acc[2 * a + 1] += ur * v.y + ui * v.x;
-      }
+  for (int mu = 0; mu < 4; ++mu) {
+    const int L = mu == 0 ? g.L0 : mu == 1 ? g.L1 : mu == 2 ? g.L2 : g.L3;
+    const int xm = mu == 0 ? x[0] : mu == 1 ? x[1] : mu == 2 ? x[2] : x[3];
+    const int xp = (xm + 1 == L) ? 0 : xm + 1, xn = (xm == 0) ? L - 1 : xm - 1;
+    const int sf = cb_of(g, mu == 0 ? xp : x[0], mu == 1 ? xp : x[1], mu == 2 ? xp : x[2], mu == 3 ? xp : x[3]);
+    const int sb = cb_of(g, mu == 0 ? xn : x[0], mu == 1 ? xn : x[1], mu == 2 ? xn : x[2], mu == 3 ? xn : x[3]);
+    const double2 *uf = canon + (mu * V + lex) * 9 + 3 * col;
+    const double2 *ub = canon + (mu * V + lex + (xn - xm) * str) * 9 + col;
+    double2 f[3], b[3], vf[3], vb[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      f[k] = __ldg(uf + k);
+      b[k] = __ldg(ub + 3 * k);
+      vf[k] = __ldg(in + k * ic + sf * is);
+      vb[k] = __ldg(in + k * ic + sb * is);
     }
+    double gf = (eb & 1) ? -1.0 : 1.0, gb = -gf;  // backward hops enter with a minus
+    if (mu == 3 && g.ap) {
+      if (xm == g.L3 - 1) gf = -gf;
+      if (xm == 0) gb = -gb;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const double fr = gf * f[k].x, fi = gf * f[k].y, br = gb * b[k].x, bi = gb * b[k].y;
+      acc.x = __fma_rn(-fi, vf[k].y, __fma_rn(fr, vf[k].x, acc.x));
+      acc.y = __fma_rn(fi, vf[k].x, __fma_rn(fr, vf[k].y, acc.y));
+      acc.x = __fma_rn(bi, vb[k].y, __fma_rn(br, vb[k].x, acc.x));
+      acc.y = __fma_rn(-bi, vb[k].x, __fma_rn(br, vb[k].y, acc.y));
+    }
+    eb += xm;
+    str *= L;
   }
-  for (int i = 0; i < 6; ++i) out[i] = acc[i];
+  return acc;
 }
 
 // Blocks an SM: 4 (128 registers) for the plain operator, 3 (168) for the CG
@@ -67,6 +101,7 @@ __global__ void __launch_bounds__(FXB, (EPI == EPI_PLAIN || EPI == EPI_MDAGM) ? 
   constexpr int NV = (EPI == EPI_CG_K2 || EPI == EPI_RESID) ? 2 : 1;
   constexpr bool REDUCES = EPI == EPI_CG_K1R || EPI == EPI_CG_K2 || EPI == EPI_RESID;
   __shared__ long long part_t[2][4][6][32];
+  __shared__ int2 part_f[2][4][3][32];  // high words of the forward hop's sums
   __shared__ int part_e[2][4][32];
   const Geom g = a.g;
   const int Ve = g.Ve, P = a.par_out, G = a.ngroups;
@@ -167,16 +202,10 @@ __global__ void __launch_bounds__(FXB, (EPI == EPI_PLAIN || EPI == EPI_MDAGM) ? 
             any |= __double2loint(wf[c].x) | __double2loint(wf[c].y) | __double2loint(wb[c].x) | __double2loint(wb[c].y);
           zero = any == 0;
         }
-        if (zero) {
-          E = FX_E0;
+        if (zero || E < FX_E0 || E > FX_E1) {
+          E = zero ? FX_ZERO : FX_FP64;
 #pragma unroll
           for (int i = 0; i < 6; ++i) T[i] = 0;
-        } else if (E < FX_E0 || E > FX_E1) {
-          E = FX_FP64;
-          double d[6];
-          hops_fp64(uf, ub, in + sf * is, in + sb * is, Ve, ic, ff, fb, d);
-#pragma unroll
-          for (int i = 0; i < 6; ++i) T[i] = __double_as_longlong(d[i]);
         } else {
           FxAcc sum[6];
 #pragma unroll
@@ -194,6 +223,9 @@ __global__ void __launch_bounds__(FXB, (EPI == EPI_PLAIN || EPI == EPI_MDAGM) ? 
               fx_mac(sum[2 * k + 1], u.z, u.w, r.h, r.l);
             }
           }
+#pragma unroll
+          for (int k = 0; k < 3; ++k)
+            part_f[buf][mu][k][lane] = make_int2((int)(sum[2 * k].hh >> 32), (int)(sum[2 * k + 1].hh >> 32));
 #pragma unroll
           for (int b = 0; b < 3; ++b) {  // (ur - i ui)(r + i m)
             const Fx r = fx_vec(__double2hiint(wb[b].x) ^ (int)fb, __double2loint(wb[b].x), E);
@@ -218,40 +250,40 @@ __global__ void __launch_bounds__(FXB, (EPI == EPI_PLAIN || EPI == EPI_MDAGM) ? 
       // barrier follows every read of this one
       __syncthreads();
       if (epi) {
-        int E = FX_E0;
-        bool f64 = false;
+        int E = FX_ZERO;
 #pragma unroll
-        for (int d = 0; d < 4; ++d) {
-          const int e = part_e[buf][d][lane];
-          f64 |= e == FX_FP64;
-          E = max(E, e);
-        }
-        double2 v;
-        if (!f64) {
+        for (int d = 0; d < 4; ++d) E = max(E, part_e[buf][d][lane]);
+        double2 v = make_double2(0.0, 0.0);
+        if (E != FX_ZERO) {
           long long re = 0, im = 0;
+          int seen_re = 0, seen_im = 0;  // bits of the direction sums' magnitudes
 #pragma unroll
           for (int d = 0; d < 4; ++d) {
             const int sh = min(E - part_e[buf][d][lane], 63);
-            re += part_t[buf][d][2 * mu][lane] >> sh;
-            im += part_t[buf][d][2 * mu + 1][lane] >> sh;
+            const long long a_re = part_t[buf][d][2 * mu][lane] >> sh, a_im = part_t[buf][d][2 * mu + 1][lane] >> sh;
+            const int h_re = (int)(a_re >> 32), h_im = (int)(a_im >> 32);
+            seen_re |= h_re ^ (h_re >> 31);
+            seen_im |= h_im ^ (h_im >> 31);
+            re += a_re;
+            im += a_im;
           }
-          // unit 2^(E - 1022 - 57): its exponent field stays in 1 .. 2046
-          const double unit = __hiloint2double((E - 1022 - FX_VBITS + 1023) << 20, 0);
-          v = make_double2((double)re * unit, (double)im * unit);
-        } else {
-          v = make_double2(0.0, 0.0);
+          bool f64 = E == FX_FP64;
+          if (seen_re < FX_LINE || seen_im < FX_LINE) {  // then those of their forward halves
 #pragma unroll 1
-          for (int d = 0; d < 4; ++d) {
-            const int e = part_e[buf][d][lane];
-            const long long re = part_t[buf][d][2 * mu][lane], im = part_t[buf][d][2 * mu + 1][lane];
-            if (e == FX_FP64) {
-              v.x += __longlong_as_double(re);
-              v.y += __longlong_as_double(im);
-            } else {
-              const double unit = __hiloint2double((e - 1022 - FX_VBITS + 1023) << 20, 0);
-              v.x += (double)re * unit;
-              v.y += (double)im * unit;
+            for (int d = 0; d < 4; ++d) {
+              const int2 f = part_f[buf][d][mu][lane];  // (unset where the direction is zero: shifted out)
+              const int sh = min(E - part_e[buf][d][lane], 31), f_re = f.x >> sh, f_im = f.y >> sh;
+              seen_re |= f_re ^ (f_re >> 31);
+              seen_im |= f_im ^ (f_im >> 31);
             }
+            f64 |= seen_re < FX_LINE || seen_im < FX_LINE;
+          }
+          if (f64) {
+            v = row_fp64(g, a.canon, in, is, ic, P, s, mu);
+          } else {
+            // unit 2^(E - 1022 - 57): its exponent field stays in 1 .. 2046
+            const double unit = __hiloint2double((E - 1022 - FX_VBITS + 1023) << 20, 0);
+            v = make_double2((double)re * unit, (double)im * unit);
           }
         }
         if (EPI == EPI_CG_K2) {

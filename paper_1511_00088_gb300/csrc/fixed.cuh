@@ -11,7 +11,12 @@
 //   hh += h h'  (unit 2^-57),   cr += h l' + l h'  (unit 2^-86);
 // l l' is dropped (below 2^-59 a product, either sign).  The sums are exact; the
 // result hh + cr / 2^29 has an absolute error near 2^-57 of the largest factor,
-// a tenth of an FP64 FMA chain's, and becomes FP64 with one rounding.
+// a tenth of an FP64 FMA chain's, and becomes FP64 with one rounding.  That error
+// is absolute: where a sum's own products are all far below the largest factor
+// (components of very different sizes that the links do not mix), it would lose
+// bits that FP64 keeps.  So every user tests its sums or products and leaves
+// such ones to FP64, and fields whose links mix too little (FX_SMALL below) run
+// on FP64 altogether.
 // Range, for a row of u of 2-norm^2 <= 2 (near_unitary: within 1e-3 of 1) on 6 components
 // |v| <= 1, eight hops: by Cauchy-Schwarz |hh| <= 8 sqrt(12) 2^57 < 2^61.8 and
 // |cr| <= 8 (sqrt(12) 2^57 + 6 2^56) < 2^62.7.
@@ -40,14 +45,16 @@ FX_HD Fx fx_split(long long V) {
 }
 
 // the FP64 number (hi, lo) as (mantissa << UP) >> (E - its exponent field),
-// E >= that field; the bits shifted out are dropped, and zeros and denormals
-// become 0 where E >= 64
-template <int UP>
+// E >= that field; the bits shifted out are dropped, or rounded (magnitudes,
+// halves up), and zeros and denormals become 0 where E >= 64
+template <int UP, bool ROUND>
 FX_HD Fx fx_from(int hi, int lo, int E) {
   int sh = E - ((hi >> 20) & 0x7ff);
   sh = sh < 63 ? sh : 63;
   unsigned long long m = ((unsigned long long)(unsigned)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)lo;
-  m = (m << UP) >> sh;
+  m <<= UP;
+  if (ROUND) m += (1ull << sh) >> 1;
+  m >>= sh;
   const Fx a = fx_split((long long)m);
   const int s = (hi >> 31) | 1;
   Fx f;
@@ -56,9 +63,9 @@ FX_HD Fx fx_from(int hi, int lo, int E) {
   return f;
 }
 // a link element, |u| < 2: u 2^58
-FX_HD Fx fx_link(int hi, int lo) { return fx_from<6>(hi, lo, 1023); }
+FX_HD Fx fx_link(int hi, int lo) { return fx_from<6, true>(hi, lo, 1023); }
 // a vector element scaled by 2^(1022 - E), E >= the exponent fields of its site: v 2^57
-FX_HD Fx fx_vec(int hi, int lo, int E) { return fx_from<4>(hi, lo, E); }
+FX_HD Fx fx_vec(int hi, int lo, int E) { return fx_from<4, false>(hi, lo, E); }
 
 // sums of products
 struct FxAcc {
@@ -105,5 +112,35 @@ FX_HD bool near_unitary(const float2 (&u)[9]) {
     }
   return ok;
 }
+
+// A field's links mix the colours, and real with imaginary parts, if few of
+// their real components are small.  With over an eighth below 2^-6 (unit,
+// diagonal, real or nearly such links) the sums of the operator would be left
+// to FP64 one by one too often, and the FP64 forms run from the start.  Links
+// exp(i c H): 3 % below at c = 0.4 and for Haar matrices, 11 % at c = 0.1.
+constexpr float FX_SMALL = 0x1p-6f;
+FX_HD int small_parts(const float2 (&u)[9]) {
+  int n = 0;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) n += (fabsf(u[k].x) < FX_SMALL) + (fabsf(u[k].y) < FX_SMALL);
+  return n;
+}
+// what a conversion found out about the nlinks links of its field
+struct FieldCheck {
+  unsigned long long small;  // real components below FX_SMALL
+  int bad;                   // a link is not near unitary
+};
+FX_HD bool fx_field(const FieldCheck &f, long long nlinks) {
+  return f.bad == 0 && 8 * f.small <= 18 * (unsigned long long)nlinks;
+}
+
+#ifdef __CUDACC__
+// one thread's link (ok: it is near unitary) into the check, all threads of a block together
+__device__ __forceinline__ void check_link(FieldCheck *f, bool ok, int nsmall) {
+  if (!ok) f->bad = 1;
+  const int n = __reduce_add_sync(0xffffffffu, nsmall);
+  if ((threadIdx.x & 31) == 0 && n > 0) atomicAdd(&f->small, (unsigned long long)n);
+}
+#endif
 
 }  // namespace stag

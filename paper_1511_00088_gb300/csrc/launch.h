@@ -152,9 +152,9 @@ cudaError_t launch_convert_vec(int PIN, int POUT, VecArg src, VecArg dst, int ns
                                cudaStream_t st);
 cudaError_t launch_pack_links(int LP, int recon, const double2 *src, void *dst, Geom g,
                               cudaStream_t st);
-// the FP64 (dst64) and fixed-point (dstfx) copies; *bad (device) set to 1 when
-// the field is not near unitary
-cudaError_t launch_pack_links_fx(const double2 *src, double2 *dst64, int4 *dstfx, Geom g, int *bad, cudaStream_t st);
+// the FP64 (dst64) and fixed-point (dstfx) copies; *check (device) zeroed before
+cudaError_t launch_pack_links_fx(const double2 *src, double2 *dst64, int4 *dstfx, Geom g, FieldCheck *check,
+                                 cudaStream_t st);
 // the tiled site-owned copy (LP = P32, P16 or PBF); dst already zeroed
 cudaError_t launch_pack_links_tiled(int LP, int recon, const double2 *src, void *dst, Geom g, int ntile,
                                     cudaStream_t st);
@@ -164,7 +164,7 @@ cudaError_t launch_su3_defect(const double2 *U, long long nlinks, unsigned long 
 // NPR one-colour-trace four-fermion contraction (npr.cu): out[h] = O(z_h) for
 // every hypercube (V / 16 entries), *sum (may be null) = their sum; U the
 // canonical [4][V][3][3] links, fields [V][3]; st = (S1, F1, S2, F2), 4-bit
-// corner masks; fx: the links are near unitary (stag_ctx::fx_ok), so the integer form runs
+// corner masks; fx: the integer form runs (stag_ctx::fx_ok)
 cudaError_t launch_npr(const int dims[4], const double2 *U, const int st[4], const double2 *cb1, const double2 *c2,
                        const double2 *cb3, const double2 *c4, double2 *out, double2 *sum, bool fx, cudaStream_t s);
 

@@ -132,6 +132,7 @@ struct DsArgs {
   // (a caller's buffer) instead of [3][Ve]
   int abi_in, abi_center, abi_out;
   const void *links;     // [2][4][NE][Ve] of the link storage type
+  const double2 *canon;  // the FP64 links [4][V][3][3] (k_dslash_fx, sums left to FP64)
   VecArg in;             // input on the other parity (EPI_CG_K1: p_old)
   VecArg center;         // EPI_MDAGM: the vector the mass term multiplies; EPI_RESID: x;
                          // EPI_CG_K2: p (read p_old, written p_new)
@@ -1597,11 +1598,10 @@ __global__ void k_pack_links(const double2 *__restrict__ src, void *dst, Geom g)
   }
 }
 
-// the FP64 and the fixed-point copies of a gauge field in one pass over it;
-// *bad is set where a link is not near unitary (near_unitary, |element| < 2):
-// such a field's fixed-point copy is not used
+// the FP64 and the fixed-point copies of a gauge field in one pass over it, and
+// what decides whether the latter is used (fx_field)
 __global__ void k_pack_links_fx(const double2 *__restrict__ src, double2 *__restrict__ dst64,
-                                int4 *__restrict__ dstfx, Geom g, int *bad);
+                                int4 *__restrict__ dstfx, Geom g, FieldCheck *check);
 
 // tiled site-owned copy of the links (see the layout notes at the top): one
 // thread per (parity, site, slot); dst zeroed beforehand (the tail of the last
