@@ -92,11 +92,10 @@ struct NprArgs {
   double2 *out;      // [nhyp]
 };
 
-__global__ void __launch_bounds__(NPR_BT) k_npr(const NprArgs a) {
-  __shared__ double2 W[256][9];      // W(A, D), index A * 16 + D, both orientations
-  __shared__ double2 fld[4][16][3];  // chibar1, chi2, chibar3, chi4 at the corners
-  __shared__ double2 red[NPR_BT / 32];
-  __shared__ unsigned char pa[120], pd[120];
+// this block's hypercube; W(A, D) at index A * 16 + D, both orientations; fld:
+// chibar1, chi2, chibar3, chi4 at the corners; red: a value a warp
+__device__ __forceinline__ void npr_fp64(const NprArgs &a, double2 (*W)[9], double2 (*fld)[16][3], double2 *red,
+                                         unsigned char *pa, unsigned char *pd) {
   const long long h = blockIdx.x;
   int zc[4];
   {
@@ -199,34 +198,108 @@ __global__ void __launch_bounds__(NPR_BT) k_npr(const NprArgs a) {
   }
 }
 
+__global__ void __launch_bounds__(NPR_BT) k_npr(const NprArgs a) {
+  __shared__ double2 W[256][9];
+  __shared__ double2 fld[4][16][3];
+  __shared__ double2 red[NPR_BT / 32];
+  __shared__ unsigned char pa[120], pd[120];
+  npr_fp64(a, W, fld, red, pa, pd);
+}
+
 // ---------------------------------------------------------------------------
-// the same contraction on the integer pipe (near-unitary fields)
+// the same contraction on the integer pipe (fields that pass fx_field)
 // ---------------------------------------------------------------------------
 // k_npr keeps the FP64 pipe 95 % busy (12 000 complex multiply-adds a
-// hypercube; 3.90 ms at 20^3 x 64, 1.24 ms here: issue slots 48 % and shared
-// memory 50 % busy, the levels' barriers between).  Here they are fixed-point sums (fixed.cuh): links and path
-// averages at 2^58, the fields at 2^57 under one exponent a field and
-// hypercube.  Ranges, every link stretching a vector by at most 1.0015
-// (near_unitary): a path average W of up to 4 links by 1.006, so its elements
-// have |h| < 2^29.1, W y of a y with components |.| <= 1 has components below
-// 1.006 sqrt(6) 2^57, |h| < 2^29.4, and x . (W y) is below 6.1 2^56.  A sum of up
-// to 4 x 3 complex products has |hh| <= 4 x 1.006 2^58 and, its limbs at most
-// 2^29.4 and 2^28, |cr| <= 48 2^57.4 < 2^63.  FP64 is left for
-// the product of the two bilinears and the sum of the 256 terms.  A hypercube
-// whose fields hold numbers far from 1, infinities or NaNs contracts its path
-// averages in FP64 as k_npr does.
+// hypercube; 3.90 ms at 20^3 x 64, 1.30 ms here: issue slots 48 % and shared
+// memory 50 % busy, the levels' barriers between).  Here they are fixed-point
+// sums (fixed.cuh): links and path averages at 2^58, a field at 2^57 under one
+// exponent a corner (its 3 colours).  FP64 is left for the product of the two
+// bilinears and the sum of the 256 terms.
+// Ranges, every link stretching a vector by at most 1.0015 (near_unitary): a path
+// average W of up to 4 links by 1.006, so its elements have |h| < 2^29.1, W y of a
+// y with components |.| <= 1 has components below 1.006 sqrt(6) 2^57, |h| < 2^29.4,
+// and x . (W y) is below 6.1 2^56.  A sum of up to 4 x 3 complex products has |hh|
+// <= 4 x 1.006 2^58 and, its limbs at most 2^29.1 and 2^28, |cr| <= 48 2^57.1 < 2^63.
+// Errors are fractions of the corners' scales: a bilinear x W y errs by up to
+// 45 x 2^-57 of their product.  What FP64 would keep beyond that stays in FP64:
+//   * corners 0 or 1 step apart, where single elements of W decide: a bilinear
+//     with a real or imaginary part whose terms' magnitudes sum to less than 2^-5
+//     is formed in FP64 from the FP64 link; the others err by at most 90 x 2^-53 of those
+//     magnitudes.  Three partial sums, each a lower bound, spare most the count: with Gaussian
+//     fields 9 % of the warps take it, 1e-5 of the threads FP64.  (Two and more
+//     steps average two and more paths of three terms each: no small W from mixing
+//     links.)
+//   * a hypercube with over an eighth of its links' real components below FX_SMALL,
+//     as in a cold region of a rough field, or whose fields hold numbers far from 1,
+//     infinities or NaNs at a corner: all of it, as k_npr does.
+
 // v / n, n = 2, 3, 4
 __device__ __forceinline__ long long fx_over(long long v, int n) {
   return n == 2 ? v >> 1 : n == 4 ? v >> 2 : fx_third(v);
 }
 
 constexpr int NPR_E0 = 600, NPR_E1 = 1400;  // exponent fields of the integer form
+constexpr int NPR_LINE = 1 << 19;           // 2^-5 of the scales, in the high word of a bilinear (unit 2^-56)
 
-__global__ void __launch_bounds__(NPR_BT, 4) k_npr_fx(const NprArgs a) {
-  __shared__ int4 W[256][9];      // as k_npr, fixed-point
+// the whole hypercube in FP64 (out of line: the kernel's registers are the integer form's)
+__device__ __noinline__ void npr_block_fp64(const NprArgs &a, double2 (*W)[9], double2 (*fld)[16][3], double2 *red,
+                                            unsigned char *pa, unsigned char *pd) {
+  npr_fp64(a, W, fld, red, pa, pd);
+}
+
+// whether the terms of x^T W y sum to less than 2^-5 in magnitude, in its real or in its imaginary part
+__device__ __forceinline__ bool terms_small(const int4 *x, const int4 *w, const int4 *y) {
+  float re = 0.f, im = 0.f;
+  for (int i = 0; i < 3; ++i) {
+    float vr = 0.f, vi = 0.f;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const float wr = fabsf((float)w[3 * i + j].x), wi = fabsf((float)w[3 * i + j].z);
+      const float yr = fabsf((float)y[j].x), yi = fabsf((float)y[j].z);
+      vr += wr * yr + wi * yi;
+      vi += wr * yi + wi * yr;
+    }
+    const float xr = fabsf((float)x[i].x), xi = fabsf((float)x[i].z);
+    re += xr * vr + xi * vi;
+    im += xr * vi + xi * vr;
+  }
+  return fminf(re, im) < 0x1p80f;  // units of 2^-28, 2^-29 and 2^-28
+}
+
+// b, or, where its terms are small, x^T W y in FP64: W = 1 (u null), the link u or (dag) its adjoint;
+// xs, ys the corners' colours, x, w, y the fixed-point ones
+__device__ __noinline__ double2 bilinear_checked(double2 b, const int4 *x, const int4 *w, const int4 *y,
+                                                 const double2 *xs, const double2 *ys, const double2 *u, bool dag) {
+  if (!terms_small(x, w, y)) return b;
+  double2 sum = make_double2(0.0, 0.0);
+  double2 v[3], f[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    v[k] = __ldg(ys + k);
+    f[k] = __ldg(xs + k);
+  }
+  for (int i = 0; i < 3; ++i) {
+    double2 l = v[i];
+    if (u != nullptr) {
+      double2 s = make_double2(0.0, 0.0);
+      for (int j = 0; j < 3; ++j) {
+        l = __ldg(u + (dag ? 3 * j + i : 3 * i + j));
+        if (dag) l.y = -l.y;
+        s = zfma(l, v[j], s);
+      }
+      l = s;
+    }
+    sum = zfma(f[i], l, sum);
+  }
+  return sum;
+}
+
+__global__ void __launch_bounds__(NPR_BT, 4) k_npr_fx(const __grid_constant__ NprArgs a) {
+  __shared__ int4 W[256][9];      // as npr_fp64, fixed-point
   __shared__ int4 fld[4][16][3];  // the fields at the corners, fixed-point
   __shared__ double2 term[NPR_BT];
-  __shared__ int top[4];  // largest exponent bits of a field
+  __shared__ int top[4][16];  // largest exponent bits of a field at a corner, 0 where it is zero
+  __shared__ int nsmall;      // real components of the links below FX_SMALL
   __shared__ unsigned char pa[120], pd[120];
   const long long h = blockIdx.x;
   int zc[4];
@@ -249,7 +322,9 @@ __global__ void __launch_bounds__(NPR_BT, 4) k_npr_fx(const NprArgs a) {
   const double2 *fsrc = ff == 0 ? a.cb1 : ff == 1 ? a.c2 : ff == 2 ? a.cb3 : a.c4;
   double2 fv = make_double2(0.0, 0.0);
   if (t < 192) fv = fsrc[site(fa) * 3 + fc];
-  if (t < 4) top[t] = 0;
+  if (t < 64) (&top[0][0])[t] = 0;
+  if (t == 64) nsmall = 0;
+  int small = 0;
   for (int k = t; k < 32 * 9; k += NPR_BT) {
     const int l = k / 9, e = k % 9, mu = l / 8, y = l % 8;
     const int A = ((y >> mu) << (mu + 1)) | (y & ((1 << mu) - 1)), D = A | (1 << mu);
@@ -257,6 +332,7 @@ __global__ void __launch_bounds__(NPR_BT, 4) k_npr_fx(const NprArgs a) {
     const Fx re = fx_link(__double2hiint(u.x), __double2loint(u.x));
     const Fx im = fx_link(__double2hiint(u.y), __double2loint(u.y));
     const int4 w = make_int4(re.h, re.l, im.h, im.l);
+    small += (abs(re.h) < (int)(FX_SMALL * 0x1p29f)) + (abs(im.h) < (int)(FX_SMALL * 0x1p29f));
     W[A * 16 + D][e] = w;
     W[D * 16 + A][(e % 3) * 3 + e / 3] = fx_conj(w);
   }
@@ -269,7 +345,14 @@ __global__ void __launch_bounds__(NPR_BT, 4) k_npr_fx(const NprArgs a) {
     pd[t] = c_pairs.d[t];
   }
   __syncthreads();
-  if (t < 192) atomicMax(&top[ff], max(__double2hiint(fv.x) & 0x7fffffff, __double2hiint(fv.y) & 0x7fffffff));
+  small = __reduce_add_sync(0xffffffffu, small);
+  if ((t & 31) == 0 && small > 0) atomicAdd(&nsmall, small);
+  if (t < 192) {
+    int hi = max(__double2hiint(fv.x) & 0x7fffffff, __double2hiint(fv.y) & 0x7fffffff);
+    if (hi == 0 && (__double2loint(fv.x) | __double2loint(fv.y)) != 0) hi = 1;  // a denormal
+    atomicMax(&top[ff][fa], hi);
+  }
+  bool off = false;  // uniform over the block after the last level
   // levels n = 2, 3: one thread a row of W(A, D) (each W(A, P) row serves three
   // elements); level 4, with only 8 pairs: one thread an element
 #pragma unroll
@@ -307,71 +390,62 @@ __global__ void __launch_bounds__(NPR_BT, 4) k_npr_fx(const NprArgs a) {
         W[D * 16 + A][(j0 + j) * 3 + i] = fx_conj(w);
       }
     }
-    __syncthreads();
+    if (n == 3 && t < 192) {  // top is complete since the last barrier
+      const int hi = top[ff][fa], E = hi >> 20;
+      off = hi != 0 && (E < NPR_E0 || E > NPR_E1);
+      const Fx re = fx_vec(__double2hiint(fv.x), __double2loint(fv.x), off ? 2047 : E);
+      const Fx im = fx_vec(__double2hiint(fv.y), __double2loint(fv.y), off ? 2047 : E);
+      fld[ff][fa][fc] = make_int4(re.h, re.l, im.h, im.l);
+    }
+    if (n < 4) __syncthreads();
   }
-  int E[4];
-  bool wide = false;  // uniform over the block
-#pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    E[f] = top[f] >> 20;
-    wide |= E[f] < NPR_E0 || E[f] > NPR_E1;
+  off = __syncthreads_or(off || nsmall > 32 * 18 / 8) != 0;
+  if (off) {
+    npr_block_fp64(a, reinterpret_cast<double2(*)[9]>(&W[0][0]), reinterpret_cast<double2(*)[16][3]>(&fld[0][0][0]),
+                   term, pa, pd);
+    return;
   }
   const int A = t >> 4, C = t & 15;
   const int B = A ^ a.S1 ^ a.F1, Dd = C ^ a.S2 ^ a.F2;
   const double s = spin_taste(a.S1, a.F1, A, B) * spin_taste(a.S2, a.F2, C, Dd);
-  if (!wide) {
-    if (t < 192) {
-      const int Ef = top[ff] >> 20;
-      const Fx re = fx_vec(__double2hiint(fv.x), __double2loint(fv.x), Ef);
-      const Fx im = fx_vec(__double2hiint(fv.y), __double2loint(fv.y), Ef);
-      fld[ff][fa][fc] = make_int4(re.h, re.l, im.h, im.l);
-    }
-    __syncthreads();
-    // one bilinear: x^T W y with x, y at 2^57, W at 2^58: W y at 2^57, the sum at 2^56
-    auto bilinear = [&](const int4 *x, const int4 *w, const int4 *y, long long &re, long long &im) {
-      CAcc sum = cacc_zero();
+  // the bilinear of fields f at corner X and g at corner Y: x^T W y with x, y at
+  // 2^57, W at 2^58: W y at 2^57, the sum at 2^56
+  auto bilinear = [&](int f, int X, int g, int Y, bool &check) {
+    const int4 *x = fld[f][X], *w = W[X * 16 + Y], *y = fld[g][Y];
+    CAcc sum = cacc_zero();
+    int seen_re = 0, seen_im = 0;  // bits of the partial sums' magnitudes
 #pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        CAcc v = cacc_zero();
-#pragma unroll
-        for (int j = 0; j < 3; ++j) fx_cmac(v, w[i * 3 + j], y[j]);
-        fx_cmac(sum, x[i], fx_cval(v));
-      }
-      re = fx_sum(sum.re);
-      im = fx_sum(sum.im);
-    };
-    long long r1, i1, r2, i2;
-    bilinear(fld[0][A], W[A * 16 + Dd], fld[3][Dd], r1, i1);
-    bilinear(fld[2][C], W[C * 16 + B], fld[1][B], r2, i2);
-    // units 2^(E - 1022) of each field and 2^-56
-    const double u1 = s * __hiloint2double((E[0] + E[3] - 2 * 1022 - 56 + 1023) << 20, 0);
-    const double u2 = __hiloint2double((E[1] + E[2] - 2 * 1022 - 56 + 1023) << 20, 0);
-    term[t] = zm(make_double2((double)r1 * u1, (double)i1 * u1), make_double2((double)r2 * u2, (double)i2 * u2));
-  } else {
-    // the path averages to FP64 in place, the fields as they are
-    double2 *Wd = reinterpret_cast<double2 *>(&W[0][0]);
-    for (int k = t; k < 256 * 9; k += NPR_BT) {
-      const int4 w = (&W[0][0])[k];
-      Wd[k] = make_double2(__fma_rn((double)w.x, 0x1p-29, (double)w.y * 0x1p-58),
-                           __fma_rn((double)w.z, 0x1p-29, (double)w.w * 0x1p-58));
-    }
-    double2 *fd = reinterpret_cast<double2 *>(&fld[0][0][0]);
-    if (t < 192) fd[t] = fv;
-    __syncthreads();
-    double2 t1 = make_double2(0.0, 0.0), t2 = make_double2(0.0, 0.0);
-#pragma unroll 1
     for (int i = 0; i < 3; ++i) {
-      double2 v1 = make_double2(0.0, 0.0), v2 = make_double2(0.0, 0.0);
-      for (int j = 0; j < 3; ++j) {
-        v1 = zfma(Wd[(A * 16 + Dd) * 9 + i * 3 + j], fd[(3 * 16 + Dd) * 3 + j], v1);
-        v2 = zfma(Wd[(C * 16 + B) * 9 + i * 3 + j], fd[(16 + B) * 3 + j], v2);
-      }
-      t1 = zfma(fd[A * 3 + i], v1, t1);
-      t2 = zfma(fd[(2 * 16 + C) * 3 + i], v2, t2);
+      CAcc v = cacc_zero();
+#pragma unroll
+      for (int j = 0; j < 3; ++j) fx_cmac(v, w[i * 3 + j], y[j]);
+      fx_cmac(sum, x[i], fx_cval(v));
+      const int hr = (int)(sum.re.hh >> 32), hi = (int)(sum.im.hh >> 32);
+      seen_re |= hr ^ (hr >> 31);
+      seen_im |= hi ^ (hi >> 31);
     }
-    const double2 z = zm(t1, t2);
-    term[t] = make_double2(s * z.x, s * z.y);
+    const int tx = top[f][X], ty = top[g][Y], step = X ^ Y;
+    // units 2^(E - 1022) of each corner and 2^-56; 0 with a zero corner
+    const bool zero = tx == 0 || ty == 0;
+    check = !zero && min(seen_re, seen_im) < NPR_LINE && (step & (step - 1)) == 0;
+    const double unit = zero ? 0.0 : __hiloint2double(((tx >> 20) + (ty >> 20) - 2 * 1022 - 56 + 1023) << 20, 0);
+    return make_double2((double)fx_sum(sum.re) * unit, (double)fx_sum(sum.im) * unit);
+  };
+  bool check1, check2;
+  double2 b1 = bilinear(0, A, 3, Dd, check1), b2 = bilinear(2, C, 1, B, check2);
+  if (check1 || check2) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      if (!(q ? check2 : check1)) continue;
+      const int X = q ? C : A, Y = q ? B : Dd, step = X ^ Y;
+      const double2 *u = step ? a.U + ((long long)(__ffs(step) - 1) * a.V + site(X & Y)) * 9 : nullptr;
+      double2 &b = q ? b2 : b1;
+      b = bilinear_checked(b, fld[q ? 2 : 0][X], W[X * 16 + Y], fld[q ? 1 : 3][Y], (q ? a.cb3 : a.cb1) + site(X) * 3,
+                           (q ? a.c2 : a.c4) + site(Y) * 3, u, X > Y);
+    }
   }
+  const double2 z = zm(b1, b2);
+  term[t] = make_double2(s * z.x, s * z.y);
   __syncthreads();
   // fixed-order sum of the 256 terms by one warp
   if (t < 32) {
