@@ -5,8 +5,8 @@
 //   2. corrections Q <- Q (1 + D) from residuals in fixed point: with M = Q^dag X,
 //      E = Q^dag Q - 1, the exact factor has D = Ds + Da to first order,
 //        Ds = -E / 2,   H Da + Da H = (M - M^dag) + Ds H - H Ds,   H = (M + M^dag) / 2,
-//      solved in FP32 (a relative accuracy near 1e-5 suffices: each correction
-//      gains that factor), until a correction is small enough to be the last;
+//      solved in FP32 (each correction gains the factor that this is accurate to),
+//      until a correction leaves too little to matter;
 //   3. the phase of det Q: z = z0 (1 - e/3 + 2 e^2/9), z0 ~ det^(-1/3) from
 //      FP32, e = z0^3 det - 1 in fixed point.
 // Everything that decides the result's last bits is an integer sum (unit 2^-58),
@@ -18,11 +18,19 @@
 
 namespace stag {
 
-// A correction below this is the last: it leaves about 1e-6 of itself.
-// Measured (elements against 80-bit arithmetic, 600 000 matrices like HYP's of
-// links with c = 0.1 ... 1): median 5e-17, at most 8.5e-17 up to condition
-// numbers near 10 and 6e-15 at 500; two corrections, rarely three.
-constexpr float FX_LAST = 0x1p-34f;
+// Each correction leaves the fraction of itself that its FP32 solution is off by:
+// 1e-6 for well-conditioned matrices, up to 1e-2 at condition numbers of some
+// hundreds.  The fraction is seen in how much smaller a correction m is than the
+// one before, so the last is the first with m (m / previous m) below FX_LEFT.  (A
+// line for m alone, 2^-34, stopped after the second correction whatever the
+// condition: at a condition number of 300 errors of 4e-13, where the FP64 form has 1e-14.)
+// Measured on the CPU (elements against 113-bit arithmetic, 1500 matrices a condition
+// number, median / largest; the FP64 form): 4: 6e-18 / 1e-17 (1e-16 / 3e-16),
+// 30: 2e-17 / 3e-16 (2e-16 / 7e-16), 100: 4e-17 / 2e-15 (4e-16 / 3e-15), 300: 1e-16 / 8e-16
+// (1e-15 / 1e-14), with the singular values spread evenly; from some hundreds on an
+// increasing part does not converge in five corrections and is left to FP64.
+// Two corrections, or three from condition numbers near 10 on.
+constexpr float FX_LEFT = 0x1p-56f;
 
 struct C3 {  // FP32 3 x 3
   float2 a[9];
@@ -260,6 +268,7 @@ FX_HD void add_product(int4 *Q, const C3 &D, float m) {
 template <int ST>
 FX_HD bool project_su3_fx(const int4 *X, int4 *Q, float *f) {
   bool good, done = false;
+  float prev = 1.f;  // the correction before
   {
     C3 y;
 #pragma unroll
@@ -334,7 +343,8 @@ FX_HD bool project_su3_fx(const int4 *X, int4 *Q, float *f) {
     }
     good = good && m < 1e-2f;  // false for NaN
     add_product<ST>(Q, D, good ? m : 1e-2f);
-    done = done || m < FX_LAST;
+    done = done || m * m < FX_LEFT * prev;
+    prev = m;
     if (!any_lane(good && !done)) break;
   }
   // det Q = row 0 . (row 1 x row 2)
