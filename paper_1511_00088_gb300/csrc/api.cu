@@ -2382,13 +2382,13 @@ int stag_hyp_smear(stag_ctx *c, const double alpha[3], const double *links_in, d
     U = reinterpret_cast<const double2 *>(c->hyp_io.p);
   }
   double2 *out = out_dev ? reinterpret_cast<double2 *>(links_out) : reinterpret_cast<double2 *>(c->hyp_io.p);
-  CK(c->defect.ensure(sizeof(unsigned long long)));
+  CK(c->defect.ensure(sizeof(FieldCheck)));
   void *fix = nullptr;  // without room for it: the FP64 form
   if (c->fx_mode) {
     if (c->hyp_u.ensure(bytes) == cudaSuccess) fix = c->hyp_u.p;
     else cudaGetLastError();
   }
-  CK(launch_hyp(c->dims, U, a, (double2 *)c->hyp_b.p, (double2 *)c->hyp_t.p, out, fix, (int *)c->defect.p, c->stream));
+  CK(launch_hyp(c->dims, U, a, (double2 *)c->hyp_b.p, (double2 *)c->hyp_t.p, out, fix, (FieldCheck *)c->defect.p, c->stream));
   if (!out_dev) CK(cudaMemcpyAsync(links_out, c->hyp_io.p, bytes, cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   return STAG_OK;

@@ -17,7 +17,7 @@
 // g = |det Y|^(-1/3); Higham, "Computing the polar decomposition", 1986),
 // which reaches the same unique factor in fewer steps than the plain one, and
 // the determinant's phase from Newton's iteration for a complex cube root.
-// Near-unitary fields run on the integer pipe instead (k_hyp*_fx below).
+// Fields that pass fx_field run on the integer pipe instead (k_hyp*_fx below).
 // One thread per (decorated link, site); links in the ABI layout
 // [direction][site][3][3] complex (decorated: [12 (mu, decoration) slots][site][3][3]).
 #include <cmath>
@@ -225,11 +225,11 @@ __device__ __forceinline__ void smear_store(const double2 *u, double a, double w
   for (int k = 0; k < 9; ++k) out[k] = W.a[k];
 }
 
-// The FP64 levels.  run != nullptr: only where *run is set (a field that the
-// fixed-point levels left alone).
+// The FP64 levels.  run != nullptr: only for a field that the fixed-point
+// levels left alone.
 // level 1: thread over (mu, e != mu, site); Vb stored [dslot(mu, e)][V]
-__global__ void k_hyp1(Lat g, const int *run, const double2 *U, double a3, double2 *Vb) {
-  if (run != nullptr && *run == 0) return;
+__global__ void k_hyp1(Lat g, const FieldCheck *run, const double2 *U, double a3, double2 *Vb) {
+  if (run != nullptr && fx_field(*run, 4 * g.V)) return;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 12 * g.V) return;
   const long long i = t % g.V;
@@ -245,8 +245,8 @@ __global__ void k_hyp1(Lat g, const int *run, const double2 *U, double a3, doubl
 }
 
 // level 2: thread over (mu, nu != mu, site); Vt stored [dslot(mu, nu)][V]
-__global__ void k_hyp2(Lat g, const int *run, const double2 *U, const double2 *Vb, double a2, double2 *Vt) {
-  if (run != nullptr && *run == 0) return;
+__global__ void k_hyp2(Lat g, const FieldCheck *run, const double2 *U, const double2 *Vb, double a2, double2 *Vt) {
+  if (run != nullptr && fx_field(*run, 4 * g.V)) return;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 12 * g.V) return;
   const long long i = t % g.V;
@@ -266,8 +266,8 @@ __global__ void k_hyp2(Lat g, const int *run, const double2 *U, const double2 *V
 }
 
 // level 3: thread over (mu, site); out may alias U (each thread reads only its own thin link)
-__global__ void k_hyp3(Lat g, const int *run, const double2 *U, const double2 *Vt, double a1, double2 *out) {
-  if (run != nullptr && *run == 0) return;
+__global__ void k_hyp3(Lat g, const FieldCheck *run, const double2 *U, const double2 *Vt, double a1, double2 *out) {
+  if (run != nullptr && fx_field(*run, 4 * g.V)) return;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 4 * g.V) return;
   const long long i = t % g.V;
@@ -304,7 +304,7 @@ __global__ void k_hyp3(Lat g, const int *run, const double2 *U, const double2 *V
 }
 
 // ---------------------------------------------------------------------------
-// the same three levels on the integer pipe (near-unitary fields)
+// the same three levels on the integer pipe (fields that pass fx_field)
 // ---------------------------------------------------------------------------
 // The FP64 levels keep the FP64 pipe 95 % busy: per site 20 700 FMAs of staples
 // and 33 600 of projections (44.8 ms at 20^3 x 64).  Here the staples are
@@ -315,8 +315,9 @@ __global__ void k_hyp3(Lat g, const int *run, const double2 *U, const double2 *V
 // positive scale.  Fields lie as [slot][element][site] int4, so that a warp's
 // 32 sites are 512 contiguous bytes a load.  A thread whose projection does not
 // converge (a sum near singular) projects in FP64; where that has no result
-// either, levels 1 and 2 set *bad, as the conversion does on a field that is not
-// near unitary, and the FP64 levels run.
+// either, levels 1 and 2 mark the field as bad, and the FP64 levels run, as on
+// a field whose conversion did not pass fx_field (links that mix too little keep
+// small elements, which fixed-point numbers hold to 2^-58 only).
 struct FLat {
   Lat g;
   FastDiv d0, d1, d2;
@@ -437,38 +438,55 @@ __device__ __forceinline__ bool smear_fx(const int4 *pu, long long V, Fx c, int 
   return project_fallback(X, Q);
 }
 
-// canonical FP64 links -> [mu][9][V] fixed-point; *bad where not near unitary
-__global__ void __launch_bounds__(256) k_hyp_fix(long long V, const double2 *__restrict__ U, int4 *F, int *bad) {
+// canonical FP64 links -> [mu][9][V] fixed-point, and the check of the field
+__global__ void __launch_bounds__(256) k_hyp_fix(long long V, const double2 *__restrict__ U, int4 *F, FieldCheck *check) {
   const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
-  if (t >= 4 * V) return;
-  const long long mu = t / V, i = t - mu * V;
-  float2 u[9];
   bool ok = true;
+  int nsmall = 0;
+  if (t < 4 * V) {
+    const long long mu = t / V, i = t - mu * V;
+    float2 u[9];
 #pragma unroll
-  for (int e = 0; e < 9; ++e) {
-    const double2 w = U[t * 9 + e];
-    const int hx = __double2hiint(w.x), hy = __double2hiint(w.y);
-    ok = ok && (hx & 0x7fffffff) < 0x40000000 && (hy & 0x7fffffff) < 0x40000000;
-    const Fx a = fx_link(hx, __double2loint(w.x)), b = fx_link(hy, __double2loint(w.y));
-    F[(mu * 9 + e) * V + i] = make_int4(a.h, a.l, b.h, b.l);
-    u[e] = make_float2((float)a.h * 0x1p-29f, (float)b.h * 0x1p-29f);
+    for (int e = 0; e < 9; ++e) {
+      const double2 w = U[t * 9 + e];
+      const int hx = __double2hiint(w.x), hy = __double2hiint(w.y);
+      ok = ok && (hx & 0x7fffffff) < 0x40000000 && (hy & 0x7fffffff) < 0x40000000;
+      const Fx a = fx_link(hx, __double2loint(w.x)), b = fx_link(hy, __double2loint(w.y));
+      F[(mu * 9 + e) * V + i] = make_int4(a.h, a.l, b.h, b.l);
+      u[e] = make_float2((float)a.h * 0x1p-29f, (float)b.h * 0x1p-29f);
+    }
+    ok = ok && near_unitary(u);
+    nsmall = small_parts(u);
   }
-  if (!ok || !near_unitary(u)) *bad = 1;
+  check_link(check, ok, nsmall);
 }
 
 struct HypFx {
   FLat f;
   long long V;
   const int4 *U;  // [4][9][V]
-  int *bad;
+  FieldCheck *check;
   Fx c;
   int q;
 };
 
+// whether a level leaves the field alone; other blocks of it may be marking the
+// field, so the block's threads decide together (whole warps project together)
+__device__ __forceinline__ bool hyp_off(const HypFx &h) {
+  bool off = false;
+  if (threadIdx.x == 0) {
+    FieldCheck f;
+    f.small = h.check->small;
+    f.bad = *(volatile int *)&h.check->bad;
+    off = !fx_field(f, 4 * h.V);
+  }
+  return __syncthreads_or(off) != 0;
+}
+
 // level 1 (LEVEL = 1: Vb from U) and level 2 (Vt from Vb); blockIdx.y = slot
 template <int LEVEL>
 __global__ void __launch_bounds__(HFX_BT, 3) k_hyp12_fx(const HypFx h, const int4 *__restrict__ src, int4 *dst) {
-  if (*(volatile int *)h.bad != 0) return;
+  if (hyp_off(h)) return;
   // threads past the last site repeat it (whole warps project together) and store nothing
   const unsigned i0 = blockIdx.x * HFX_BT + threadIdx.x, i = i0 < h.V ? i0 : (unsigned)h.V - 1;
   const int pr = blockIdx.y, mu = pr / 3, e = (pr % 3 >= mu) ? pr % 3 + 1 : pr % 3;
@@ -493,7 +511,7 @@ __global__ void __launch_bounds__(HFX_BT, 3) k_hyp12_fx(const HypFx h, const int
     for (int neg = 0; neg < 2; ++neg)
       staple_fx(A + (neg ? dn : i), B + (neg ? dn : up), A + (neg ? dnmu : imu), (int)V, neg, X);
   }
-  if (!smear_fx(h.U + (long long)mu * 9 * V + i, V, h.c, h.q, X, Q, &hsh->f[0][threadIdx.x])) *h.bad = 1;
+  if (!smear_fx(h.U + (long long)mu * 9 * V + i, V, h.c, h.q, X, Q, &hsh->f[0][threadIdx.x])) h.check->bad = 1;
   if (i0 >= h.V) return;
 #pragma unroll
   for (int k = 0; k < 9; ++k) dst[((long long)pr * 9 + k) * V + i] = Q[k * HFX_BT];
@@ -501,7 +519,7 @@ __global__ void __launch_bounds__(HFX_BT, 3) k_hyp12_fx(const HypFx h, const int
 
 // level 3 (the smeared links, FP64 ABI layout; may be the buffer U came from); blockIdx.y = mu
 __global__ void __launch_bounds__(HFX_BT, 3) k_hyp3_fx(const HypFx h, const int4 *__restrict__ Vt, double2 *out) {
-  if (*(volatile int *)h.bad != 0) return;
+  if (hyp_off(h)) return;
   const unsigned i0 = blockIdx.x * HFX_BT + threadIdx.x, i = i0 < h.V ? i0 : (unsigned)h.V - 1;
   const int mu = blockIdx.y;
   const long long V = h.V;
@@ -549,7 +567,7 @@ bool mix_of(double a, double w, int staples, Fx *c, int *q) {
 }  // namespace
 
 cudaError_t launch_hyp(const int dims[4], const double2 *U, const double alpha[3], double2 *Vb, double2 *Vt,
-                       double2 *out, void *fixU, int *bad, cudaStream_t st) {
+                       double2 *out, void *fixU, FieldCheck *check, cudaStream_t st) {
   Lat g;
   for (int k = 0; k < 4; ++k) g.L[k] = dims[k];
   g.V = (long long)dims[0] * dims[1] * dims[2] * dims[3];
@@ -557,16 +575,16 @@ cudaError_t launch_hyp(const int dims[4], const double2 *U, const double alpha[3
   Fx c[3];
   int q[3];
   cudaError_t e = cudaSuccess;
-  const int *run = nullptr;
+  const FieldCheck *run = nullptr;
   if (fixU != nullptr && g.V < (1ll << 27) && mix_of(alpha[2], alpha[2] / 2.0, 2, &c[0], &q[0]) &&
       mix_of(alpha[1], alpha[1] / 4.0, 4, &c[1], &q[1]) && mix_of(alpha[0], alpha[0] / 6.0, 6, &c[2], &q[2])) {
     for (const void *k : {(const void *)k_hyp12_fx<1>, (const void *)k_hyp12_fx<2>, (const void *)k_hyp3_fx}) {
       e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(HfxShared));
       if (e != cudaSuccess) return e;
     }
-    e = cudaMemsetAsync(bad, 0, sizeof(int), st);
+    e = cudaMemsetAsync(check, 0, sizeof(FieldCheck), st);
     if (e != cudaSuccess) return e;
-    run = bad;
+    run = check;
     HypFx h;
     h.f.g = g;
     h.f.d0 = make_fastdiv((unsigned)dims[0]);
@@ -574,8 +592,8 @@ cudaError_t launch_hyp(const int dims[4], const double2 *U, const double alpha[3
     h.f.d2 = make_fastdiv((unsigned)dims[2]);
     h.V = g.V;
     h.U = reinterpret_cast<const int4 *>(fixU);
-    h.bad = bad;
-    k_hyp_fix<<<(unsigned)((4 * g.V + 255) / 256), 256, 0, st>>>(g.V, U, reinterpret_cast<int4 *>(fixU), bad);
+    h.check = check;
+    k_hyp_fix<<<(unsigned)((4 * g.V + 255) / 256), 256, 0, st>>>(g.V, U, reinterpret_cast<int4 *>(fixU), check);
     const unsigned nb = (unsigned)((g.V + HFX_BT - 1) / HFX_BT);
     h.c = c[0];
     h.q = q[0];
