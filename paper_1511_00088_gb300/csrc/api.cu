@@ -2254,13 +2254,13 @@ int stag_links_upload(stag_ctx *c, const double *links) {
   }
   CK(c->links64.ensure(cplx_bytes(P64) * 9ull * 8ull * c->Ve));
   // The FP64 copy, and with room for it the fixed-point copy; a field that does
-  // not pass fx_field keeps the FP64 operator.
-  // (Below 128 sites a parity the FP64 form stays: a few warps' work, where the
-  // pipe does not matter.)
+  // not pass fx_field keeps the FP64 operator.  No lattice is too small for it
+  // (2^4, 8 sites a parity: M^dag M call 27 us, 42 with the FP64 form and its
+  // copies between layouts; NPR contraction 50 and 60; FP64 CG 0.5 and 0.8 ms).
   const bool fx_was = c->fx_ok;
   FieldCheck check = {0, 1};
   c->fx_ok = false;
-  if (c->fx_mode && c->Ve >= 128 && c->links_fx.ensure(cplx_bytes(PFX) * 9ull * 8ull * c->Ve) == cudaSuccess) {
+  if (c->fx_mode && c->links_fx.ensure(cplx_bytes(PFX) * 9ull * 8ull * c->Ve) == cudaSuccess) {
     CK(c->defect.ensure(sizeof(FieldCheck)));
     CK(cudaMemsetAsync(c->defect.p, 0, sizeof(FieldCheck), c->stream));
     CK(launch_pack_links_fx(reinterpret_cast<const double2 *>(c->links_canon.p), (double2 *)c->links64.p,

@@ -107,7 +107,15 @@ def test_every_component_as_in_fp64(kind, spread):
                                           ("phases", False)])
 def test_the_form_that_runs(kind, integer, monkeypatch):
     """Other bits than the FP64 form's where the integer form runs, the same where it does not."""
-    L = (6, 4, 4, 8)
+    check_form((6, 4, 4, 8), kind, integer, monkeypatch)
+
+
+@pytest.mark.parametrize("L", [(2, 2, 2, 2), (4, 4, 2, 6), (4, 2, 6, 4)])
+def test_small_lattices_run_the_integer_form(L, monkeypatch):
+    check_form(L, "rough", True, monkeypatch)
+
+
+def check_form(L, kind, integer, monkeypatch):
     U = links(kind, L, 1211)
     v = synth.gaussian_vector(synth.volume(L) // 2, 1212)
     got = []

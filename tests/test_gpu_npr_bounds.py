@@ -195,10 +195,10 @@ def test_ends_of_the_range_on_the_integer_kernel(how):
     assert np.all(np.abs(O - clean)[~bad] <= BOUND * S[~bad])
 
 
-def test_the_forms_that_run(monkeypatch):
+@pytest.mark.parametrize("L", [(2, 2, 2, 2), (4, 2, 6, 4), (4, 4, 4, 8)])
+def test_the_forms_that_run(L, monkeypatch):
     """Rough SU(3) fields contract on the integer pipe (other bits than the FP64 form); fields that are nearly
     diagonal or not unitary in FP64 (the same bits)."""
-    L = (4, 4, 4, 8)
     V = synth.volume(L)
     fs = [synth.gaussian_vector(V, 1162 + k) for k in range(4)]
     fields = {"rough": synth.random_links(L, 0.4, 1161), "cold": synth.random_links(L, 0.02, 1161),
