@@ -657,16 +657,18 @@ __global__ void k_ps_map(const PsArgs a, int nblocks, int full) {
   }
 }
 
-// launch k, or (kptr) return it
-cudaError_t ps_launch(void (*k)(PsArgs), unsigned smem, int nblocks, cudaStream_t st, const PsArgs &a, const void **kptr) {
+// launch k, or (kptr) return it.  The limit of a kernel's dynamic shared memory
+// belongs to the process, not to the launch: it is set to `most`, all that any
+// launch of k asks for, as another thread's context may be between its own
+// setting and its launch.
+cudaError_t ps_launch(void (*k)(PsArgs), unsigned smem, unsigned most, int nblocks, cudaStream_t st, const PsArgs &a,
+                      const void **kptr) {
   if (kptr) {
     *kptr = (const void *)k;
     return cudaSuccess;
   }
-  if (smem > 0) {
-    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.dynamicSmemBytes = smem;
   cfg.gridDim = dim3((unsigned)nblocks);
@@ -701,9 +703,10 @@ cudaError_t launch_cg_persist(int recon, int lanes, int nblocks, cudaStream_t st
     if (e != cudaSuccess) return e;
   }
   const unsigned link = (recon ? 6u : 9u) * 32u * 8u;  // bytes of one link of 32 lanes
-  if (lanes == 1)
-    return ps_launch(recon ? k_cg_persist_sm<1> : k_cg_persist_sm<0>, PS_CW * (unsigned)ps_staged_links(recon) * link,
-                     nblocks, st, a, kptr);
+  if (lanes == 1) {
+    const unsigned bytes = PS_CW * (unsigned)ps_staged_links(recon) * link;
+    return ps_launch(recon ? k_cg_persist_sm<1> : k_cg_persist_sm<0>, bytes, bytes, nblocks, st, a, kptr);
+  }
   // shared memory for the links of as many chunks as fit, at most all of a block's
   const int sites = 32 / lanes, nall = (a.g.Ve + sites - 1) / sites;
   const unsigned bytes = (unsigned)(8 / lanes) * link;
@@ -712,7 +715,8 @@ cudaError_t launch_cg_persist(int recon, int lanes, int nblocks, cudaStream_t st
   a.nres = (int)(PS_SMEM / bytes);
   if (a.nres > most) a.nres = most;
 #define STAG_PS(R_, L_) \
-  if (recon == R_ && lanes == L_) return ps_launch(k_cg_persist<R_, L_>, (unsigned)a.nres * bytes, nblocks, st, a, kptr);
+  if (recon == R_ && lanes == L_) \
+    return ps_launch(k_cg_persist<R_, L_>, (unsigned)a.nres * bytes, PS_SMEM / bytes * bytes, nblocks, st, a, kptr);
   STAG_PS(0, 4) STAG_PS(1, 4) STAG_PS(0, 2) STAG_PS(1, 2)
 #undef STAG_PS
   return cudaErrorNotSupported;

@@ -1,0 +1,49 @@
+"""Calls around the persistent CG kernel that the two-kernel form answers: several contexts at once, sources near the
+ends of FP32's range, streams with part of the GPU, switches at their defaults, a form asked for after an upload."""
+import threading
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1511_00088_gb300 import stag, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_1511_00088_gb300 import build
+    build.build()
+    stag.load()
+
+
+@pytest.mark.parametrize("eager", ["1", "0"])
+def test_threads_with_lattices_of_different_sizes(eager, monkeypatch):
+    """Two threads whose contexts run the same kernel with different amounts of shared memory."""
+    monkeypatch.setenv("STAG_EAGER", eager)
+    sizes = [(8, 8, 8, 8), (4, 4, 4, 4)]
+    streams = [torch.cuda.Stream() for _ in sizes]
+    failures = []
+
+    def work(k):
+        try:
+            L = sizes[k]
+            b = synth.gaussian_vector(synth.volume(L) // 2, 1302 + k)
+            U = synth.random_links(L, 0.4, 1301)
+            for _ in range(6):  # a graph is built for every upload
+                with stag.Context(L, stream=streams[k].cuda_stream) as ctx:
+                    ctx.links_upload(U)
+                    for _ in range(40):
+                        x = ctx.cg_solve([b], [0.3])[0][0]
+                    assert ctx.solve_form()["kernels"] == "k_cg_persist" and ctx.solve_form()["lanes_k1"] == 4
+            assert oracle.true_residual(L, U, 0.3, b, x) <= 1e-10
+        except Exception as e:  # noqa: BLE001 (reported by the main thread)
+            failures.append((k, e))
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failures, failures
