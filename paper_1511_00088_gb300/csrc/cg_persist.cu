@@ -83,29 +83,31 @@ __device__ __forceinline__ void read_slots(const PsArgs &a, int half, int grp, i
   }
 }
 
-// Sum of a warp's FP32 values (bit patterns), the same whatever their order: each
-// at 20 bits below the largest one's last place, added as integers (what lies
-// below, 2^-44 of the largest value, is dropped).  FP64 additions, 67 clocks each
+// Sum of a warp's FP32 values (bit patterns) x 2^up, the same whatever their
+// order: each at 20 bits below the largest one's last place, added as integers
+// (what lies below, 2^-44 of the largest value, is dropped: the values are FP32
+// sums, good to 2^-24 of themselves).  Denormals count: a source of 1e-12 has
+// nothing else once its residual is 1e-10 of it.  FP64 additions, 67 clocks each
 // in a chain of ten, took three times as long, and every block waits for this.
-__device__ __forceinline__ double fixed_sum(const unsigned (&x)[PS_PER]) {
+__device__ __forceinline__ double fixed_sum(const unsigned (&x)[PS_PER], int up) {
   unsigned top = 0;
 #pragma unroll
   for (int u = 0; u < PS_PER; ++u) top = max(top, x[u] & 0x7fffffffu);
   top = __reduce_max_sync(0xffffffffu, top);
-  const int E = (int)(top >> 23);
+  const int E = max((int)(top >> 23), 1);
   if (E == 255) return __longlong_as_double(0x7ff8000000000000ll);
   long long t = 0;
 #pragma unroll
   for (int u = 0; u < PS_PER; ++u) {
     const int e = (int)(x[u] >> 23) & 0xff;
-    const unsigned long long m = e ? ((unsigned long long)((x[u] & 0x7fffffu) | 0x800000u) << 20) : 0ull;
-    const long long v = (long long)(m >> min(E - e, 63));
+    const unsigned long long m = (unsigned long long)((x[u] & 0x7fffffu) | (e ? 0x800000u : 0u)) << 20;
+    const long long v = (long long)(m >> min(E - max(e, 1), 63));
     t += (int)x[u] < 0 ? -v : v;
   }
   const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)t & 0xffffffu);
   const int hi = __reduce_add_sync(0xffffffffu, (int)(t >> 24));
   const double d = (double)(((long long)hi << 24) + (long long)lo);
-  return d * __hiloint2double((E - 127 - 23 - 20 + 1023) << 20, 0);  // exact: E - 170 is in FP64's range
+  return d * __hiloint2double((E + up - 127 - 23 - 20 + 1023) << 20, 0);  // exact: E - 170 is in FP64's range
 }
 
 // a / b as FP32, from an FP32 quotient of the significands and its residual in
@@ -168,10 +170,14 @@ __device__ __forceinline__ void scalar_warp(const PsArgs &a, PsShared &sh, int g
     const double m4p2 = st.m4 * (st.rho + st.beta * (2.0 * st.rp + st.beta * st.pnorm2));
     const double rho = st.rho, low = st.delta * st.delta * st.rmax2;
     const bool last = st.iter + 1 >= st.maxiter;
+    // a block adds its warps' sums in FP32: scaled down where the sum of 15 might
+    // overflow (|t|^2 <= 64 |p|^2; all blocks hold the same state)
+    const int up = fmax(st.rho, st.pnorm2) > 0x1p90 ? 4 : 0;
+    const float down = up ? 0x1p-4f : 1.f;
     unsigned x0[PS_PER], x1[PS_PER];
     bar_sync(BAR_DONE);
     {
-      const float w = warp_sum(lane < PS_CW ? sh.red[0][lane] : 0.f);
+      const float w = warp_sum(lane < PS_CW ? down * sh.red[0][lane] : 0.f);
       arrivals += nbg;
       if (lane == 0) {
         post(a, 0, grp, blk, w, 0.f);
@@ -182,7 +188,7 @@ __device__ __forceinline__ void scalar_warp(const PsArgs &a, PsShared &sh, int g
     bar_arrive(BAR_DATA);
     {
       read_slots(a, 0, grp, nbg, x0, x1);
-      const double sum[2] = {fixed_sum(x0), 0.0};
+      const double sum[2] = {fixed_sum(x0, up), 0.0};
       const double pAp = m4p2 + sum[0];
       const bool stop = !(pAp > 0.0) || !isfinite(pAp) || !ok;
       if (lane == 0) {
@@ -200,8 +206,8 @@ __device__ __forceinline__ void scalar_warp(const PsArgs &a, PsShared &sh, int g
     // may not have, so the two halves use different words.
     bar_sync(BAR_DONE);
     {
-      const float w0 = warp_sum(lane < PS_CW ? sh.red[0][lane] : 0.f);
-      const float w1 = warp_sum(lane < PS_CW ? sh.red[1][lane] : 0.f);
+      const float w0 = warp_sum(lane < PS_CW ? down * sh.red[0][lane] : 0.f);
+      const float w1 = warp_sum(lane < PS_CW ? down * sh.red[1][lane] : 0.f);
       arrivals += nbg;
       if (lane == 0) {
         post(a, 1, grp, blk, w0, w1);
@@ -212,7 +218,7 @@ __device__ __forceinline__ void scalar_warp(const PsArgs &a, PsShared &sh, int g
     bar_arrive(BAR_DATA);
     {
       read_slots(a, 1, grp, nbg, x0, x1);
-      const double rr = fixed_sum(x0);
+      const double rr = fixed_sum(x0, up);
       // finalize_system's conditions for FIN_NORM
       const bool stop = !isfinite(rr) || rr <= tol2 || last || rr < low || !ok;
       if (lane == 0) {
@@ -221,7 +227,7 @@ __device__ __forceinline__ void scalar_warp(const PsArgs &a, PsShared &sh, int g
       }
       __syncwarp();
       bar_arrive(BAR_SCAL);
-      const double sum[2] = {rr, fixed_sum(x1)};
+      const double sum[2] = {rr, fixed_sum(x1, up)};
       if (lane == 0) finalize_system(st, FIN_NORM, sum);
       __syncwarp();
       if (stop) break;

@@ -47,3 +47,20 @@ def test_threads_with_lattices_of_different_sizes(eager, monkeypatch):
     for t in threads:
         t.join()
     assert not failures, failures
+
+
+@pytest.mark.parametrize("L,scale,tol", [((16, 16, 16, 32), 1.6e17, 1e-10), ((16, 16, 16, 32), 1e-12, 1e-10),
+                                         ((16, 16, 16, 32), 1e-13, 1e-10), ((8, 8, 8, 8), 1e-12, 1e-10),
+                                         ((8, 8, 8, 8), 1e-17, 1e-4)])
+def test_sources_near_the_ends_of_fp32(L, scale, tol, monkeypatch):
+    """FP32 sums of squares near overflow, and among the denormals: both forms solve."""
+    U = synth.random_links(L, 0.4, 1311)
+    b = scale * synth.gaussian_vector(synth.volume(L) // 2, 1312)
+    for ps in (None, "0"):
+        if ps is not None:
+            monkeypatch.setenv("STAG_PS", ps)
+        with stag.Context(L, recon12=True) as ctx:
+            ctx.links_upload(U)
+            xs, _, _, _ = ctx.cg_solve([b], [0.2], tol=tol, maxiter=2000)
+            assert (ctx.solve_form()["kernels"] == "k_cg_persist") == (ps is None)
+        assert oracle.true_residual(L, U, 0.2, b, xs[0]) <= 1.001 * tol
