@@ -155,6 +155,7 @@ struct Work {
                                    // the links staged once per tile): threads per site, + 10 with
                                    // one link stage
   const void *links_tile = nullptr;
+  int op64 = P64;                  // FP64 operator form (lp_for) that the launch forms were chosen for
   int ps_form = 0;                 // > 0: the iterations run in k_cg_persist, this form
   int ps_blocks = 0;               // its blocks, all systems together
   DevBuf ps_sync;                  // its exchange words and arrival counts
@@ -846,8 +847,11 @@ int work_prepare(stag_ctx *c, int nsys, int precision, int ms = 0) {
   }
   int psf = 0, psn = 0;
   choose_persist(c, prec, VP, nsys, ms, &psf, &psn);
-  if (w.nsys == nsys && w.prec == prec && w.VP == VP && w.recon == recon && w.ps_form == psf) return STAG_OK;
+  const int op64 = lp_for(c, P64);
+  if (w.nsys == nsys && w.prec == prec && w.VP == VP && w.recon == recon && w.ps_form == psf && w.op64 == op64)
+    return STAG_OK;
   w.drop_graph();
+  w.op64 = op64;
   w.ps_form = psf;
   w.ps_blocks = psn;
   if (psf) CK(w.ps_sync.ensure(ps_sync_bytes(nsys)));
@@ -2257,7 +2261,6 @@ int stag_links_upload(stag_ctx *c, const double *links) {
   // not pass fx_field keeps the FP64 operator.  No lattice is too small for it
   // (2^4, 8 sites a parity: M^dag M call 27 us, 42 with the FP64 form and its
   // copies between layouts; NPR contraction 50 and 60; FP64 CG 0.5 and 0.8 ms).
-  const bool fx_was = c->fx_ok;
   FieldCheck check = {0, 1};
   c->fx_ok = false;
   if (c->fx_mode && c->links_fx.ensure(cplx_bytes(PFX) * 9ull * 8ull * c->Ve) == cudaSuccess) {
@@ -2276,7 +2279,6 @@ int stag_links_upload(stag_ctx *c, const double *links) {
   c->w.drop_graph();  // the graph holds link pointers of the reduced-precision copies
   CK(cudaStreamSynchronize(c->stream));
   c->fx_ok = fx_field(check, 4 * c->V);
-  if (c->fx_ok != fx_was) c->w.nsys = 0;  // the FP64 launch forms were chosen for the other operator
   return STAG_OK;
 }
 

@@ -64,3 +64,19 @@ def test_sources_near_the_ends_of_fp32(L, scale, tol, monkeypatch):
             xs, _, _, _ = ctx.cg_solve([b], [0.2], tol=tol, maxiter=2000)
             assert (ctx.solve_form()["kernels"] == "k_cg_persist") == (ps is None)
         assert oracle.true_residual(L, U, 0.2, b, xs[0]) <= 1.001 * tol
+
+
+def test_the_form_of_the_last_solve_outlives_an_upload():
+    """stag_solve_form and stag_solve_stats describe the last solve also after a field of the other operator form."""
+    L = (4, 4, 4, 8)
+    U = synth.random_links(L, 0.4, 1321)
+    b = synth.gaussian_vector(synth.volume(L) // 2, 1322)
+    fields = (U, 2.0 * U, U)
+    with stag.Context(L) as ctx:
+        for k, W in enumerate(fields):
+            ctx.links_upload(W)
+            if k:
+                assert ctx.solve_form() == form and ctx.solve_stats() == stats
+            xs, _, _, _ = ctx.cg_solve([b] * 5, [0.3], precision=stag.STAG_FP64)
+            assert all(oracle.true_residual(L, W, 0.3, b, x) <= 1e-10 for x in xs)
+            form, stats = ctx.solve_form(), ctx.solve_stats()
