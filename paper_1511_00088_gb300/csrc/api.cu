@@ -2163,11 +2163,6 @@ int stag_create(const int dims[4], int flags, void *cuda_stream, stag_ctx **out)
   }
   const char *eager = getenv("STAG_EAGER");
   c->use_graph = !(eager && eager[0] == '1');
-  const char *ps = getenv("STAG_PS");
-  if (ps && ps[0] != 0) c->ps_mode = atoi(ps);
-  // a form forced for the two-kernel iteration
-  for (const char *v : {"STAG_TMA", "STAG_LANES", "STAG_NS", "STAG_MRHS", "STAG_NRHS", "STAG_FOLD", "STAG_PERSIST", "STAG_PDL"})
-    if (getenv(v)) c->ps_mode = 0;
   const char *fx = getenv("STAG_FX");
   c->fx_mode = !(fx && fx[0] == '0');
   const char *pdl = getenv("STAG_PDL");
@@ -2183,6 +2178,18 @@ int stag_create(const int dims[4], int flags, void *cuda_stream, stag_ctx **out)
   // memory caps the sites in flight per SM below what the registers hold)
   if (tma && (tma[0] == '0' || tma[0] == '1' || tma[0] == '2') && tma[1] == 0) c->tma_modes = 1 << (tma[0] - '0');
   else if (tma && tma[0] == 't' && tma[1] == 0) c->tma_modes = 0b111;
+  // STAG_PS = 0, 1, 2 or 4; without it, a switch that asks for a form of the
+  // two-kernel iteration keeps that iteration
+  const char *ps = getenv("STAG_PS");
+  if (ps && ps[0] != 0) {
+    c->ps_mode = atoi(ps);
+  } else {
+    if (!c->pdl || !c->fold || !c->persist) c->ps_mode = 0;
+    for (const char *v : {"STAG_TMA", "STAG_LANES", "STAG_NS", "STAG_MRHS", "STAG_NRHS"}) {
+      const char *set = getenv(v);
+      if (set && set[0] != 0) c->ps_mode = 0;
+    }
+  }
   const char *giveup = getenv("STAG_TEST_WAIT_GIVEUP");
   c->wait_giveup = (giveup && giveup[0] == '1') ? 1 : 0;
   cudaError_t e = cudaGetDevice(&c->device);

@@ -80,3 +80,18 @@ def test_the_form_of_the_last_solve_outlives_an_upload():
             xs, _, _, _ = ctx.cg_solve([b] * 5, [0.3], precision=stag.STAG_FP64)
             assert all(oracle.true_residual(L, W, 0.3, b, x) <= 1e-10 for x in xs)
             form, stats = ctx.solve_form(), ctx.solve_stats()
+
+
+@pytest.mark.parametrize("switch", ["STAG_PDL", "STAG_FOLD", "STAG_PERSIST"])
+def test_a_switch_at_its_default_changes_nothing(switch, monkeypatch):
+    L = (8, 8, 8, 8)
+    U = synth.random_links(L, 0.4, 1331)
+    b = synth.gaussian_vector(synth.volume(L) // 2, 1332)
+    got = {}
+    for value in ("", "1", "0"):
+        monkeypatch.setenv(switch, value)
+        with stag.Context(L) as ctx:
+            ctx.links_upload(U)
+            ctx.cg_solve([b], [0.3])
+            got[value] = ctx.solve_form()["kernels"]
+    assert got == {"": "k_cg_persist", "1": "k_cg_persist", "0": "k_dslash"}
