@@ -836,7 +836,18 @@ void choose_persist(const stag_ctx *c, int LP, int VP, int nsys, int ms, int *fo
   *blocks = (long long)nsys * full < c->nsm ? nsys * full : c->nsm;
 }
 
+int work_fill(stag_ctx *c, int nsys, int precision, int ms);
+
+// The workspace of nsys systems; ms: shifted systems riding on each (multi-shift
+// CG).  One that could not be completed (no memory, say) counts as none: the
+// next call starts over.
 int work_prepare(stag_ctx *c, int nsys, int precision, int ms = 0) {
+  const int st = work_fill(c, nsys, precision, ms);
+  if (st != STAG_OK) c->w.nsys = 0;
+  return st;
+}
+
+int work_fill(stag_ctx *c, int nsys, int precision, int ms) {
   Work &w = c->w;
   int prec, VP, RP;
   if (!solver_precs(precision, &prec, &VP, &RP)) return arg_err(c, "bad solver precision");
