@@ -224,9 +224,8 @@ struct stag_ctx {
   int l2_modes = 0b11;    // 0b11: by rule; else bit p: the tuner may choose L2 mode p (STAG_L2PERSIST fixes it)
   size_t l2_max_persist = 0, l2_max_window = 0;
   DevBuf links_canon;  // [4][V][3][3] FP64, kept for lazy reduced-precision copies
-  DevBuf links64;
-  DevBuf links_fx;     // fixed-point copy (fixed.cuh) of a field it holds (fx_field), else unused
-  bool fx_ok = false;  // the FP64 operator runs from links_fx
+  DevBuf links64;      // the FP64 operator's copy: fixed-point (fixed.cuh) of a field that passes fx_field, else FP64
+  bool fx_ok = false;  // links64 is fixed-point
   bool fx_mode = true; // STAG_FX=0: never (the FP64 pipe's operator, for A/B runs)
   DevBuf links_lo[4][2];
   bool lo_ok[4][2] = {{false, false}, {false, false}, {false, false}, {false, false}};
@@ -333,7 +332,6 @@ int vec_out(stag_ctx *c, const VecBuf &v, int k, double *dst) {
 // FP64 operator form of the uploaded field: PFX (integer-pipe products of the
 // fixed-point links) on near-unitary fields that mix (fx_field), P64 on any other
 int lp_for(const stag_ctx *c, int P) { return (P == P64 && c->fx_ok) ? PFX : P; }
-const void *links64_op(const stag_ctx *c) { return c->fx_ok ? c->links_fx.p : c->links64.p; }
 // launch_dslash with the FP64 form of this field
 cudaError_t launch_ds(const stag_ctx *c, int LP, int recon, int VP, int OP, int NS, int EPI, int lanes, int nblocks,
                       cudaStream_t st, const DsArgs &a, const void **kptr = nullptr) {
@@ -346,7 +344,7 @@ int links_for(stag_ctx *c, int P, const void **out) {
     return STAG_ERR_STATE;
   }
   if (P == P64) {
-    *out = links64_op(c);
+    *out = c->links64.p;
     return STAG_OK;
   }
   const int rc = (c->flags & STAG_RECON12) ? 1 : 0;
@@ -403,7 +401,7 @@ void set_l2_window(stag_ctx *c, int P, int tma, int on, DsArgs &a) {
   if (!c->l2persist || !on) return;
   const int rc = (P != P64 && (c->flags & STAG_RECON12)) ? 1 : 0;
   const DevBuf &b = (on == 2) ? c->w.vpool
-                              : (P == P64) ? (c->fx_ok ? c->links_fx : c->links64)
+                              : (P == P64) ? c->links64
                                            : (tma ? c->links_tile[P][rc] : c->links_lo[P][rc]);
   if (!b.p || b.n == 0) return;
   a.l2_base = b.p;
@@ -1072,7 +1070,7 @@ int work_fill(stag_ctx *c, int nsys, int precision, int ms) {
   }
   // the thread mapping of the plain inner and the FP64 half operators
   if (!w.ps_form) CKS(tune_lanes(c, prec, recon, VP, w.NS, w.G, nsys, lo, w.p.arg(), w.t.arg(), &w.lanes));
-  CKS(tune_lanes(c, P64, 0, P64, w.NS64, w.G64, nsys, links64_op(c), w.x64.arg(), w.t64.arg(), &w.lanes64));
+  CKS(tune_lanes(c, P64, 0, P64, w.NS64, w.G64, nsys, c->links64.p, w.x64.arg(), w.t64.arg(), &w.lanes64));
   return STAG_OK;
 }
 
@@ -1333,7 +1331,7 @@ int enqueue_update(stag_ctx *c, cudaStream_t s, const Ctl &ctl) {
                      q));
   }
   DsArgs a = ds_base(c);
-  a.links = links64_op(c);
+  a.links = c->links64.p;
   a.nsys = w.nsys;
   a.ngroups = w.G64;
   a.ctl = ctl;
@@ -1638,9 +1636,9 @@ VecArg vec_slot(const VecBuf &v, int k) {
 
 int apply_m64(stag_ctx *c, int par_out, double m4, double scale, VecArg in, VecArg center, VecArg out) {
   int lanes = 1;
-  CKS(tune_lanes(c, P64, 0, P64, 1, 1, 1, links64_op(c), in, out, &lanes));
+  CKS(tune_lanes(c, P64, 0, P64, 1, 1, 1, c->links64.p, in, out, &lanes));
   DsArgs a = ds_base(c);
-  a.links = links64_op(c);
+  a.links = c->links64.p;
   a.nsys = 1;
   a.ngroups = 1;
   a.ctl = no_ctl();
@@ -1900,9 +1898,9 @@ int ms_impl(stag_ctx *c, const double *const src[], int nrhs, const double masse
 // out = D in (FP64) on the sites of parity par_out, one system
 int apply_m64_plain(stag_ctx *c, int par_out, VecArg in, VecArg out) {
   int lanes = 1;
-  CKS(tune_lanes(c, P64, 0, P64, 1, 1, 1, links64_op(c), in, out, &lanes));
+  CKS(tune_lanes(c, P64, 0, P64, 1, 1, 1, c->links64.p, in, out, &lanes));
   DsArgs a = ds_base(c);
-  a.links = links64_op(c);
+  a.links = c->links64.p;
   a.nsys = 1;
   a.ngroups = 1;
   a.ctl = no_ctl();
@@ -1962,7 +1960,8 @@ int force_impl(stag_ctx *c, const double *x_even, double scale, double *grad_lin
     if (g_host) off += gbytes;
   }
   if (lie_force) ldev = l_host ? (double *)((char *)c->stage_out.p + off) : lie_force;
-  CK(launch_force(c->g, (const double2 *)c->api_a.data.p, (const double2 *)c->api_b.data.p, c->links64.p, gdev, ldev,
+  CK(launch_force(c->g, (const double2 *)c->api_a.data.p, (const double2 *)c->api_b.data.p,
+                  (const double2 *)c->links_canon.p, gdev, ldev,
                   scale, c->stream));
   if (g_host) CK(cudaMemcpyAsync(grad_links, gdev, gbytes, cudaMemcpyDeviceToHost, c->stream));
   if (l_host) CK(cudaMemcpyAsync(lie_force, ldev, lbytes, cudaMemcpyDeviceToHost, c->stream));
@@ -2107,9 +2106,9 @@ int ragged_impl(const stag_solve_desc *d, int n, double tol, int maxiter, int pr
 
 // Internal accessors used by noalloc.cu (not part of the C ABI).
 namespace stag {
-int ctx_fp64_links(const stag_ctx *c, const void **links, cudaStream_t *stream) {
+int ctx_fp64_links(const stag_ctx *c, const double2 **links, cudaStream_t *stream) {
   if (!c->have_links) return STAG_ERR_STATE;
-  *links = c->links64.p;
+  *links = (const double2 *)c->links_canon.p;
   *stream = c->stream;
   return STAG_OK;
 }
@@ -2274,29 +2273,32 @@ int stag_links_upload(stag_ctx *c, const double *links) {
       return STAG_ERR_NOT_SU3;
     }
   }
+  // The FP64 operator's copy: fixed-point, unless the field does not pass fx_field.
+  // No lattice is too small for it (2^4, 8 sites a parity: M^dag M call 27 us, 42 with
+  // the FP64 form and its copies between layouts; NPR contraction 50 and 60; FP64
+  // CG 0.5 and 0.8 ms).  Both forms take 16 bytes an element, so one buffer serves.
+  static_assert(sizeof(int4) == sizeof(double2), "one buffer for either form");
   CK(c->links64.ensure(cplx_bytes(P64) * 9ull * 8ull * c->Ve));
-  // The FP64 copy, and with room for it the fixed-point copy; a field that does
-  // not pass fx_field keeps the FP64 operator.  No lattice is too small for it
-  // (2^4, 8 sites a parity: M^dag M call 27 us, 42 with the FP64 form and its
-  // copies between layouts; NPR contraction 50 and 60; FP64 CG 0.5 and 0.8 ms).
-  FieldCheck check = {0, 1};
-  c->fx_ok = false;
-  if (c->fx_mode && c->links_fx.ensure(cplx_bytes(PFX) * 9ull * 8ull * c->Ve) == cudaSuccess) {
+  c->have_links = c->fx_ok = false;
+  const double2 *canon = reinterpret_cast<const double2 *>(c->links_canon.p);
+  bool fx = false;
+  if (c->fx_mode) {
+    FieldCheck check;
     CK(c->defect.ensure(sizeof(FieldCheck)));
     CK(cudaMemsetAsync(c->defect.p, 0, sizeof(FieldCheck), c->stream));
-    CK(launch_pack_links_fx(reinterpret_cast<const double2 *>(c->links_canon.p), (double2 *)c->links64.p,
-                            (int4 *)c->links_fx.p, c->g, (FieldCheck *)c->defect.p, c->stream));
+    CK(launch_pack_links_fx(canon, (int4 *)c->links64.p, c->g, (FieldCheck *)c->defect.p, c->stream));
     CK(cudaMemcpyAsync(&check, c->defect.p, sizeof check, cudaMemcpyDeviceToHost, c->stream));
-  } else {
-    cudaGetLastError();
-    CK(launch_pack_links(P64, 0, reinterpret_cast<const double2 *>(c->links_canon.p), c->links64.p, c->g,
-                         c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    fx = fx_field(check, 4 * c->V);
+  }
+  if (!fx) {
+    CK(launch_pack_links(P64, 0, canon, c->links64.p, c->g, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
   }
   for (int p = 0; p < 4; ++p) c->lo_ok[p][0] = c->lo_ok[p][1] = c->tile_ok[p][0] = c->tile_ok[p][1] = false;
   c->have_links = true;
+  c->fx_ok = fx;
   c->w.drop_graph();  // the graph holds link pointers of the reduced-precision copies
-  CK(cudaStreamSynchronize(c->stream));
-  c->fx_ok = fx_field(check, 4 * c->V);
   return STAG_OK;
 }
 

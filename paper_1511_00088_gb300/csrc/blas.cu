@@ -251,11 +251,11 @@ cudaError_t launch_pack_links(int LP, int recon, const double2 *src, void *dst, 
   return cudaErrorNotSupported;
 }
 
-// One thread per link: bound by memory (144 B read, 288 B written); the
+// One thread per link: bound by memory (144 B read, 144 B written); the
 // fixed-point split works on the FP64 bit patterns, as its conversions would
 // otherwise hold the FP64 pipe for longer than the copy takes.
-__global__ void __launch_bounds__(256) k_pack_links_fx(const double2 *__restrict__ src, double2 *__restrict__ dst64,
-                                                       int4 *__restrict__ dstfx, Geom g, FieldCheck *check) {
+__global__ void __launch_bounds__(256) k_pack_links_fx(const double2 *__restrict__ src, int4 *__restrict__ dst, Geom g,
+                                                       FieldCheck *check) {
   const long long V = 2ll * g.Ve;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   bool ok = true;
@@ -271,11 +271,10 @@ __global__ void __launch_bounds__(256) k_pack_links_fx(const double2 *__restrict
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
       const double2 w = src[i * 9 + e];
-      dst64[o + (long long)e * g.Ve] = w;
       const int hx = __double2hiint(w.x), hy = __double2hiint(w.y);
       ok = ok && (hx & 0x7fffffff) < 0x40000000 && (hy & 0x7fffffff) < 0x40000000;  // |.| < 2 (false for NaN)
       const Fx a = fx_link(hx, __double2loint(w.x)), b = fx_link(hy, __double2loint(w.y));
-      dstfx[o + (long long)e * g.Ve] = make_int4(a.h, a.l, b.h, b.l);
+      dst[o + (long long)e * g.Ve] = make_int4(a.h, a.l, b.h, b.l);
       u[e] = make_float2((float)a.h * 0x1p-29f, (float)b.h * 0x1p-29f);
     }
     ok = ok && near_unitary(u);
@@ -284,9 +283,8 @@ __global__ void __launch_bounds__(256) k_pack_links_fx(const double2 *__restrict
   check_link(check, ok, nsmall);
 }
 
-cudaError_t launch_pack_links_fx(const double2 *src, double2 *dst64, int4 *dstfx, Geom g, FieldCheck *check,
-                                 cudaStream_t st) {
-  k_pack_links_fx<<<nblk(8ll * g.Ve, 256), 256, 0, st>>>(src, dst64, dstfx, g, check);
+cudaError_t launch_pack_links_fx(const double2 *src, int4 *dst, Geom g, FieldCheck *check, cudaStream_t st) {
+  k_pack_links_fx<<<nblk(8ll * g.Ve, 256), 256, 0, st>>>(src, dst, g, check);
   return cudaGetLastError();
 }
 

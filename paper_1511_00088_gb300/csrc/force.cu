@@ -13,9 +13,10 @@
 
 namespace stag {
 
-// one thread per link (mu, lexicographic site); X, Y in the device SoA layout
+// one thread per link (mu, lexicographic site); X, Y in the device SoA layout,
+// links [4][V][3][3]
 __global__ void k_force(const Geom g, const double2 *__restrict__ X, const double2 *__restrict__ Y,
-                        const void *links64, double2 *__restrict__ grad, double *__restrict__ lie,
+                        const double2 *__restrict__ links, double2 *__restrict__ grad, double *__restrict__ lie,
                         double scale) {
   const long long V = 2ll * g.Ve;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -70,8 +71,7 @@ __global__ void k_force(const Geom g, const double2 *__restrict__ X, const doubl
       for (int b = 0; b < 3; ++b) G[3 * a + b] = make_double2(K[3 * b + a].x, -K[3 * b + a].y);  // K^dag
   }
   if (lie) {
-    double u[18];
-    load_link<P64, 0>(links64, g.Ve, par, mu, s, u);
+    const double2 *u = links + i * 9;
     double2 M[9];  // M = U K
 #pragma unroll
     for (int a = 0; a < 3; ++a)
@@ -80,7 +80,7 @@ __global__ void k_force(const Geom g, const double2 *__restrict__ X, const doubl
         double re = 0.0, im = 0.0;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-          const double ur = u[2 * (3 * a + k)], ui = u[2 * (3 * a + k) + 1];
+          const double ur = u[3 * a + k].x, ui = u[3 * a + k].y;
           re += ur * K[3 * k + b].x - ui * K[3 * k + b].y;
           im += ur * K[3 * k + b].y + ui * K[3 * k + b].x;
         }
@@ -100,10 +100,10 @@ __global__ void k_force(const Geom g, const double2 *__restrict__ X, const doubl
   }
 }
 
-cudaError_t launch_force(Geom g, const double2 *X, const double2 *Y, const void *links64, double2 *grad,
+cudaError_t launch_force(Geom g, const double2 *X, const double2 *Y, const double2 *links, double2 *grad,
                          double *lie, double scale, cudaStream_t st) {
   const long long n = 8ll * g.Ve;
-  k_force<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(g, X, Y, links64, grad, lie, scale);
+  k_force<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(g, X, Y, links, grad, lie, scale);
   return cudaGetLastError();
 }
 

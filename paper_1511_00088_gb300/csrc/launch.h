@@ -152,9 +152,8 @@ cudaError_t launch_convert_vec(int PIN, int POUT, VecArg src, VecArg dst, int ns
                                cudaStream_t st);
 cudaError_t launch_pack_links(int LP, int recon, const double2 *src, void *dst, Geom g,
                               cudaStream_t st);
-// the FP64 (dst64) and fixed-point (dstfx) copies; *check (device) zeroed before
-cudaError_t launch_pack_links_fx(const double2 *src, double2 *dst64, int4 *dstfx, Geom g, FieldCheck *check,
-                                 cudaStream_t st);
+// the fixed-point copy; *check (device) zeroed before
+cudaError_t launch_pack_links_fx(const double2 *src, int4 *dst, Geom g, FieldCheck *check, cudaStream_t st);
 // the tiled site-owned copy (LP = P32, P16 or PBF); dst already zeroed
 cudaError_t launch_pack_links_tiled(int LP, int recon, const double2 *src, void *dst, Geom g, int ntile,
                                     cudaStream_t st);
@@ -177,7 +176,7 @@ cudaError_t launch_hyp(const int dims[4], const double2 *U, const double alpha[3
 
 // k_force over all 4 V links (force.cu): X even, Y = D_oe X odd (device SoA,
 // FP64); grad [4][V][3][3] complex and/or lie [4][V][8] (either may be null)
-cudaError_t launch_force(Geom g, const double2 *X, const double2 *Y, const void *links64, double2 *grad,
+cudaError_t launch_force(Geom g, const double2 *X, const double2 *Y, const double2 *links, double2 *grad,
                          double *lie, double scale, cudaStream_t st);
 // S = 2 Re<phi, x> - Re<x, ax> over Ve sites of one system (FP64 SoA), in
 // double-word arithmetic and a fixed order: part holds 2 action_blocks(Ve)

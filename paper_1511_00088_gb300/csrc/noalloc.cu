@@ -25,7 +25,7 @@
 #include "stag.h"
 
 namespace stag {
-int ctx_fp64_links(const stag_ctx *c, const void **links, cudaStream_t *stream);
+int ctx_fp64_links(const stag_ctx *c, const double2 **links, cudaStream_t *stream);
 void ctx_set_error(stag_ctx *c, const char *msg);
 Geom ctx_geom(const stag_ctx *c);
 int ctx_device(const stag_ctx *c);
@@ -74,8 +74,19 @@ __device__ __forceinline__ void na_store(double2 *v, int s, const double (&x)[6]
   for (int c = 0; c < 3; ++c) v[(long long)s * 3 + c] = make_double2(x[2 * c], x[2 * c + 1]);
 }
 
-// D applied at output site s of parity P to the ABI-layout vector `in` (FP64)
-__device__ __forceinline__ void na_hop_sum(const Geom &g, const void *links, int P, int s, const double2 *in,
+// a link of the canonical field
+__device__ __forceinline__ void na_link(const double2 *links, long long i, double (&u)[18]) {
+#pragma unroll
+  for (int e = 0; e < 9; ++e) {
+    const double2 w = __ldg(links + i * 9 + e);
+    u[2 * e] = w.x;
+    u[2 * e + 1] = w.y;
+  }
+}
+
+// D applied at output site s of parity P to the ABI-layout vector `in` (FP64);
+// links [4][V][3][3]
+__device__ __forceinline__ void na_hop_sum(const Geom &g, const double2 *links, int P, int s, const double2 *in,
                                            double (&acc)[6]) {
   int x[4];
   site_coords(g, P, s, x);
@@ -83,6 +94,9 @@ __device__ __forceinline__ void na_hop_sum(const Geom &g, const void *links, int
 #pragma unroll
   for (int i = 0; i < 6; ++i) acc[i] = 0.0;
   int eta_bits = 0;
+  const long long V = 2ll * g.Ve;
+  const long long lex = x[0] + (long long)g.L0 * (x[1] + (long long)g.L1 * (x[2] + (long long)g.L2 * x[3]));
+  long long str = 1;
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) {
     const double eta = (eta_bits & 1) ? -1.0 : 1.0;
@@ -99,17 +113,18 @@ __device__ __forceinline__ void na_hop_sum(const Geom &g, const void *links, int
       if (x[3] == 0) bb = -bb;
     }
     double u[18], v[6];
-    load_link<P64, 0>(links, g.Ve, P, mu, s, u);
+    na_link(links, mu * V + lex, u);
     na_load(in, sf, v);
     mv_acc(u, v, bf, acc);
-    load_link<P64, 0>(links, g.Ve, 1 - P, mu, sb, u);
+    na_link(links, mu * V + lex + (xb[mu] - x[mu]) * str, u);
     na_load(in, sb, v);
     mvdag_acc(u, v, -bb, acc);
+    str *= Ls[mu];
   }
 }
 
 // t_odd = D_oe in_even
-__global__ void __launch_bounds__(NA_BT) k_na_doe(const Geom g, const void *links, const double2 *in,
+__global__ void __launch_bounds__(NA_BT) k_na_doe(const Geom g, const double2 *links, const double2 *in,
                                                   double2 *t) {
   const int s = blockIdx.x * NA_BT + threadIdx.x;
   if (s >= g.Ve) return;
@@ -120,7 +135,7 @@ __global__ void __launch_bounds__(NA_BT) k_na_doe(const Geom g, const void *link
 
 // out_even = m4 in - D_eo t; dot = sum Re<in, out> (FP64, fixed-order reduction
 // through the static scratch: ticket at offset 0, partials at NA_TICKET_BYTES)
-__global__ void __launch_bounds__(NA_BT) k_na_deo_dot(const Geom g, const void *links, double m4,
+__global__ void __launch_bounds__(NA_BT) k_na_deo_dot(const Geom g, const double2 *links, double m4,
                                                       const double2 *in, const double2 *t, double2 *out,
                                                       double *dot, unsigned char *scratch) {
   unsigned *ticket = reinterpret_cast<unsigned *>(scratch);
@@ -205,7 +220,7 @@ extern "C" int stag_mdagm_dot_noalloc(stag_ctx *ctx, double mass, const double *
     ctx_set_error(ctx, "stag_mdagm_dot_noalloc: every pointer must be device memory of the context's GPU");
     return STAG_ERR_ARG;
   }
-  const void *links = nullptr;
+  const double2 *links = nullptr;
   cudaStream_t st;
   if (ctx_fp64_links(ctx, &links, &st) != STAG_OK) {
     ctx_set_error(ctx, "no gauge field: call stag_links_upload first");

@@ -1598,10 +1598,8 @@ __global__ void k_pack_links(const double2 *__restrict__ src, void *dst, Geom g)
   }
 }
 
-// the FP64 and the fixed-point copies of a gauge field in one pass over it, and
-// what decides whether the latter is used (fx_field)
-__global__ void k_pack_links_fx(const double2 *__restrict__ src, double2 *__restrict__ dst64,
-                                int4 *__restrict__ dstfx, Geom g, FieldCheck *check);
+// the fixed-point copy of a gauge field, and what decides whether it is used (fx_field)
+__global__ void k_pack_links_fx(const double2 *__restrict__ src, int4 *__restrict__ dst, Geom g, FieldCheck *check);
 
 // tiled site-owned copy of the links (see the layout notes at the top): one
 // thread per (parity, site, slot); dst zeroed beforehand (the tail of the last

@@ -7,6 +7,7 @@ from paper_1511_00088_gb300 import stag, synth
 
 pytestmark = pytest.mark.gpu
 
+
 @pytest.fixture(scope="module", autouse=True)
 def _built():
     from paper_1511_00088_gb300 import build
@@ -33,3 +34,30 @@ def test_a_solve_that_does_not_fit_can_be_repeated():
         for m, y, t in zip((1.0, 2.0), xs, tr):
             r = b - ctx.mdagm(y, m)
             assert torch.linalg.norm(r) <= 1.001e-10 * torch.linalg.norm(b) and t <= 1e-10
+
+
+L = (16, 16, 16, 32)
+FIELD = 4 * synth.volume(L) * 144  # bytes of a gauge field
+SLACK = 8 << 20                    # the driver's allocation granularity
+
+
+def used():
+    torch.cuda.synchronize()
+    free, total = torch.cuda.mem_get_info()
+    return total - free
+
+
+@pytest.mark.parametrize("scale", [1.0, 3.0])
+def test_upload_holds_two_copies(scale):
+    U = scale * synth.random_links_device(L, 0.4, 1401)
+    x = torch.from_numpy(synth.gaussian_vector(synth.volume(L) // 2, 1402)).cuda()
+    with stag.Context((4, 4, 4, 4)) as ctx:  # modules loaded
+        ctx.links_upload(synth.random_links((4, 4, 4, 4), 0.4, 1))
+    before = used()
+    with stag.Context(L) as ctx:
+        ctx.links_upload(U)
+        assert used() - before <= 2 * FIELD + SLACK
+        held = used()
+        g, f = ctx.force(x, grad=False, lie=True)  # needs no copy of its own
+        del g
+        assert used() - held <= f.numel() * 8 + 3 * x.numel() * 16 + SLACK
