@@ -236,7 +236,6 @@ struct stag_ctx {
   VecBuf full_e, full_o, full_x;  // full-lattice solve: halves of the sources, odd half of a solution
   DevBuf red;                     // block sums of the action's reduction
   DevBuf hyp_b, hyp_t, hyp_io;    // HYP smearing: the two decorated levels, host staging
-  DevBuf hyp_u;                   // its thin links in fixed point
   DevBuf npr_f, npr_o;            // NPR contraction: staged fields, per-hypercube values and their sum
   VecBuf ms_p, ms_x;              // multi-shift CG: shifted directions and solutions (FP32)
   DevBuf ms_sh;                   // their ShiftState
@@ -2405,12 +2404,8 @@ int stag_hyp_smear(stag_ctx *c, const double alpha[3], const double *links_in, d
   }
   double2 *out = out_dev ? reinterpret_cast<double2 *>(links_out) : reinterpret_cast<double2 *>(c->hyp_io.p);
   CK(c->defect.ensure(sizeof(FieldCheck)));
-  void *fix = nullptr;  // without room for it: the FP64 form
-  if (c->fx_mode) {
-    if (c->hyp_u.ensure(bytes) == cudaSuccess) fix = c->hyp_u.p;
-    else cudaGetLastError();
-  }
-  CK(launch_hyp(c->dims, U, a, (double2 *)c->hyp_b.p, (double2 *)c->hyp_t.p, out, fix, (FieldCheck *)c->defect.p, c->stream));
+  CK(launch_hyp(c->dims, U, a, (double2 *)c->hyp_b.p, (double2 *)c->hyp_t.p, out,
+                c->fx_mode ? (FieldCheck *)c->defect.p : nullptr, c->stream));
   if (!out_dev) CK(cudaMemcpyAsync(links_out, c->hyp_io.p, bytes, cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   return STAG_OK;

@@ -421,12 +421,19 @@ struct HfxShared {
   float f[27][HFX_BT];
 };
 
-// the link's mix of c U and the staples in X, and its projection into Q; c = (h, l) limbs
-__device__ __forceinline__ bool smear_fx(const int4 *pu, long long V, Fx c, int q, int4 *X, int4 *Q, float *f) {
+// a thin link's element in fixed point
+__device__ __forceinline__ int4 thin_fx(const double2 &w) {
+  const Fx a = fx_link(__double2hiint(w.x), __double2loint(w.x)), b = fx_link(__double2hiint(w.y), __double2loint(w.y));
+  return make_int4(a.h, a.l, b.h, b.l);
+}
+
+// the mix of c U (U(k): its element k) and the staples in X, and its projection into Q; c = (h, l) limbs
+template <class Thin>
+__device__ __forceinline__ bool smear_fx(const Thin &U, Fx c, int q, int4 *X, int4 *Q, float *f) {
   const long long half = q > 0 ? 1ll << (q - 1) : 0ll;
 #pragma unroll 3
   for (int k = 0; k < 9; ++k) {
-    const int4 u = __ldg(pu + k * V);
+    const int4 u = U(k);
     FxAcc re, im;
     re.hh = re.cr = im.hh = im.cr = 0;
     fx_mac(re, u.x, u.y, c.h, c.l);
@@ -451,9 +458,9 @@ __global__ void __launch_bounds__(256) k_hyp_fix(long long V, const double2 *__r
       const double2 w = U[t * 9 + e];
       const int hx = __double2hiint(w.x), hy = __double2hiint(w.y);
       ok = ok && (hx & 0x7fffffff) < 0x40000000 && (hy & 0x7fffffff) < 0x40000000;
-      const Fx a = fx_link(hx, __double2loint(w.x)), b = fx_link(hy, __double2loint(w.y));
-      F[(mu * 9 + e) * V + i] = make_int4(a.h, a.l, b.h, b.l);
-      u[e] = make_float2((float)a.h * 0x1p-29f, (float)b.h * 0x1p-29f);
+      const int4 v = thin_fx(w);
+      F[(mu * 9 + e) * V + i] = v;
+      u[e] = make_float2((float)v.x * 0x1p-29f, (float)v.z * 0x1p-29f);
     }
     ok = ok && near_unitary(u);
     nsmall = small_parts(u);
@@ -464,7 +471,7 @@ __global__ void __launch_bounds__(256) k_hyp_fix(long long V, const double2 *__r
 struct HypFx {
   FLat f;
   long long V;
-  const int4 *U;  // [4][9][V]
+  const double2 *U;  // the thin links, canonical
   FieldCheck *check;
   Fx c;
   int q;
@@ -511,7 +518,11 @@ __global__ void __launch_bounds__(HFX_BT, 3) k_hyp12_fx(const HypFx h, const int
     for (int neg = 0; neg < 2; ++neg)
       staple_fx(A + (neg ? dn : i), B + (neg ? dn : up), A + (neg ? dnmu : imu), (int)V, neg, X);
   }
-  if (!smear_fx(h.U + (long long)mu * 9 * V + i, V, h.c, h.q, X, Q, &hsh->f[0][threadIdx.x])) h.check->bad = 1;
+  // level 1 reads the thin links in fixed point anyway (src)
+  const int4 *pf = src + (long long)mu * 9 * V + i;
+  const double2 *pu = h.U + ((long long)mu * V + i) * 9;
+  auto thin = [&](int k) { return LEVEL == 1 ? __ldg(pf + k * V) : thin_fx(__ldg(pu + k)); };
+  if (!smear_fx(thin, h.c, h.q, X, Q, &hsh->f[0][threadIdx.x])) h.check->bad = 1;
   if (i0 >= h.V) return;
 #pragma unroll
   for (int k = 0; k < 9; ++k) dst[((long long)pr * 9 + k) * V + i] = Q[k * HFX_BT];
@@ -541,7 +552,11 @@ __global__ void __launch_bounds__(HFX_BT, 3) k_hyp3_fx(const HypFx h, const int4
     for (int neg = 0; neg < 2; ++neg)
       staple_fx(A + (neg ? dn : i), B + (neg ? dn : up), A + (neg ? dnmu : imu), (int)V, neg, X);
   }
-  const bool ok = smear_fx(h.U + (long long)mu * 9 * V + i, V, h.c, h.q, X, Q, &hsh->f[0][threadIdx.x]);
+  // out may be the thin links' buffer: each thread reads its own link before it
+  // writes it, and those past the last site, whose link another thread writes, read none
+  const double2 *pu = h.U + ((long long)mu * V + i) * 9;
+  auto thin = [&](int k) { return i0 < V ? thin_fx(pu[k]) : make_int4(k % 4 == 0 ? 1 << FX_LO : 0, 0, 0, 0); };
+  const bool ok = smear_fx(thin, h.c, h.q, X, Q, &hsh->f[0][threadIdx.x]);
   if (i0 >= h.V) return;
   const double one = ok ? 0x1p-58 : __longlong_as_double(0x7ff8000000000000ll);
   double2 *o = out + ((long long)mu * V + i) * 9;
@@ -567,7 +582,7 @@ bool mix_of(double a, double w, int staples, Fx *c, int *q) {
 }  // namespace
 
 cudaError_t launch_hyp(const int dims[4], const double2 *U, const double alpha[3], double2 *Vb, double2 *Vt,
-                       double2 *out, void *fixU, FieldCheck *check, cudaStream_t st) {
+                       double2 *out, FieldCheck *check, cudaStream_t st) {
   Lat g;
   for (int k = 0; k < 4; ++k) g.L[k] = dims[k];
   g.V = (long long)dims[0] * dims[1] * dims[2] * dims[3];
@@ -576,7 +591,7 @@ cudaError_t launch_hyp(const int dims[4], const double2 *U, const double alpha[3
   int q[3];
   cudaError_t e = cudaSuccess;
   const FieldCheck *run = nullptr;
-  if (fixU != nullptr && g.V < (1ll << 27) && mix_of(alpha[2], alpha[2] / 2.0, 2, &c[0], &q[0]) &&
+  if (check != nullptr && g.V < (1ll << 27) && mix_of(alpha[2], alpha[2] / 2.0, 2, &c[0], &q[0]) &&
       mix_of(alpha[1], alpha[1] / 4.0, 4, &c[1], &q[1]) && mix_of(alpha[0], alpha[0] / 6.0, 6, &c[2], &q[2])) {
     for (const void *k : {(const void *)k_hyp12_fx<1>, (const void *)k_hyp12_fx<2>, (const void *)k_hyp3_fx}) {
       e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(HfxShared));
@@ -591,13 +606,14 @@ cudaError_t launch_hyp(const int dims[4], const double2 *U, const double alpha[3
     h.f.d1 = make_fastdiv((unsigned)dims[1]);
     h.f.d2 = make_fastdiv((unsigned)dims[2]);
     h.V = g.V;
-    h.U = reinterpret_cast<const int4 *>(fixU);
+    h.U = U;
+    int4 *fixU = reinterpret_cast<int4 *>(Vt);  // level 1's thin links, until level 2 writes Vt
     h.check = check;
-    k_hyp_fix<<<(unsigned)((4 * g.V + 255) / 256), 256, 0, st>>>(g.V, U, reinterpret_cast<int4 *>(fixU), check);
+    k_hyp_fix<<<(unsigned)((4 * g.V + 255) / 256), 256, 0, st>>>(g.V, U, fixU, check);
     const unsigned nb = (unsigned)((g.V + HFX_BT - 1) / HFX_BT);
     h.c = c[0];
     h.q = q[0];
-    k_hyp12_fx<1><<<dim3(nb, 12), HFX_BT, sizeof(HfxShared), st>>>(h, h.U, reinterpret_cast<int4 *>(Vb));
+    k_hyp12_fx<1><<<dim3(nb, 12), HFX_BT, sizeof(HfxShared), st>>>(h, fixU, reinterpret_cast<int4 *>(Vb));
     h.c = c[1];
     h.q = q[1];
     k_hyp12_fx<2><<<dim3(nb, 12), HFX_BT, sizeof(HfxShared), st>>>(h, reinterpret_cast<const int4 *>(Vb), reinterpret_cast<int4 *>(Vt));

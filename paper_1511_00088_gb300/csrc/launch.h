@@ -169,10 +169,9 @@ cudaError_t launch_npr(const int dims[4], const double2 *U, const int st[4], con
 
 // HYP smearing (hyp.cu): out [4][V][3][3] = the smeared links of U (same
 // layout; out may alias U); Vb, Vt scratch of 12 V links each; alpha = (a1, a2,
-// a3).  fixU: scratch of 4 V links for the fixed-point form with its *check
-// (device), or null: FP64 only
+// a3).  check: device memory for the fixed-point form, or null: FP64 only
 cudaError_t launch_hyp(const int dims[4], const double2 *U, const double alpha[3], double2 *Vb, double2 *Vt,
-                       double2 *out, void *fixU, FieldCheck *check, cudaStream_t st);
+                       double2 *out, FieldCheck *check, cudaStream_t st);
 
 // k_force over all 4 V links (force.cu): X even, Y = D_oe X odd (device SoA,
 // FP64); grad [4][V][3][3] complex and/or lie [4][V][8] (either may be null)

@@ -61,3 +61,12 @@ def test_upload_holds_two_copies(scale):
         g, f = ctx.force(x, grad=False, lie=True)  # needs no copy of its own
         del g
         assert used() - held <= f.numel() * 8 + 3 * x.numel() * 16 + SLACK
+
+
+def test_hyp_holds_two_levels():
+    U = synth.random_links_device(L, 0.4, 1411)
+    out = torch.empty_like(U)
+    before = used()
+    with stag.Context(L) as ctx:
+        ctx.hyp_smear(U, out=out)
+        assert used() - before <= 6 * FIELD + SLACK
