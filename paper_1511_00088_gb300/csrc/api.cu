@@ -31,6 +31,8 @@
 // that kernel and the updates.
 // Without conditional-node support the same kernel sequence runs eagerly, with
 // the host polling a device flag every few loop passes.
+#include <cuda.h>
+
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -208,6 +210,7 @@ struct stag_ctx {
   bool coop = false;   // the device runs cooperative launches
   int nsm = 0;
   int ps_mode = -1;    // k_cg_persist: -1 by rule, 0 never, else this form (STAG_PS)
+  signed char ps_fit[2][5] = {{-1, -1, -1, -1, -1}, {-1, -1, -1, -1, -1}};  // [recon][form]: an SM holds a block of it (-1 unknown)
   bool pdl = true;  // CG kernels launched as programmatic dependents of their predecessors
   bool fold = true;     // each CG kernel finishes its predecessor's reduction itself
   bool persist = true;  // CG kernels launched as one wave of resident blocks
@@ -803,8 +806,37 @@ size_t ps_sync_bytes(int nsys) {
   return (sizeof(unsigned long long) * 2 * PS_MAXB + sizeof(unsigned) * (PS_ASTRIDE + 2)) * (size_t)nsys + 2 * sizeof(int);
 }
 
+// SMs that the context's stream may use: all, or those of a green context's stream
+int stream_sms(const stag_ctx *c) {
+  typedef CUresult (*GetGreen)(CUstream, CUgreenCtx *);
+  typedef CUresult (*GetResource)(CUgreenCtx, CUdevResource *, CUdevResourceType);
+  struct Driver {
+    GetGreen green = nullptr;
+    GetResource resource = nullptr;
+    Driver() {
+      void *a = nullptr, *b = nullptr;
+      cudaDriverEntryPointQueryResult ra, rb;
+      if (cudaGetDriverEntryPointByVersion("cuStreamGetGreenCtx", &a, 12040, cudaEnableDefault, &ra) == cudaSuccess &&
+          cudaGetDriverEntryPointByVersion("cuGreenCtxGetDevResource", &b, 12040, cudaEnableDefault, &rb) == cudaSuccess &&
+          ra == cudaDriverEntryPointSuccess && rb == cudaDriverEntryPointSuccess) {
+        green = (GetGreen)a;
+        resource = (GetResource)b;
+      }
+      cudaGetLastError();
+    }
+  };
+  static const Driver drv;
+  CUgreenCtx g = nullptr;
+  CUdevResource r;
+  if (c->stream != nullptr && drv.green && drv.green((CUstream)c->stream, &g) == CUDA_SUCCESS && g != nullptr &&
+      drv.resource(g, &r, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS && r.sm.smCount > 0 && (int)r.sm.smCount < c->nsm)
+    return (int)r.sm.smCount;
+  return c->nsm;
+}
+
 // The persistent form (k_cg_persist) of a workspace: lanes a site and blocks, or
-// form 0 where the two-kernel forms are the better ones.  Measured on 152 SMs, us per iteration of a whole solve (persistent / two kernels):
+// form 0 where the two-kernel forms are the better ones, or its blocks, which wait
+// for one another, would not all be resident.  Measured on 152 SMs, us per iteration of a whole solve (persistent / two kernels):
 //   lanes: 4 while a group's warps hold all sites at once (17 280 sites a parity: 4 lanes
 //   7.3, 2 lanes 8.2 / 17.8; 24 576: 9.0, 8.3 / 16.3); 2 while two rounds do (49 152: 2 lanes 11.7,
 //   1 lane 12.6 / 23.3; 98 304: 18.6, 17.1 / 28.0); else 1;
@@ -814,23 +846,32 @@ size_t ps_sync_bytes(int nsys) {
 //   several: by all systems' sites an SM, 2600 with reconstruct-12 (16^3 x 32 x 6: 50.3 / 68.2,
 //   12^3 x 24 x 12: 41.6 / 42.8; 20^3 x 64 x 2: 81.5 / 78.5), 1300 with full links (16^3 x 32 x 3:
 //   30.1 / 34.1; x 6: 58.0 / 51.2).
-void choose_persist(const stag_ctx *c, int LP, int VP, int nsys, int ms, int *form, int *blocks) {
+void choose_persist(stag_ctx *c, int LP, int VP, int nsys, int ms, int *form, int *blocks) {
   *form = *blocks = 0;
   if (!c->coop || c->ps_mode == 0 || LP != P32 || VP != P32 || ms != 0) return;
-  int nb = c->nsm / nsys;
+  const int nsm = stream_sms(c);
+  int nb = nsm / nsys;
   if (nb > PS_MAXB) nb = PS_MAXB;
   if (nb < 1) return;
   const int Ve = c->Ve, rc = (c->flags & STAG_RECON12) ? 1 : 0;
   int f = c->ps_mode;
   if (f < 0) {
     const double lb = 8.0 * (rc ? 6 : 9) * 8.0 * Ve, set_aside = c->l2_max_persist ? (double)c->l2_max_persist : 80e6;
-    if (nsys == 1 ? lb > (rc ? 1.25 : 1.0) * set_aside : (double)nsys * Ve > (rc ? 2600.0 : 1300.0) * c->nsm) return;
+    if (nsys == 1 ? lb > (rc ? 1.25 : 1.0) * set_aside : (double)nsys * Ve > (rc ? 2600.0 : 1300.0) * nsm) return;
     f = Ve <= nb * cg_persist_sites(4) ? 4 : Ve <= 2 * nb * cg_persist_sites(2) ? 2 : 1;
   }
+  if (f != 1 && f != 2 && f != 4) return;
+  signed char &fit = c->ps_fit[rc][f];
+  if (fit < 0) {
+    int per_sm = 0;
+    fit = cg_persist_fit(rc, f, &per_sm) == cudaSuccess && per_sm >= 1;
+    cudaGetLastError();
+  }
+  if (!fit) return;
   const int per = cg_persist_sites(f);
   const int full = (Ve + per - 1) / per;
   *form = f;
-  *blocks = (long long)nsys * full < c->nsm ? nsys * full : c->nsm;
+  *blocks = (long long)nsys * full < nsm ? nsys * full : nsm;
 }
 
 int work_fill(stag_ctx *c, int nsys, int precision, int ms);
@@ -856,7 +897,8 @@ int work_fill(stag_ctx *c, int nsys, int precision, int ms) {
   int psf = 0, psn = 0;
   choose_persist(c, prec, VP, nsys, ms, &psf, &psn);
   const int op64 = lp_for(c, P64);
-  if (w.nsys == nsys && w.prec == prec && w.VP == VP && w.recon == recon && w.ps_form == psf && w.op64 == op64)
+  if (w.nsys == nsys && w.prec == prec && w.VP == VP && w.recon == recon && w.ps_form == psf && w.ps_blocks == psn &&
+      w.op64 == op64)
     return STAG_OK;
   w.drop_graph();
   w.op64 = op64;
@@ -2043,10 +2085,11 @@ int ragged_impl(const stag_solve_desc *d, int n, double tol, int maxiter, int pr
       std::stable_sort(order.begin(), order.end(),
                        [&](int p, int q) { return d[p].ctx->w.ps_blocks < d[q].ctx->w.ps_blocks; });
       std::vector<cudaGraphNode_t> before, wave;
+      const int sms = stream_sms(c0);
       int held = 0;
       for (int q = 0; q < n && st == STAG_OK; ++q) {
         const int i = order[q], nb = d[i].ctx->w.ps_form ? d[i].ctx->w.ps_blocks : 0;
-        if (nb > 0 && held > 0 && held + nb > c0->nsm) {
+        if (nb > 0 && held > 0 && held + nb > sms) {
           before.swap(wave);
           wave.clear();
           held = 0;

@@ -663,17 +663,30 @@ __global__ void k_ps_map(const PsArgs a, int nblocks, int full) {
   }
 }
 
-// launch k, or (kptr) return it.  The limit of a kernel's dynamic shared memory
-// belongs to the process, not to the launch: it is set to `most`, all that any
-// launch of k asks for, as another thread's context may be between its own
-// setting and its launch.
-cudaError_t ps_launch(void (*k)(PsArgs), unsigned smem, unsigned most, int nblocks, cudaStream_t st, const PsArgs &a,
-                      const void **kptr) {
-  if (kptr) {
-    *kptr = (const void *)k;
-    return cudaSuccess;
+// A kernel and the most dynamic shared memory that any launch of it asks for.
+// That limit belongs to the process, not to the launch: it is always set to
+// `most`, as another thread's context may be between its own setting and its launch.
+struct PsKernel {
+  void (*k)(PsArgs) = nullptr;
+  unsigned most = 0;
+};
+constexpr unsigned ps_link_bytes(int recon) { return (recon ? 6u : 9u) * 32u * 8u; }  // one link of 32 lanes
+// of a chunk (32 / lanes sites)
+constexpr unsigned ps_chunk_bytes(int recon, int lanes) { return (unsigned)(8 / lanes) * ps_link_bytes(recon); }
+PsKernel ps_kernel(int recon, int lanes) {
+  PsKernel p;
+  if (lanes == 1) {
+    p.k = recon ? k_cg_persist_sm<1> : k_cg_persist_sm<0>;
+    p.most = PS_CW * (unsigned)ps_staged_links(recon) * ps_link_bytes(recon);
+  } else if (lanes == 2 || lanes == 4) {
+    p.k = lanes == 2 ? (recon ? k_cg_persist<1, 2> : k_cg_persist<0, 2>) : (recon ? k_cg_persist<1, 4> : k_cg_persist<0, 4>);
+    p.most = PS_SMEM / ps_chunk_bytes(recon, lanes) * ps_chunk_bytes(recon, lanes);
   }
-  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+  return p;
+}
+
+cudaError_t ps_launch(const PsKernel &p, unsigned smem, int nblocks, cudaStream_t st, const PsArgs &a) {
+  const cudaError_t e = cudaFuncSetAttribute(p.k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.most);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.dynamicSmemBytes = smem;
@@ -695,37 +708,37 @@ cudaError_t ps_launch(void (*k)(PsArgs), unsigned smem, unsigned most, int nbloc
   }
   cfg.attrs = at;
   cfg.numAttrs = n;
-  return cudaLaunchKernelEx(&cfg, k, a);
+  return cudaLaunchKernelEx(&cfg, p.k, a);
 }
 
 }  // namespace
 
 int cg_persist_sites(int lanes) { return 32 * PS_CW / lanes; }
 
-cudaError_t launch_cg_persist(int recon, int lanes, int nblocks, cudaStream_t st, PsArgs a, const void **kptr) {
-  if (!kptr) {
-    k_ps_map<<<1, 32, 0, st>>>(a, nblocks, (a.g.Ve + cg_persist_sites(lanes) - 1) / cg_persist_sites(lanes));
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  const unsigned link = (recon ? 6u : 9u) * 32u * 8u;  // bytes of one link of 32 lanes
-  if (lanes == 1) {
-    const unsigned bytes = PS_CW * (unsigned)ps_staged_links(recon) * link;
-    return ps_launch(recon ? k_cg_persist_sm<1> : k_cg_persist_sm<0>, bytes, bytes, nblocks, st, a, kptr);
-  }
+cudaError_t cg_persist_fit(int recon, int lanes, int *blocks_per_sm) {
+  *blocks_per_sm = 0;
+  const PsKernel p = ps_kernel(recon, lanes);
+  if (p.k == nullptr) return cudaErrorNotSupported;
+  const cudaError_t e = cudaFuncSetAttribute(p.k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.most);
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, p.k, PS_BT, p.most);
+}
+
+cudaError_t launch_cg_persist(int recon, int lanes, int nblocks, cudaStream_t st, PsArgs a) {
+  const PsKernel p = ps_kernel(recon, lanes);
+  if (p.k == nullptr) return cudaErrorNotSupported;
+  k_ps_map<<<1, 32, 0, st>>>(a, nblocks, (a.g.Ve + cg_persist_sites(lanes) - 1) / cg_persist_sites(lanes));
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  if (lanes == 1) return ps_launch(p, p.most, nblocks, st, a);
   // shared memory for the links of as many chunks as fit, at most all of a block's
   const int sites = 32 / lanes, nall = (a.g.Ve + sites - 1) / sites;
-  const unsigned bytes = (unsigned)(8 / lanes) * link;
+  const unsigned bytes = ps_chunk_bytes(recon, lanes);
   const int nbg = a.nsys > 0 && nblocks >= a.nsys ? nblocks / a.nsys : 1;  // while all systems run
   const int most = 2 * ((nall + nbg - 1) / nbg);
-  a.nres = (int)(PS_SMEM / bytes);
+  a.nres = (int)(p.most / bytes);
   if (a.nres > most) a.nres = most;
-#define STAG_PS(R_, L_) \
-  if (recon == R_ && lanes == L_) \
-    return ps_launch(k_cg_persist<R_, L_>, (unsigned)a.nres * bytes, PS_SMEM / bytes * bytes, nblocks, st, a, kptr);
-  STAG_PS(0, 4) STAG_PS(1, 4) STAG_PS(0, 2) STAG_PS(1, 2)
-#undef STAG_PS
-  return cudaErrorNotSupported;
+  return ps_launch(p, (unsigned)a.nres * bytes, nblocks, st, a);
 }
 
 }  // namespace stag

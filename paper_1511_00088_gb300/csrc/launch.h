@@ -126,8 +126,8 @@ struct PsArgs {
   size_t l2_bytes;
   float l2_hit;
 };
-cudaError_t launch_cg_persist(int recon, int lanes, int nblocks, cudaStream_t st, PsArgs a,
-                              const void **kptr = nullptr);
+cudaError_t launch_cg_persist(int recon, int lanes, int nblocks, cudaStream_t st, PsArgs a);
+cudaError_t cg_persist_fit(int recon, int lanes, int *blocks_per_sm);  // blocks of it an SM holds
 int cg_persist_sites(int lanes);  // sites of a block's warps at a time
 
 cudaError_t launch_accum_x(int RP, int NS, int nblocks, cudaStream_t st, const BlasArgs &a);

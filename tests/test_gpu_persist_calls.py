@@ -1,5 +1,6 @@
 """Calls around the persistent CG kernel that the two-kernel form answers: several contexts at once, sources near the
 ends of FP32's range, streams with part of the GPU, switches at their defaults, a form asked for after an upload."""
+import ctypes
 import threading
 
 import numpy as np
@@ -95,3 +96,48 @@ def test_a_switch_at_its_default_changes_nothing(switch, monkeypatch):
             ctx.cg_solve([b], [0.3])
             got[value] = ctx.solve_form()["kernels"]
     assert got == {"": "k_cg_persist", "1": "k_cg_persist", "0": "k_dslash"}
+
+
+class PartOfTheGpu:
+    """A stream that may use some 16 SMs of the GPU (a green context), by the driver API."""
+
+    def __enter__(self):
+        torch.cuda.init()
+        torch.cuda.synchronize()
+        cu = ctypes.CDLL("libcuda.so.1")
+
+        def call(name, *args):
+            assert getattr(cu, name)(*args) == 0, name
+        self.call, size = call, 1024  # of a resource, more than it needs
+        whole, part, rest = (ctypes.create_string_buffer(size) for _ in range(3))
+        dev, n = ctypes.c_int(), ctypes.c_uint(1)
+        desc, self.green, self.stream = ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_void_p()
+        call("cuDeviceGet", ctypes.byref(dev), torch.cuda.current_device())
+        call("cuDeviceGetDevResource", dev, whole, 1)  # the SMs
+        call("cuDevSmResourceSplitByCount", part, ctypes.byref(n), whole, rest, 0, 16)
+        call("cuDevResourceGenerateDesc", ctypes.byref(desc), part, 1)
+        call("cuGreenCtxCreate", ctypes.byref(self.green), desc, dev, 1)
+        call("cuGreenCtxStreamCreate", ctypes.byref(self.stream), self.green, 1, 0)
+        return self.stream.value
+
+    def __exit__(self, *_):
+        torch.cuda.synchronize()
+        self.call("cuStreamDestroy_v2", self.stream)
+        self.call("cuGreenCtxDestroy", self.green)
+
+
+@pytest.mark.parametrize("L", [(8, 8, 8, 8), (12, 12, 12, 24), (16, 16, 16, 32)])
+@pytest.mark.parametrize("eager", ["1", "0"])
+def test_a_stream_with_part_of_the_gpu(L, eager, monkeypatch):
+    """As many blocks as the stream's SMs hold."""
+    monkeypatch.setenv("STAG_EAGER", eager)
+    U = synth.random_links(L, 0.4, 1351)
+    b = synth.gaussian_vector(synth.volume(L) // 2, 1352)
+    with PartOfTheGpu() as stream:
+        for masses in ([0.3], [0.3, 0.5]):
+            with stag.Context(L, stream=stream) as ctx:
+                ctx.links_upload(U)
+                xs = ctx.cg_solve([b], masses)[0]
+                ctx.solve_form()
+            for m, x in zip(masses, xs):
+                assert oracle.true_residual(L, U, m, b, x) <= 1e-10
