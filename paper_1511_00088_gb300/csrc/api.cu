@@ -217,7 +217,8 @@ struct stag_ctx {
   int tma_modes = 0b101;  // link paths (bit t: DsArgs::tma = t) the tuner may choose for one system
   // STAG_TEST_WAIT_GIVEUP=1: in the solve loop, the bounded waits (of the
   // shared-memory link path, of the persistent kernel's blocks for one another)
-  // give up at once (tests of the failure path)
+  // give up at once (tests of the failure path); 2: the latter only, and such a
+  // solve is run again (two_kernel_again)
   int wait_giveup = 0;
   // L2 residency of the inner-precision links during a solve: the CG kernels
   // mark them as an access-policy window whose lines persist in L2 (the rest
@@ -1210,7 +1211,7 @@ int enqueue_main(stag_ctx *c, cudaStream_t s, const Ctl &ctl) {
   a.pdl = c->pdl ? 1 : 0;
   if (w.tma) CKS(links_tile_for(c, w.prec, &w.links_tile));
   a.tma = w.tma;
-  a.wait_giveup = c->wait_giveup;
+  a.wait_giveup = c->wait_giveup == 1;
   a.links_tile = w.links_tile;
   a.ntile = link_tiles(c->Ve);
   set_l2_window(c, w.prec, w.tma, w.l2p, a);
@@ -1272,7 +1273,7 @@ int enqueue_pass(stag_ctx *c, cudaStream_t s, const Ctl &ctl, int unroll) {
     p.counted = p.arrived + (long long)PS_ASTRIDE * w.nsys;
     p.map = (int *)(p.counted + w.nsys);
     p.nsys = w.nsys;
-    p.giveup = c->wait_giveup;
+    p.giveup = c->wait_giveup != 0;
     DsArgs win = ds_base(c);
     set_l2_window(c, w.prec, 0, w.l2p, win);
     p.l2_base = win.l2_base;
@@ -1304,7 +1305,7 @@ int enqueue_pass(stag_ctx *c, cudaStream_t s, const Ctl &ctl, int unroll) {
   a.pdl = c->pdl ? 1 : 0;
   if (w.tma) CKS(links_tile_for(c, w.prec, &w.links_tile));
   a.tma = w.tma;
-  a.wait_giveup = c->wait_giveup;
+  a.wait_giveup = c->wait_giveup == 1;
   a.links_tile = w.links_tile;
   a.ntile = link_tiles(c->Ve);
   set_l2_window(c, w.prec, w.tma, w.l2p, a);
@@ -1632,10 +1633,34 @@ int solve_status(stag_ctx *c, int iters[], double true_res[]) {
 
 int solve_run(stag_ctx *c, int maxiter);
 
+// A persistent kernel whose blocks gave up waiting for one another (work of
+// others held part of the GPU for seconds) says nothing about the systems: the
+// solve is run again in the two-kernel form, which waits for nothing, from the
+// sources still in w.b64.  The context returns to the persistent form after it.
+struct TwoKernel {
+  stag_ctx *c;
+  int mode;
+  explicit TwoKernel(stag_ctx *ctx) : c(ctx), mode(ctx->ps_mode) { c->ps_mode = 0; }
+  ~TwoKernel() { c->ps_mode = mode; }
+};
+bool gave_up(const stag_ctx *c, int status) {
+  return status == STAG_ERR_TIMEOUT && c->w.ps_form != 0 && c->wait_giveup != 1;
+}
+int two_kernel_again(stag_ctx *c, int nsys, const double masses[], int nmass, double tol, int maxiter, int prec,
+                     const FullRef *full) {
+  TwoKernel hold(c);
+  CKS(work_prepare(c, nsys, prec));
+  CKS(solve_start(c, masses, nmass, tol, maxiter, full));
+  return solve_run(c, maxiter);
+}
+
 int solve_impl(stag_ctx *c, const double *const src[], int nrhs, const double masses[], int nmass,
                double tol, int maxiter, int prec, double *const x[], int iters[], double true_res[]) {
   CKS(solve_stage(c, src, nrhs, masses, nmass, tol, maxiter, prec));
   CKS(solve_run(c, maxiter));
+  const int st = solve_finish(c, x, iters, true_res);
+  if (!gave_up(c, st)) return st;
+  CKS(two_kernel_again(c, nrhs * nmass, masses, nmass, tol, maxiter, prec, nullptr));
   return solve_finish(c, x, iters, true_res);
 }
 
@@ -1695,6 +1720,31 @@ int apply_m64(stag_ctx *c, int par_out, double m4, double scale, VecArg in, VecA
   return STAG_OK;
 }
 
+// a full-lattice solve's odd halves, solutions and statistics; its status
+int full_finish(stag_ctx *c, int nsys, const double masses[], int nmass, double *const x[], int iters[],
+                double true_res[]) {
+  Work &w = c->w;
+  const size_t full_bytes = sizeof(double) * 6ull * (size_t)c->V;
+  CK(cudaMemcpyAsync(w.h_st.p, w.st.p, sizeof(SysState) * nsys, cudaMemcpyDeviceToHost, c->stream));
+  CK(cudaMemcpyAsync(w.h_flags.p, w.flags.p, sizeof(int) * 8, cudaMemcpyDeviceToHost, c->stream));
+  // x_o = (b_o - D_oe x_e) / (2m), then both halves into the caller's full vector
+  for (int j = 0; j < nsys; ++j) {
+    const int r = j / nmass, k = j % nmass;
+    CKS(apply_m64(c, 1, 1.0, 1.0 / (2.0 * masses[k]), vec_slot(w.x64, j), vec_slot(c->full_o, r),
+                  c->full_x.arg()));
+    if (is_device_ptr(x[j])) {
+      CK(launch_merge_full(w.x64.arg(), j, c->full_x.arg(), 0, reinterpret_cast<double2 *>(x[j]), c->g,
+                           c->stream));
+    } else {
+      CK(c->stage_out.ensure(full_bytes));
+      CK(launch_merge_full(w.x64.arg(), j, c->full_x.arg(), 0, reinterpret_cast<double2 *>(c->stage_out.p), c->g,
+                           c->stream));
+      CK(cudaMemcpyAsync(x[j], c->stage_out.p, full_bytes, cudaMemcpyDeviceToHost, c->stream));
+    }
+  }
+  return solve_status(c, iters, true_res);
+}
+
 // The full-lattice equation M x = b, M = 2m + D, through the even-site CG:
 //   b_s = 2m b_e - D_eo b_o;  (4m^2 - D_eo D_oe) x_e = b_s;  x_o = (b_o - D_oe x_e) / (2m)
 // (all FP64 except the CG's inner iteration).  The CG's reference norm is
@@ -1734,24 +1784,10 @@ int solve_full_impl(stag_ctx *c, const double *const src[], int nrhs, const doub
   ref.bo = c->full_o.arg();
   CKS(solve_start(c, masses, nmass, tol, maxiter, &ref));
   CKS(solve_run(c, maxiter));
-  CK(cudaMemcpyAsync(w.h_st.p, w.st.p, sizeof(SysState) * nsys, cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaMemcpyAsync(w.h_flags.p, w.flags.p, sizeof(int) * 8, cudaMemcpyDeviceToHost, c->stream));
-  // x_o = (b_o - D_oe x_e) / (2m), then both halves into the caller's full vector
-  for (int j = 0; j < nsys; ++j) {
-    const int r = j / nmass, k = j % nmass;
-    CKS(apply_m64(c, 1, 1.0, 1.0 / (2.0 * masses[k]), vec_slot(w.x64, j), vec_slot(c->full_o, r),
-                  c->full_x.arg()));
-    if (is_device_ptr(x[j])) {
-      CK(launch_merge_full(w.x64.arg(), j, c->full_x.arg(), 0, reinterpret_cast<double2 *>(x[j]), c->g,
-                           c->stream));
-    } else {
-      CK(c->stage_out.ensure(full_bytes));
-      CK(launch_merge_full(w.x64.arg(), j, c->full_x.arg(), 0, reinterpret_cast<double2 *>(c->stage_out.p), c->g,
-                           c->stream));
-      CK(cudaMemcpyAsync(x[j], c->stage_out.p, full_bytes, cudaMemcpyDeviceToHost, c->stream));
-    }
-  }
-  return solve_status(c, iters, true_res);
+  const int st = full_finish(c, nsys, masses, nmass, x, iters, true_res);
+  if (!gave_up(c, st)) return st;
+  CKS(two_kernel_again(c, nsys, masses, nmass, tol, maxiter, prec, &ref));
+  return full_finish(c, nsys, masses, nmass, x, iters, true_res);
 }
 
 // operator calls of the ABI: the FP64 input is rounded to `prec` (per-site
@@ -1914,16 +1950,23 @@ int ms_impl(stag_ctx *c, const double *const src[], int nrhs, const double masse
   std::vector<int> ms_it(nsys2);
   for (int j = 0; j < nsys2; ++j) ms_it[j] = hs[j].iter;
   // phase 2: the shifted systems from their phase-1 solutions
-  CKS(solve_stage(c, src, nrhs, sm.data(), nsh, tol, maxiter, prec));
-  CK(launch_convert_vec(P32, P64, c->ms_x.arg(), w.x64.arg(), nsys2, Ve, c->stream));
-  CK(launch_mark_update(w.st.p ? (SysState *)w.st.p : nullptr, nsys2, c->stream));
-  CKS(enqueue_update(c, c->stream, work_ctl(c, false)));
-  CKS(solve_run(c, maxiter));
-  CK(cudaMemcpyAsync(w.h_st.p, w.st.p, sizeof(SysState) * nsys2, cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaMemcpyAsync(w.h_flags.p, w.flags.p, sizeof(int) * 8, cudaMemcpyDeviceToHost, c->stream));
-  for (int r = 0; r < nrhs; ++r)
-    for (int q = 0; q < nsh; ++q) CKS(vec_out(c, w.x64, r * nsh + q, x[r * nmass + sk[q]]));
-  const int st2 = solve_status(c, it2.data(), tr2.data());
+  auto phase2 = [&]() -> int {
+    CKS(solve_stage(c, src, nrhs, sm.data(), nsh, tol, maxiter, prec));
+    CK(launch_convert_vec(P32, P64, c->ms_x.arg(), w.x64.arg(), nsys2, Ve, c->stream));
+    CK(launch_mark_update(w.st.p ? (SysState *)w.st.p : nullptr, nsys2, c->stream));
+    CKS(enqueue_update(c, c->stream, work_ctl(c, false)));
+    CKS(solve_run(c, maxiter));
+    CK(cudaMemcpyAsync(w.h_st.p, w.st.p, sizeof(SysState) * nsys2, cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaMemcpyAsync(w.h_flags.p, w.flags.p, sizeof(int) * 8, cudaMemcpyDeviceToHost, c->stream));
+    for (int r = 0; r < nrhs; ++r)
+      for (int q = 0; q < nsh; ++q) CKS(vec_out(c, w.x64, r * nsh + q, x[r * nmass + sk[q]]));
+    return solve_status(c, it2.data(), tr2.data());
+  };
+  int st2 = phase2();
+  if (gave_up(c, st2)) {
+    TwoKernel hold(c);
+    st2 = phase2();
+  }
   for (int r = 0; r < nrhs; ++r) {
     if (iters) iters[r * nmass + k0] = it1[r];
     if (true_res) true_res[r * nmass + k0] = tr1[r];
@@ -2133,7 +2176,12 @@ int ragged_impl(const stag_solve_desc *d, int n, double tol, int maxiter, int pr
     }
   int status = STAG_OK;
   for (int i = 0; i < n; ++i) {
-    const int st = solve_finish(d[i].ctx, d[i].x, d[i].iters, d[i].true_res);
+    stag_ctx *c = d[i].ctx;
+    int st = solve_finish(c, d[i].x, d[i].iters, d[i].true_res);
+    if (gave_up(c, st)) {
+      st = two_kernel_again(c, d[i].nrhs * d[i].nmass, d[i].masses, d[i].nmass, tol, maxiter, prec, nullptr);
+      if (st == STAG_OK) st = solve_finish(c, d[i].x, d[i].iters, d[i].true_res);
+    }
     if (st < 0 || (st == STAG_NOT_CONVERGED && status == STAG_OK)) status = st;
   }
   if (status != STAG_OK) {
@@ -2243,7 +2291,7 @@ int stag_create(const int dims[4], int flags, void *cuda_stream, stag_ctx **out)
     }
   }
   const char *giveup = getenv("STAG_TEST_WAIT_GIVEUP");
-  c->wait_giveup = (giveup && giveup[0] == '1') ? 1 : 0;
+  c->wait_giveup = giveup && (giveup[0] == '1' || giveup[0] == '2') ? giveup[0] - '0' : 0;
   cudaError_t e = cudaGetDevice(&c->device);
   if (e != cudaSuccess) {
     cudaGetLastError();

@@ -38,6 +38,7 @@ namespace {
 constexpr int PS_CW = 15;                // compute warps (with a 17th warp a thread has 96 registers, not 128)
 constexpr int PS_BT = 32 * (PS_CW + 1);  // threads of a block
 constexpr unsigned PS_SMEM = 226u * 1024u;  // dynamic shared memory a block may ask for
+constexpr unsigned PS_POLLS = 1u << 21;
 constexpr int BAR_DATA = 1, BAR_SCAL = 2, BAR_DONE = 3;
 
 __device__ __forceinline__ void bar_sync(int id) { asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(PS_BT) : "memory"); }
@@ -46,7 +47,9 @@ __device__ __forceinline__ void bar_arrive(int id) { asm volatile("bar.arrive %0
 __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 // The scalar warp's side of the exchange.  post: this block's sums (w0, w1) into
 // its word, then, everything the block wrote before being visible, one arrival.
-// wait: until `target` arrivals have been counted; false after about two seconds.
+// wait: until `target` arrivals have been counted; false after two seconds and
+// 2^21 polls (over a second of the block's own time: time in which the GPU ran
+// something else does not count).
 // One word is polled, by one lane a block: with every block polling the words of
 // all, the posts queued behind the polls (152 blocks: 4 us from the last post to
 // the first block that saw it).
@@ -62,11 +65,11 @@ __device__ __forceinline__ bool wait_for(const PsArgs &a, int grp, unsigned targ
   const unsigned *p = a.arrived + grp * PS_ASTRIDE;
   if (a.giveup) return false;
   const unsigned long long t0 = global_ns();
-  for (int poll = 0;; ++poll) {
+  for (unsigned poll = 0;; ++poll) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     if ((int)(v - target) >= 0) return true;
-    if ((poll & 63) == 63 && global_ns() - t0 > 2000000000ull) return false;
+    if (poll >= PS_POLLS && (poll & 63) == 63 && global_ns() - t0 > 2000000000ull) return false;
   }
 }
 // all blocks' words (every lane of the warp; after the wait)

@@ -141,3 +141,33 @@ def test_a_stream_with_part_of_the_gpu(L, eager, monkeypatch):
                 ctx.solve_form()
             for m, x in zip(masses, xs):
                 assert oracle.true_residual(L, U, m, b, x) <= 1e-10
+
+
+def test_a_solve_whose_blocks_gave_up_is_run_again(monkeypatch):
+    """Blocks of the persistent kernel that stop waiting for one another: every solve call falls back to the two-kernel
+    form, also one whose solution replaces its source."""
+    monkeypatch.setenv("STAG_TEST_WAIT_GIVEUP", "2")
+    L, masses = (8, 8, 8, 8), [0.2, 0.4]
+    V = synth.volume(L)
+    U = synth.random_links(L, 0.4, 1361)
+    b, f = synth.gaussian_vector(V // 2, 1362), synth.gaussian_vector(V, 1363)
+    with stag.Context(L) as ctx, stag.Context((4, 4, 4, 8)) as small:
+        ctx.links_upload(U)
+        W = synth.random_links((4, 4, 4, 8), 0.4, 1364)
+        small.links_upload(W)
+        bs = synth.gaussian_vector(256, 1365)
+        for _ in range(2):
+            xs = ctx.cg_solve([b], masses)[0]
+            assert ctx.solve_form()["kernels"] != "k_cg_persist"
+            ms = ctx.cg_solve_multishift([b], masses)[0]
+            (rag, ragged), (one,) = [o for o in stag.cg_solve_ragged([(ctx, [b], masses), (small, [bs], [0.2])])[0]]
+            for x in (xs, ms, (rag, ragged)):
+                assert all(oracle.true_residual(L, U, m, b, y) <= 1e-10 for m, y in zip(masses, x))
+            assert oracle.true_residual((4, 4, 4, 8), W, 0.2, bs, one) <= 1e-10
+            full = ctx.solve_full([f], masses)[0]
+            for m, y in zip(masses, full):
+                r = f - 2.0 * m * y - oracle.dslash_full(L, U, y)
+                assert np.linalg.norm(r) <= 1e-10 * np.linalg.norm(f)
+        y = torch.from_numpy(b.copy()).cuda()
+        ctx.cg_solve([y], [0.2], xs=[y])
+        assert oracle.true_residual(L, U, 0.2, b, y.cpu().numpy()) <= 1e-10
