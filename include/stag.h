@@ -52,7 +52,7 @@ extern "C" {
 #define STAG_ERR_STATE (-7)  /* operator used before stag_links_upload */
 
 /* arithmetic/storage precision of the inner (Krylov) iteration */
-#define STAG_FP64 0 /* FP64 storage and arithmetic */
+#define STAG_FP64 0 /* FP64 storage, arithmetic of FP64 accuracy (see stag_links_upload) */
 #define STAG_FP32 1 /* FP32 storage and arithmetic */
 #define STAG_FP16 2 /* FP16 storage (per-site scale for vectors), FP32 arithmetic */
 #define STAG_BF16 3 /* BF16 storage (per-site scale for vectors), FP32 arithmetic */
@@ -101,8 +101,20 @@ int stag_destroy(stag_ctx *ctx);
 /*
  * Copy a gauge field into the context's own device layouts (Sec. 3: the
  * operator's one-link smeared SU(3) field).  `links` is [4][V][3][3][2] FP64,
- * host or device.  The FP64 copy is always kept (true residual, FP64 solves);
- * FP32/FP16/BF16 copies are made on first use.  Staggered phases and the
+ * host or device.  Two copies are kept: the links as they are, and one for the
+ * FP64 operator (true residual, FP64 solves); FP32/FP16/BF16 copies are made on
+ * first use.  The FP64 operator's copy, and with it the arithmetic of the
+ * FP64 operator and of stag_npr_contract, has one of two forms:
+ *   fixed point (58 bits, products on the integer pipe) where U U^dag = 1 to
+ *     1e-3 in every element for every link, and at most an eighth of the links'
+ *     real components are below 2^-6 in magnitude (unit, diagonal or real
+ *     links have more);
+ *   FP64 for any other field.
+ * In fixed point every real component of D v errs by at most 99 x 2^-53 of the
+ * sum of its 48 products' magnitudes (48 FP64 FMAs: 48 x 2^-53; the typical error
+ * is a fifth of theirs): components that the arithmetic does not hold to that,
+ * and those next to infinities, NaNs or values near the ends of the exponent
+ * range, are summed in FP64.  Staggered phases and the
  * boundary sign are applied inside the kernels, never folded into the links.
  * With STAG_RECON12 the links must be SU(3): a unitarity or determinant
  * defect above 1e-12 returns STAG_ERR_NOT_SU3.
@@ -150,9 +162,10 @@ int stag_mdagm(stag_ctx *ctx, int precision, double mass, const double *in_even,
  * Returns STAG_OK when every system converged, STAG_NOT_CONVERGED when some
  * system hit maxiter (its x is the last iterate), STAG_ERR_BREAKDOWN on a
  * non-positive <p, A p> or a non-finite residual, STAG_ERR_TIMEOUT when a
- * kernel's bounded wait gave up (for its staged links, with the shared-memory
- * link path, STAG_TMA=1; for the other blocks of its grid, in the persistent
- * form), STAG_ERR_ARG / _STATE / _CUDA.
+ * kernel's bounded wait for its staged links gave up (only with the
+ * shared-memory link path, STAG_TMA=1; where blocks of the persistent form
+ * give up waiting for one another, the solve is run again in the two-kernel form),
+ * STAG_ERR_ARG / _STATE / _CUDA.
  */
 int stag_cg_solve(stag_ctx *ctx, const double *const src[], int nrhs, const double masses[],
                   int nmass, double tol, int maxiter, int precision, double *const x[],
@@ -178,7 +191,13 @@ int stag_cg_solve(stag_ctx *ctx, const double *const src[], int nrhs, const doub
  *   O_hyp       [V/16][2] (may be NULL): O(z) at hypercube index
  *               z0 + (Lx/2)(z1 + (Ly/2)(z2 + (Lz/2) z3)), host or device;
  *   O_sum       [2] (may be NULL): sum over z, fixed-order FP64 reduction.
- * Uses the uploaded gauge field (FP64).  Errors: STAG_ERR_ARG, _STATE, _CUDA.
+ * Uses the uploaded gauge field, in the form that stag_links_upload chose for it;
+ * in fixed point a hypercube whose own links mix too little (its share of small
+ * components over an eighth), or whose fields are not finite or are far from 1 at a
+ * corner (below 2^-422 or above 2^378), is contracted in FP64, as are single bilinears of corners
+ * 0 or 1 step apart whose terms are small against the largest colours: O(z) errs
+ * by some 1e-14 of the sum of its terms' magnitudes in either form.
+ * Errors: STAG_ERR_ARG, _STATE, _CUDA.
  */
 int stag_npr_contract(stag_ctx *ctx, const int spin_taste[4], const double *chibar1, const double *chi2,
                       const double *chibar3, const double *chi4, double *O_hyp, double *O_sum);
@@ -197,8 +216,12 @@ int stag_npr_contract(stag_ctx *ctx, const int spin_taste[4], const double *chib
  *   alpha      (a1, a2, a3); NULL = (0.75, 0.6, 0.3);
  *   links_in, links_out  [4][V][3][3][2] FP64 as stag_links_upload, host or
  *              device; they may be the same buffer.
- * FP64 throughout on the GPU; the context provides the lattice and the
- * stream (its gauge field is not touched: upload the result to use it).
+ * Fields that stag_links_upload would hold in fixed point are smeared in it
+ * (staples 58-bit, projections FP32 steps corrected from 58-bit residuals; every
+ * element errs by no more than the FP64 form's projection, near 1e-16 for
+ * well-conditioned sums), any other field, and sums too near singular for that, in
+ * FP64.  The context provides the lattice and the stream (its gauge field is not
+ * touched: upload the result to use it).
  * Scratch: 2 x 12 V links of the context's device memory.
  * Errors: STAG_ERR_ARG, STAG_ERR_CUDA, STAG_ERR_OOM.
  */
