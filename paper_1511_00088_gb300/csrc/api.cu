@@ -842,11 +842,18 @@ int stream_sms(const stag_ctx *c) {
 //   7.3, 2 lanes 8.2 / 17.8; 24 576: 9.0, 8.3 / 16.3); 2 while two rounds do (49 152: 2 lanes 11.7,
 //   1 lane 12.6 / 23.3; 98 304: 18.6, 17.1 / 28.0); else 1;
 //   one system: while its links stay in L2 -- reconstruct-12 up to 1.25 of the persisting
-//   set-aside (20^3 x 64, 98 MB: 39.3 / 49.2; 32^3 x 64, 402 MB: 218 / 198), full links up to the
-//   set-aside (20^3 x 32, 74 MB: 25.1 / 31.0; 20^3 x 44, 101 MB: 46.2 / 43.9);
-//   several: by all systems' sites an SM, 2600 with reconstruct-12 (16^3 x 32 x 6: 50.3 / 68.2,
-//   12^3 x 24 x 12: 41.6 / 42.8; 20^3 x 64 x 2: 81.5 / 78.5), 1300 with full links (16^3 x 32 x 3:
-//   30.1 / 34.1; x 6: 58.0 / 51.2).
+//   set-aside (20^3 x 64, 98 MB: 39.3 / 49.2; the persistent form is still ahead at 123 MB, 20^3 x 80:
+//   65.3 / 70.5, and 170 MB, 24^3 x 64: 85.1 / 87.6, and behind at 402 MB, 32^3 x 64: 218 / 198: the line is on
+//   the safe side), full links up to the set-aside (20^3 x 36, 83 MB: 30.4 / 37.8; 20^3 x 40, 92 MB: 41.8 / 42.0;
+//   20^3 x 44, 101 MB: 47.4 / 44.4);
+//   several: by the sites of a block, which is what its time goes with -- 2650 with reconstruct-12
+//   (16^3 x 32 x 6, 2621: 50.3 / 56.9; 12^3 x 24 x 19, 2592: 51.2 / 52.7, x 24, 3456: 65.2 / 63.8; 20^3 x 32 x 3,
+//   2560: 53.4 / 55.7; 8^3 x 16 x 77, 4096: 69.8 / 51.4), 1350 with full links (16^3 x 32 x 3, 1311: 30.1 / 34.4;
+//   12^3 x 24 x 9, 1296: 30.6 / 32.2, x 12, 1728: 39.0 / 38.1; 8^3 x 16 x 39, 1365: 30.3 / 29.7) -- and, above 1200 sites
+//   a block, only where the systems' equal shares use 0.7 of the SMs (8^4 x 77, 0.51: full 43.4 / 34.4,
+//   reconstruct-12 40.5 / 37.3; x 96, 0.63: 41.3 / 39.1; x 112, 0.74: 41.8 / 44.9; 6^3 x 12 x 100, 0.66: 33.7 / 29.9, x 128, 0.84:
+//   34.8 / 35.3); smaller shares win unevenly divided too (8^4 x 51, 1024 sites, 0.67: 25.6 / 25.3 and
+//   24.7 / 30.7; 4^3 x 8 x 77, 0.51: 11.4 / 19.2).
 void choose_persist(stag_ctx *c, int LP, int VP, int nsys, int ms, int *form, int *blocks) {
   *form = *blocks = 0;
   if (!c->coop || c->ps_mode == 0 || LP != P32 || VP != P32 || ms != 0) return;
@@ -858,7 +865,10 @@ void choose_persist(stag_ctx *c, int LP, int VP, int nsys, int ms, int *form, in
   int f = c->ps_mode;
   if (f < 0) {
     const double lb = 8.0 * (rc ? 6 : 9) * 8.0 * Ve, set_aside = c->l2_max_persist ? (double)c->l2_max_persist : 80e6;
-    if (nsys == 1 ? lb > (rc ? 1.25 : 1.0) * set_aside : (double)nsys * Ve > (rc ? 2600.0 : 1300.0) * nsm) return;
+    const double share = (double)Ve / nb;  // sites of a block
+    if (nsys == 1 ? lb > (rc ? 1.25 : 1.0) * set_aside
+                  : share > (rc ? 2650.0 : 1350.0) || (share > 1200.0 && nsys * nb < 0.7 * nsm))
+      return;
     f = Ve <= nb * cg_persist_sites(4) ? 4 : Ve <= 2 * nb * cg_persist_sites(2) ? 2 : 1;
   }
   if (f != 1 && f != 2 && f != 4) return;

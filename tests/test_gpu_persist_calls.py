@@ -171,3 +171,21 @@ def test_a_solve_whose_blocks_gave_up_is_run_again(monkeypatch):
         y = torch.from_numpy(b.copy()).cuda()
         ctx.cg_solve([y], [0.2], xs=[y])
         assert oracle.true_residual(L, U, 0.2, b, y.cpu().numpy()) <= 1e-10
+
+
+@pytest.mark.parametrize("nrhs,nmass,persistent", [(4, 19, True), (7, 11, False)])
+def test_many_systems_with_idle_sms(nrhs, nmass, persistent):
+    """76 systems get two blocks each; 77 would leave half of the SMs idle, and keep the two-kernel form."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("counts for 152 SMs")
+    L = (8, 8, 8, 8)
+    U = synth.random_links(L, 0.4, 1371)
+    bs = [synth.gaussian_vector(synth.volume(L) // 2, 1372 + r) for r in range(nrhs)]
+    masses = [0.3 + 0.05 * k for k in range(nmass)]
+    with stag.Context(L) as ctx:
+        ctx.links_upload(U)
+        xs, _, _, tr = ctx.cg_solve(bs, masses)
+        assert (ctx.solve_form()["kernels"] == "k_cg_persist") == persistent
+    assert max(tr) <= 1e-10
+    for r, k in ((0, 0), (nrhs - 1, nmass - 1)):
+        assert oracle.true_residual(L, U, masses[k], bs[r], xs[r * nmass + k]) <= 1e-10
