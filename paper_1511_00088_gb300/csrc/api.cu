@@ -2692,8 +2692,20 @@ int stag_time_cg_kernel(stag_ctx *c, int precision, int kernel, int nlaunch, dou
   Work &w = c->w;
   const void *lo = nullptr;
   CKS(links_for(c, w.prec, &lo));
-  // the two kernels with the solver's launch configuration (state zeroed:
-  // alpha = beta = 0, every system processed)
+  // the two kernels with the solver's launch configuration.  The states: finished
+  // systems (the folded scalar logic leaves them alone) with alpha = beta = 0, so
+  // that every launch of the timing works on the same finite vectors; before any
+  // solve, vectors of one value (bytes 0x3f: 4.8e-4, 0.75 or 1.8).  What the FP64
+  // operator's integer form takes depends on them: zeros it skips, NaNs it leaves to FP64.
+  {
+    std::vector<SysState> hs(w.nsys);
+    memset(hs.data(), 0, sizeof(SysState) * w.nsys);
+    for (SysState &s : hs) s.done = 1;
+    CK(cudaMemcpyAsync(w.st.p, hs.data(), sizeof(SysState) * w.nsys, cudaMemcpyHostToDevice, c->stream));
+    CK(cudaMemcpyAsync(w.st2.p, hs.data(), sizeof(SysState) * w.nsys, cudaMemcpyHostToDevice, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+  }
+  if (c->last_nsys == 0) CK(cudaMemsetAsync(w.vpool.p, 0x3f, w.vpool.n, c->stream));
   DsArgs a1 = ds_base(c);
   a1.links = lo;
   a1.nsys = w.nsys;
@@ -2720,8 +2732,8 @@ int stag_time_cg_kernel(stag_ctx *c, int precision, int kernel, int nlaunch, dou
   // As in the solve's folded loop, each kernel first finishes its
   // predecessor's reduction in every block (fold_state over the other
   // kernel's partials, states double-buffered); GATE_NONE keeps every system
-  // processed whatever the (zeroed, meaningless) states say, so the timing
-  // holds the fold's reads and arithmetic and the whole kernel body.
+  // processed whatever the states say, so the timing holds the fold's reads and
+  // sums and the whole kernel body.
   const bool folded = c->fold && !w.nrhs_sl;
   SysState *S[2] = {(SysState *)w.st.p, (SysState *)w.st2.p};
   double *PA = (double *)w.partials.p, *PB = (double *)w.partials2.p;

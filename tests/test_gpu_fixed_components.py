@@ -126,3 +126,16 @@ def check_form(L, kind, integer, monkeypatch):
             ctx.links_upload(U)
             got.append(ctx.dslash_oe(v))
     assert np.array_equal(*got) == (not integer)
+
+
+def test_kernel_timing_before_any_solve():
+    """The timing entry point works on finite vectors before any solve, too: the same kernels, the same time (NaNs
+    would take the FP64 branch at every site, eight times as long)."""
+    L = (16, 16, 16, 32)
+    with stag.Context(L) as ctx:
+        ctx.links_upload(synth.random_links_device(L, 0.4, 1221))
+        fresh = ctx.time_dslash(stag.STAG_FP64, nlaunch=20)[0]
+        b = torch.from_numpy(synth.gaussian_vector(synth.volume(L) // 2, 1222)).cuda()
+        ctx.cg_solve([b], [0.1], maxiter=30, precision=stag.STAG_FP64, allow_not_converged=True)
+        after = ctx.time_dslash(stag.STAG_FP64, nlaunch=20)[0]
+    assert 0.6 * after <= fresh <= 1.6 * after
