@@ -148,23 +148,25 @@ def peaks():
         return 6800.0, "fallback"
 
 
-def kernel_source_hash():
-    """Hash of the sources that define the single-system FP32 CG kernels (the
+def kernel_source_hash(key=""):
+    """Hash of the sources that define the FP32 CG kernels of a traffic key (the
     traffic figures of an ncu capture stand only for the code they measured)."""
     h = hashlib.sha256()
-    for f in ("stag_kernels.cuh", "dslash_p32.cu", "dslash_inst.cuh"):
+    for f in (("stag_kernels.cuh", "cg_persist.cu") if key.startswith("cg_persist")
+              else ("stag_kernels.cuh", "dslash_p32.cu", "dslash_inst.cuh")):
         with open(os.path.join(ROOT, "paper_1511_00088_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
 
 
 def ncu_traffic(key):
-    """DRAM bytes per launch of `key` from the committed ncu summary, when it was
-    taken on the current kernel source; else None."""
+    """DRAM bytes per launch of `key` (per iteration, of the persistent CG) from
+    the committed ncu summary, when it was taken on the current kernel source;
+    else None."""
     p = os.path.join(ROOT, "profiles", "ncu_traffic.txt")
     if not os.path.exists(p):
         return None
-    cur = kernel_source_hash()
+    cur = kernel_source_hash(key)
     for line in open(p):
         parts = line.split()
         if len(parts) >= 3 and not line.startswith("#") and parts[0] == key and parts[1] == cur:

@@ -24,11 +24,14 @@
 //   * k_cg_persist_sm (lattices with work for one thread a site): the links of the
 //     next chunk ahead in shared memory.
 // Measured (us per iteration of a whole solve, reliable updates included; two kernels
-// an iteration / this): 8^4 12.4 / 6.9, 12^3 x 24 17.9 / 8.4, 16^3 x 32 22.6 / 13.8 (full
-// links); 20^3 x 64 with reconstruct-12 49.2 / 39.3, near the copy rate for its 258 MB
-// an iteration, a part of which L2 holds.
+// an iteration / this): 8^4 12.4 / 7.1, 12^3 x 24 17.9 / 8.4, 16^3 x 32 22.6 / 13.9 (full
+// links); 20^3 x 64 with reconstruct-12 49.2 / 39.4.  There an iteration's algorithmic
+// bytes are 258 MB; 120 MB of them cross DRAM (0.4 of the copy rate, the rest is
+// served by L2, where 85 MB of the 98 MB of links persist), 390 MB cross L2 at 8.4 TB/s,
+// and a third of the issue slots are used: bound by the gathers' way through L2.
 // Every wait is bounded; a block that gives up sets the error flag and ends, and
-// so do the others, their waits running out.
+// so do the others, their waits running out.  The host then runs the solve again
+// with two kernels an iteration.
 #include "launch.h"
 
 namespace stag {

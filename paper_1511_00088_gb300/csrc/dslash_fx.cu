@@ -1,6 +1,6 @@
 // dslash_fx.cu -- the FP64 half operator from fixed-point links (PFX): the
-// FP64 CG, the reliable updates and the operator calls on near-unitary gauge
-// fields.  The products run on the integer pipe (fixed.cuh).
+// FP64 CG, the reliable updates and the operator calls on gauge fields that pass
+// fx_field.  The products run on the integer pipe (fixed.cuh).
 //
 // A block owns chunks of 32 output sites; warp mu holds direction mu of all of
 // them, one lane a site, and each thread takes the forward and the backward
@@ -15,9 +15,9 @@
 // lane, as they are the scarce ones (a warp's takes 16 clocks of an SM).
 // Measured (M^dag M call on device buffers, 20^3 x 64; its two passes over the
 // links take 96 us at the copy rate): 364 us on FP64 FMAs with packed copies of
-// the vectors, 178 us in this form, 149 us with the caller's layout read and
+// the vectors, 178 us in this form, 156 us with the caller's layout read and
 // written directly (abi_in, abi_center, abi_out); FP64 CG iteration on 16^3 x 32:
-// 115 us before, 50 us.
+// 115 us before, 51 us.
 // The error of such a sum is absolute: up to 11.4 units of 2^-57 of a direction's
 // scale 2^E, the power of two above its largest neighbour component (neighbours truncated
 // 4.9, links rounded 3, l l' dropped 3, rounding 1/2), so up to 50 of the site's with the
@@ -93,7 +93,7 @@ __device__ __noinline__ double2 row_fp64(const Geom &g, const double2 *canon, co
 
 // Blocks an SM: 4 (128 registers) for the plain operator, 3 (168) for the CG
 // kernels and the residual, whose epilogue operands would spill (20^3 x 64: M^dag
-// M call 149 us at 4, 163 at 3; FP64 CG on 16^3 x 32, 713 iterations: 42 and 35.5 ms).
+// M call 151 us at 4, 167 at 3; FP64 CG on 16^3 x 32, 708 iterations: 41.2 and 36.0 ms).
 template <int EPI, int OP>
 __global__ void __launch_bounds__(FXB, (EPI == EPI_PLAIN || EPI == EPI_MDAGM) ? 4 : 3) k_dslash_fx(const DsArgs a) {
   typedef typename Tr<OP>::S2 OS2;
