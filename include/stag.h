@@ -103,13 +103,11 @@ int stag_destroy(stag_ctx *ctx);
  * operator's one-link smeared SU(3) field).  `links` is [4][V][3][3][2] FP64,
  * host or device.  Two copies are kept: the links as they are, and one for the
  * FP64 operator (true residual, FP64 solves); FP32/FP16/BF16 copies are made on
- * first use.  The FP64 operator's copy, and with it the arithmetic of the
- * FP64 operator and of stag_npr_contract, has one of two forms:
- *   fixed point (58 bits, products on the integer pipe) where U U^dag = 1 to
- *     1e-3 in every element for every link, and at most an eighth of the links'
- *     real components are below 2^-6 in magnitude (unit, diagonal or real
- *     links have more);
- *   FP64 for any other field.
+ * first use.  The FP64 operator's copy, and with it that operator's arithmetic,
+ * is fixed point (58 bits, products on the integer pipe) where U U^dag = 1 to 1e-3
+ * in every element for every link, FP64 for any other field.  Where moreover
+ * at most an eighth of the links' real components are below 2^-6 in magnitude
+ * (unit, diagonal or real links have more), stag_npr_contract takes fixed point.
  * In fixed point every real component of D v errs by at most 99 x 2^-53 of the
  * sum of its 48 products' magnitudes (48 FP64 FMAs: 48 x 2^-53; the typical error
  * is a fifth of theirs): components that the arithmetic does not hold to that,
@@ -191,7 +189,7 @@ int stag_cg_solve(stag_ctx *ctx, const double *const src[], int nrhs, const doub
  *   O_hyp       [V/16][2] (may be NULL): O(z) at hypercube index
  *               z0 + (Lx/2)(z1 + (Ly/2)(z2 + (Lz/2) z3)), host or device;
  *   O_sum       [2] (may be NULL): sum over z, fixed-order FP64 reduction.
- * Uses the uploaded gauge field, in the form that stag_links_upload chose for it;
+ * Uses the uploaded gauge field, in fixed point or FP64 (stag_links_upload);
  * in fixed point a hypercube whose own links mix too little (its share of small
  * components over an eighth), or whose fields are not finite or are far from 1 at a
  * corner (below 2^-422 or above 2^378), is contracted in FP64, as are single bilinears of corners
@@ -216,7 +214,7 @@ int stag_npr_contract(stag_ctx *ctx, const int spin_taste[4], const double *chib
  *   alpha      (a1, a2, a3); NULL = (0.75, 0.6, 0.3);
  *   links_in, links_out  [4][V][3][3][2] FP64 as stag_links_upload, host or
  *              device; they may be the same buffer.
- * Fields that stag_links_upload would hold in fixed point are smeared in it
+ * Fields that stag_npr_contract would take in fixed point are smeared in it
  * (staples 58-bit, projections FP32 steps corrected from 58-bit residuals; every
  * element errs by no more than the FP64 form's projection, near 1e-16 for
  * well-conditioned sums), any other field, and sums too near singular for that, in

@@ -228,8 +228,9 @@ struct stag_ctx {
   int l2_modes = 0b11;    // 0b11: by rule; else bit p: the tuner may choose L2 mode p (STAG_L2PERSIST fixes it)
   size_t l2_max_persist = 0, l2_max_window = 0;
   DevBuf links_canon;  // [4][V][3][3] FP64, kept for lazy reduced-precision copies
-  DevBuf links64;      // the FP64 operator's copy: fixed-point (fixed.cuh) of a field that passes fx_field, else FP64
+  DevBuf links64;      // the FP64 operator's copy: fixed-point (fixed.cuh) of a near-unitary field, else FP64
   bool fx_ok = false;  // links64 is fixed-point
+  bool fx_mix = false; // the field passes fx_field: so does the NPR contraction
   bool fx_mode = true; // STAG_FX=0: never (the FP64 pipe's operator, for A/B runs)
   DevBuf links_lo[4][2];
   bool lo_ok[4][2] = {{false, false}, {false, false}, {false, false}, {false, false}};
@@ -333,7 +334,7 @@ int vec_out(stag_ctx *c, const VecBuf &v, int k, double *dst) {
 }
 
 // FP64 operator form of the uploaded field: PFX (integer-pipe products of the
-// fixed-point links) on near-unitary fields that mix (fx_field), P64 on any other
+// fixed-point links) on near-unitary fields, P64 on any other
 int lp_for(const stag_ctx *c, int P) { return (P == P64 && c->fx_ok) ? PFX : P; }
 // launch_dslash with the FP64 form of this field
 cudaError_t launch_ds(const stag_ctx *c, int LP, int recon, int VP, int OP, int NS, int EPI, int lanes, int nblocks,
@@ -2373,31 +2374,30 @@ int stag_links_upload(stag_ctx *c, const double *links) {
       return STAG_ERR_NOT_SU3;
     }
   }
-  // The FP64 operator's copy: fixed-point, unless the field does not pass fx_field.
+  // The FP64 operator's copy: fixed-point where every link is near unitary.
   // No lattice is too small for it (2^4, 8 sites a parity: M^dag M call 27 us, 42 with
   // the FP64 form and its copies between layouts; NPR contraction 50 and 60; FP64
   // CG 0.5 and 0.8 ms).  Both forms take 16 bytes an element, so one buffer serves.
   static_assert(sizeof(int4) == sizeof(double2), "one buffer for either form");
   CK(c->links64.ensure(cplx_bytes(P64) * 9ull * 8ull * c->Ve));
-  c->have_links = c->fx_ok = false;
+  c->have_links = c->fx_ok = c->fx_mix = false;
   const double2 *canon = reinterpret_cast<const double2 *>(c->links_canon.p);
-  bool fx = false;
+  FieldCheck check = {0, 1};
   if (c->fx_mode) {
-    FieldCheck check;
     CK(c->defect.ensure(sizeof(FieldCheck)));
     CK(cudaMemsetAsync(c->defect.p, 0, sizeof(FieldCheck), c->stream));
     CK(launch_pack_links_fx(canon, (int4 *)c->links64.p, c->g, (FieldCheck *)c->defect.p, c->stream));
     CK(cudaMemcpyAsync(&check, c->defect.p, sizeof check, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
-    fx = fx_field(check, 4 * c->V);
   }
-  if (!fx) {
+  if (check.bad) {
     CK(launch_pack_links(P64, 0, canon, c->links64.p, c->g, c->stream));
     CK(cudaStreamSynchronize(c->stream));
   }
   for (int p = 0; p < 4; ++p) c->lo_ok[p][0] = c->lo_ok[p][1] = c->tile_ok[p][0] = c->tile_ok[p][1] = false;
   c->have_links = true;
-  c->fx_ok = fx;
+  c->fx_ok = !check.bad;
+  c->fx_mix = fx_field(check, 4 * c->V);
   c->w.drop_graph();  // the graph holds link pointers of the reduced-precision copies
   return STAG_OK;
 }
@@ -2474,7 +2474,7 @@ int stag_npr_contract(stag_ctx *c, const int spin_taste[4], const double *chibar
   double2 *out = (O_hyp && is_device_ptr(O_hyp)) ? reinterpret_cast<double2 *>(O_hyp) : (double2 *)c->npr_o.p;
   double2 *sum = (double2 *)c->npr_o.p + nh;
   CK(launch_npr(c->dims, reinterpret_cast<const double2 *>(c->links_canon.p), spin_taste, d[0], d[1], d[2], d[3],
-                out, O_sum ? sum : nullptr, c->fx_ok, c->stream));
+                out, O_sum ? sum : nullptr, c->fx_mix, c->stream));
   if (O_hyp && out == (double2 *)c->npr_o.p)
     CK(cudaMemcpyAsync(O_hyp, out, sizeof(double2) * (size_t)nh, cudaMemcpyDeviceToHost, c->stream));
   if (O_sum) CK(cudaMemcpyAsync(O_sum, sum, sizeof(double2), cudaMemcpyDefault, c->stream));

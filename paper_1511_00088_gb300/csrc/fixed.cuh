@@ -14,9 +14,9 @@
 // a tenth of an FP64 FMA chain's, and becomes FP64 with one rounding.  That error
 // is absolute: where a sum's own products are all far below the largest factor
 // (components of very different sizes that the links do not mix), it would lose
-// bits that FP64 keeps.  So every user tests its sums or products and leaves
-// such ones to FP64, and fields whose links mix too little (FX_SMALL below) run
-// on FP64 altogether.
+// bits that FP64 keeps.  So the operator and the NPR contraction test their sums
+// and leave such ones to FP64, and HYP and NPR run on FP64 altogether on fields
+// whose links mix too little (FX_SMALL below).
 // Range, for a row of u of 2-norm^2 <= 2 (near_unitary: within 1e-3 of 1) on 6 components
 // |v| <= 1, eight hops: by Cauchy-Schwarz |hh| <= 8 sqrt(12) 2^57 < 2^61.8 and
 // |cr| <= 8 (sqrt(12) 2^57 + 6 2^56) < 2^62.7.
@@ -114,10 +114,11 @@ FX_HD bool near_unitary(const float2 (&u)[9]) {
 }
 
 // A field's links mix the colours, and real with imaginary parts, if few of
-// their real components are small.  With over an eighth below 2^-6 (unit,
-// diagonal, real or nearly such links) the sums of the operator would be left
-// to FP64 one by one too often, and the FP64 forms run from the start.  Links
+// their real components are small.  HYP smearing and the NPR contraction, whose
+// products of links keep small elements only to 2^-58, run on FP64 where over an
+// eighth are below 2^-6 (unit, diagonal, real or nearly such links).  Links
 // exp(i c H): 3 % below at c = 0.4 and for Haar matrices, 11 % at c = 0.1.
+// (The operator tests each of its sums, and takes every near-unitary field.)
 constexpr float FX_SMALL = 0x1p-6f;
 FX_HD int small_parts(const float2 (&u)[9]) {
   int n = 0;

@@ -163,7 +163,7 @@ cudaError_t launch_su3_defect(const double2 *U, long long nlinks, unsigned long 
 // NPR one-colour-trace four-fermion contraction (npr.cu): out[h] = O(z_h) for
 // every hypercube (V / 16 entries), *sum (may be null) = their sum; U the
 // canonical [4][V][3][3] links, fields [V][3]; st = (S1, F1, S2, F2), 4-bit
-// corner masks; fx: the integer form runs (stag_ctx::fx_ok)
+// corner masks; fx: the integer form runs (stag_ctx::fx_mix)
 cudaError_t launch_npr(const int dims[4], const double2 *U, const int st[4], const double2 *cb1, const double2 *c2,
                        const double2 *cb3, const double2 *c4, double2 *out, double2 *sum, bool fx, cudaStream_t s);
 

@@ -1598,7 +1598,7 @@ __global__ void k_pack_links(const double2 *__restrict__ src, void *dst, Geom g)
   }
 }
 
-// the fixed-point copy of a gauge field, and what decides whether it is used (fx_field)
+// the fixed-point copy of a gauge field, and what decides whether it is used (FieldCheck)
 __global__ void k_pack_links_fx(const double2 *__restrict__ src, int4 *__restrict__ dst, Geom g, FieldCheck *check);
 
 // tiled site-owned copy of the links (see the layout notes at the top): one

@@ -63,6 +63,8 @@ def links(kind, L, seed):
         ph = np.exp(2j * np.pi * rng.uniform(size=(4, V, 3)))
         return ph[..., None] * np.eye(3)
     U = synth.random_links(L, {"rough": 0.4, "smooth": 0.1}.get(kind, 0.4), seed)
+    if kind == "scaled":
+        U *= 1.01
     if kind == "some_cold":  # one link in thirty nearly diagonal, off-diagonal elements of 1e-7
         cold = rng.random((4, V)) < 1 / 30
         n = int(cold.sum())
@@ -103,8 +105,8 @@ def test_every_component_as_in_fp64(kind, spread):
     check(L, U, b, eo, oracle.dslash_eo(L, U, b), 0)
 
 
-@pytest.mark.parametrize("kind,integer", [("rough", True), ("smooth", True), ("some_cold", True), ("unit", False),
-                                          ("phases", False)])
+@pytest.mark.parametrize("kind,integer", [("rough", True), ("smooth", True), ("some_cold", True), ("unit", True),
+                                          ("phases", True), ("scaled", False)])
 def test_the_form_that_runs(kind, integer, monkeypatch):
     """Other bits than the FP64 form's where the integer form runs, the same where it does not."""
     check_form((6, 4, 4, 8), kind, integer, monkeypatch)
